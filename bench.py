@@ -315,6 +315,7 @@ def gpu_arm(args, ws, rank, local):
                      "achieved": None if achieved is None else achieved / 1e12,
                      "peak": peak64 / 1e12, "unit": "TFLOP/s",
                      "peak_source": "FP64 FMA probe (nb_probe_fma_peak) in this run: best of 5 runs before and 5 after the timed region",
+                     "note": "79 flops per pair over the DFMA peak; the FP64 pair terms run mostly on the integer pipes, so the fraction may exceed 1",
                      "frac": None if achieved is None else achieved / peak64,
                      "traffic": eval_traffic(),
                      "traffic_unit": "DRAM bytes per launch (ncu, mean of 5 launches), null if the kernel changed",

@@ -52,10 +52,9 @@ nb_status nb_selftest_wait_timeout(double budget_seconds, void *stream);
  * nb_probe_rsqrt -- the evaluation kernel's reciprocal square roots applied
  * elementwise, for accuracy tests against a higher-precision reference:
  *   y[k] = 1 / sqrt(x[k])
- *   which : 0 = the FP64 form the FP64 pair terms use (x scaled into
- *               [1, 4), SFU seed refined in float-float on the FP32 pipe,
- *               assembled as a double on the integer pipe, one FP64 Newton
- *               step: three DFMAs);
+ *   which : 0 = the form the FP64 pair terms use (block fixed point: SFU seed,
+ *               one third-order step on integers; here with r = 0 and
+ *               eps^2 = x, the result rounded to a double);
  *           1 = the float-float form of the EX pair terms, on x rounded to a
  *               float-float pair, result returned as hi + lo in FP64;
  *           2 = the earlier five-DFMA FP64 form (integer-built FP32 seed,

@@ -436,7 +436,7 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
 
     int64_t *d_offs = nullptr, *d_jofs = nullptr, *d_cb = nullptr, *d_ce = nullptr;
     int32_t *d_ccl = nullptr, *d_cc0 = nullptr;
-    size_t jbytes = p->precision == NB_FP64 ? sizeof(J64)
+    size_t jbytes = p->precision == NB_FP64 ? sizeof(JFX)
                     : (p->precision == NB_FP32 ? sizeof(J32) : sizeof(JEX));  // EX, FP32X
 #define ALLOC(ptr, cnt)                                                                      \
     do {                                                                                     \
@@ -457,11 +457,7 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
     unsigned char *jraw = nullptr;
     ALLOC(jraw, nj * jbytes);
     d.jarr = jraw;
-    if (p->precision == NB_FP64) {
-        d.jarr64 = reinterpret_cast<J64 *>(jraw);
-    } else {
-        ALLOC(d.jarr64, nj);
-    }
+    ALLOC(d.jarr64, nj);
     ALLOC(d.chunk_min, n_chunks);
     ALLOC(d.chunk_cnt, n_chunks);
     ALLOC(d.tnext, n_clusters);

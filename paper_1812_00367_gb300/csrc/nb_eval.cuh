@@ -11,12 +11,12 @@
 // i.e. NM08's A1 = m v/s^3 - 3 alpha A0 and A2 = m a/s^3 - 6 alpha A1 - 3 beta A0
 // with the large alpha terms cancelling inside each pair before it is summed
 // (that keeps the FP32 path within its bound on strongly cancelling sums).
-// Every per-pair operation is a multiply, an add or a fused multiply-add:
-// 50 FP64 instructions per pair on the FP64 path (the reciprocal square
-// root's seed is refined on the FP32 and integer pipes, NB_FP64_RSQRT3; one
-// exact doubling is done on the integer pipe; the potential m y is summed in
-// float-float on the FP32 pipe, NB_FP64_POT_FF).  The 4th-order scheme (Makino & Aarseth 1992) keeps
-// A0, A1 and the potential only (interact4: 29 FP64 instructions per pair).
+// FP64: the pair terms run in block fixed point on the integer pipes
+// (nb_fixed.cuh); 12 FP64 instructions per pair remain, the coordinate
+// differences and the nine running sums (9 in the 4th-order form); the
+// potential m y is summed in float-float on the FP32 pipe.  The 4th-order
+// scheme (Makino & Aarseth 1992) keeps A0, A1 and the potential only
+// (interact4).
 //
 // Work decomposition: a piece of work is (cluster, i-tile, j-range).  An
 // i-tile holds kTPB / gl active particles; gl lanes of a warp share one i and
@@ -34,6 +34,7 @@
 // only its own state in registers.
 #pragma once
 
+#include "nb_fixed.cuh"
 #include "nb_internal.cuh"
 #include "nb_step.cuh"
 
@@ -43,135 +44,183 @@ template <int P>
 struct Prec;
 
 // ===================================================================== FP64
+// Block fixed-point pair terms (nb_fixed.cuh): the coordinate differences and
+// the nine running sums stay on the FP64 pipe (12 instructions per pair, 9 in
+// the 4th-order form), everything between them runs on the integer pipes.
+// Bound: the issue of half-rate integer instructions (shifts, logic,
+// IMAD.WIDE; about 680 instructions a pair and warp, 61 % of the ALU pipe and
+// 59 % of the FP64 pipe busy).  Measured, N = 65536 all active: 139.7 ms
+// (3.07e10 pairs/s) against 361.2 ms for the same terms in doubles (50 DFMA a
+// pair, the FP64 pipe 95 % busy); 4th order, N = 30011: 18.4 against 44.8 ms;
+// A = 48: 151 against 324 us.  Residency: 3, 4, 5 or 6 CTAs per SM measured
+// within 1 % of one another.
 template <>
 struct Prec<NB_FP64> {
-    using J = J64;
+    using J = JFX;
     static constexpr int kPerRec = 1;  // particles per record
     struct I {
-        double x[3], v[3], a[3];
-        double m1, nz;  // -1.0, -0.0 from kernel parameters (see Dev)
+        double x[3];
+        int64_t v[3], a[3];
+        int32_t ev, ea;
+        double m1;       // -1.0 from the kernel parameters (see Dev)
+        uint64_t eps_x;  // eps^2 as a fixed-point number and its block exponent
+        uint32_t emin;
+        FxK K;
     };
     struct Acc {
         double a[3], j[3], s[3], p;
-#if NB_FP64_POT_FF
-        ff pf;  // the current j-tile's potential as a float pair
-#endif
+        ff pf;         // the current j-tile's potential as a float pair
+        int32_t fv, fa;  // largest stored exponent of v, a seen (kFxBad: a non-finite one)
     };
     static __device__ __forceinline__ void prepare(I &i, const Dev &d) {
         i.m1 = d.neg_one;
-        i.nz = d.neg_zero;
-    }
-    // product and difference; as FMAs with run-time -0.0 / -1.0 when
-    // NB_FP64_ALL_FMA (same IEEE results: a*b + (-0) == a*b, b*(-1) + a == a - b)
-    static __device__ __forceinline__ double fma_rt(double a, double b, double c) {
-        double r;
-        asm("fma.rn.f64 %0, %1, %2, %3;" : "=d"(r) : "d"(a), "d"(b), "d"(c));
-        return r;
-    }
-    static __device__ __forceinline__ double mul(const I &i, double a, double b) {
-        if constexpr (NB_FP64_ALL_FMA) return fma_rt(a, b, i.nz);
-        else return a * b;
-    }
-    static __device__ __forceinline__ double sub(const I &i, double a, double b) {
-        if constexpr (NB_FP64_ALL_FMA) return fma_rt(b, i.m1, a);
-        else return a - b;
+        i.eps_x = d.eps_x;
+        i.emin = d.eps_emin;
+        i.K = d.fxk;
     }
     static __device__ __forceinline__ I load_i(const J *jarr, int64_t k) {
         const J e = jarr[k];
         I r;
-        r.x[0] = e.q[0].x; r.x[1] = e.q[0].y; r.x[2] = e.q[1].x;
-        r.v[0] = e.q[2].x; r.v[1] = e.q[2].y; r.v[2] = e.q[3].x;
-        r.a[0] = e.q[3].y; r.a[1] = e.q[4].x; r.a[2] = e.q[4].y;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            r.x[q] = e.x[q];
+            r.v[q] = e.v[q];
+            r.a[q] = e.a[q];
+        }
+        r.ev = jfx_ev(e);
+        r.ea = jfx_ea(e);
         return r;
     }
     static __device__ __forceinline__ void zero(Acc &c) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) c.a[k] = c.j[k] = c.s[k] = 0.0;
         c.p = 0.0;
-#if NB_FP64_POT_FF
         c.pf = ff{0.f, 0.f};
-#endif
+        c.fv = c.fa = kFxMinExp;
     }
-    // potential term m y: FP64 DFMA, or float-float on the FP32 pipe
-    static __device__ __forceinline__ void pot_term(const J &jj, bool self, double m, double y,
-                                                    Acc &c) {
-#if NB_FP64_POT_FF
-        (void)m;
-        const float2 mf = jj.mf;
-        const ff yf = ff_from_pos_double(y);
-        const ff mff = ff{self ? 0.f : mf.x, self ? 0.f : mf.y};
-        // renormalised every term (|lo| stays below half an ulp of hi): a
-        // 64-term tile sum is good to ~2^-45, and tiles add up in FP64
-        c.pf = ff_add(c.pf, ff_mul_lazy(mff, yf));
-#else
-        (void)jj;
-        (void)self;
-        c.p = fma(m, y, c.p);
-#endif
+    // potential term m y in float-float, renormalised every term (|lo| stays
+    // below half an ulp of hi): a 64-term tile sum is good to ~2^-45, and
+    // tiles add up in FP64
+    static __device__ __forceinline__ void pot_term(const J &jj, bool self, const FxRoot &t, Acc &c) {
+        // y = Y 2^(-62 - g) as 24 + 24 bits
+        const float s1 = __int_as_float((127 - 23 - t.g) << 23);
+        const float yh = __fmul_rn((float)(uint32_t)(t.y >> 39), s1);
+        const float yl = __fmul_rn((float)((uint32_t)(t.y >> 15) & 0xffffffu), __fmul_rn(s1, 5.9604644775390625e-08f));
+        const ff mff = ff{self ? 0.f : jj.mf.x, self ? 0.f : jj.mf.y};
+        c.pf = ff_add(c.pf, ff_mul_lazy(mff, ff{yh, yl}));
     }
-#if NB_FP64_POT_FF
     // End of a j-tile: the tile's float-pair potential joins the FP64 total.
     static __device__ __forceinline__ void tile_done(Acc &c) {
         c.p += (double)c.pf.hi + (double)c.pf.lo;
         c.pf = ff{0.f, 0.f};
     }
-#else
-    static __device__ __forceinline__ void tile_done(Acc &) {}
-#endif
-    static __device__ __forceinline__ void interact(const I &i, const J &jj, bool self,
-                                                    double eps2, float, Acc &c) {
-        const double2 q0 = jj.q[0], q1 = jj.q[1], q2 = jj.q[2], q3 = jj.q[3], q4 = jj.q[4];
-        const double rx = sub(i, q0.x, i.x[0]), ry = sub(i, q0.y, i.x[1]), rz = sub(i, q1.x, i.x[2]);
-        const double vx = sub(i, q2.x, i.v[0]), vy = sub(i, q2.y, i.v[1]), vz = sub(i, q3.x, i.v[2]);
-        const double ax = sub(i, q3.y, i.a[0]), ay = sub(i, q4.x, i.a[1]), az = sub(i, q4.y, i.a[2]);
-        double r2 = fma(rx, rx, fma(ry, ry, fma(rz, rz, eps2)));
-        double m = q1.y;
-        r2 = self ? 1.0 : r2;  // selects, not FP64 arithmetic
-        m = self ? 0.0 : m;
-        const double y = NB_FP64_RSQRT3 ? rsqrt_f64_3(r2, i.nz)
-                         : (NB_FP64_ALL_FMA ? rsqrt_f64_fma(r2, i.nz) : rsqrt_f64(r2));
-        const double y2 = mul(i, y, y);
-        pot_term(jj, self, m, y, c);               // potential: sum m y
-        const double q = mul(i, mul(i, m, y2), y); // m y^3
-        const double rv = fma(rx, vx, fma(ry, vy, mul(i, rz, vz)));
-        const double w = fma(vx, vx, fma(vy, vy, fma(vz, vz, fma(rx, ax, fma(ry, ay, mul(i, rz, az))))));
-        const double al = mul(i, rv, y2);
-        const double ze = mul(i, w, y2);
-        const double al3 = mul(i, 3.0, al);
-        const double be3 = mul(i, 3.0, fma(al, al, ze));  // 3 beta
-        const double al6 = twice_int(al3);          // exact doubling, integer pipe
-        const double w1x = fma(-al3, rx, vx), w1y = fma(-al3, ry, vy), w1z = fma(-al3, rz, vz);
-        const double w2x = fma(-be3, rx, fma(-al6, w1x, ax));
-        const double w2y = fma(-be3, ry, fma(-al6, w1y, ay));
-        const double w2z = fma(-be3, rz, fma(-al6, w1z, az));
-        c.a[0] = fma(q, rx, c.a[0]); c.a[1] = fma(q, ry, c.a[1]); c.a[2] = fma(q, rz, c.a[2]);
-        c.j[0] = fma(q, w1x, c.j[0]); c.j[1] = fma(q, w1y, c.j[1]); c.j[2] = fma(q, w1z, c.j[2]);
-        c.s[0] = fma(q, w2x, c.s[0]); c.s[1] = fma(q, w2y, c.s[1]); c.s[2] = fma(q, w2z, c.s[2]);
+    template <bool kOrder6>
+    static __device__ __forceinline__ void pair(const I &i, const J &jj, bool self, Acc &c) {
+        double r[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) r[k] = fma_rn_f64(i.x[k], i.m1, jj.x[k]);
+        const int evj = jfx_ev(jj);
+        const Fx3 R = fx_decode(r, i.emin);
+        const Fx3 V = fx_diff_norm(jj.v, evj, i.v, i.ev);
+        FxS Rs[3], Vs[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            Rs[k] = fx_split(R.w[k]);
+            Vs[k] = fx_split(V.w[k]);
+        }
+        const FxRoot t = fx_root(Rs, R.e, i.eps_x, i.emin, i.K);
+        pot_term(jj, self, t, c);
+        const double q = fx_q(t, jj.mm, jfx_em(jj), jfx_sign(jj), self, i.K);
+        c.fv = max(c.fv, evj);
+        Fx3 A;
+        if constexpr (kOrder6) {
+            const int eaj = jfx_ea(jj);
+            c.fa = max(c.fa, eaj);
+            A = fx_diff_norm(jj.a, eaj, i.a, i.ea);
+        }
+        double w1[3], w2[3];
+        if (fx_inside(r, i.emin)) {
+            // r below the softening's scale (and the pair i == j): its block
+            // would carry too few bits, so alpha, beta, w1 and w2 are formed
+            // in doubles.  Rare: a few pairs of each particle.
+            double v[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) v[k] = fx_to_double(V.w[k], V.e - 61 + 1023);
+            const double y2 = fx_to_double((int64_t)t.y2, -60 - 2 * t.g + 1023);
+            const double rv = fma(r[0], v[0], fma(r[1], v[1], r[2] * v[2]));
+            const double al = rv * y2;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) w1[k] = fma(-3.0 * al, r[k], v[k]);
+            if constexpr (kOrder6) {
+                double a[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) a[k] = fx_to_double(A.w[k], A.e - 61 + 1023);
+                const double w = fma(v[0], v[0], fma(v[1], v[1], fma(v[2], v[2],
+                                 fma(r[0], a[0], fma(r[1], a[1], r[2] * a[2])))));
+                const double be3 = 3.0 * fma(al, al, w * y2);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) w2[k] = fma(-be3, r[k], fma(-6.0 * al, w1[k], a[k]));
+            }
+        } else {
+            const FxS Y2 = fx_split((int64_t)t.y2);
+            const FxW1 u = fx_w1(Rs, Vs, V.w, t, Y2, i.K);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) w1[k] = fx_to_double(u.w[k], V.e - 59 + 1023);
+            if constexpr (kOrder6) {
+                int64_t x2[3];
+                int ez;
+                fx_w2(Rs, R.e, Vs, V.e, A, t, Y2, u, x2, ez, i.K);
+                const int base = min(ez - R.e, 900) - 52 + 1023;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) w2[k] = fx_to_double(x2[k], base);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            c.a[k] = fma(q, r[k], c.a[k]);
+            c.j[k] = fma(q, w1[k], c.j[k]);
+            if constexpr (kOrder6) c.s[k] = fma(q, w2[k], c.s[k]);
+        }
     }
-    // 4th-order pair term (Makino & Aarseth 1992): A0 = q r, A1 = q (v - 3 alpha r);
-    // 29 FP64 instructions (31 with the 5-operation root, one more without
-    // NB_FP64_POT_FF)
-    static __device__ __forceinline__ void interact4(const I &i, const J &jj, bool self,
-                                                     double eps2, float, Acc &c) {
-        const double2 q0 = jj.q[0], q1 = jj.q[1], q2 = jj.q[2], q3 = jj.q[3];
-        const double rx = sub(i, q0.x, i.x[0]), ry = sub(i, q0.y, i.x[1]), rz = sub(i, q1.x, i.x[2]);
-        const double vx = sub(i, q2.x, i.v[0]), vy = sub(i, q2.y, i.v[1]), vz = sub(i, q3.x, i.v[2]);
-        double r2 = fma(rx, rx, fma(ry, ry, fma(rz, rz, eps2)));
-        double m = q1.y;
-        r2 = self ? 1.0 : r2;
-        m = self ? 0.0 : m;
-        const double y = NB_FP64_RSQRT3 ? rsqrt_f64_3(r2, i.nz)
-                         : (NB_FP64_ALL_FMA ? rsqrt_f64_fma(r2, i.nz) : rsqrt_f64(r2));
-        const double y2 = mul(i, y, y);
-        pot_term(jj, self, m, y, c);
-        const double q = mul(i, mul(i, m, y2), y);
-        const double rv = fma(rx, vx, fma(ry, vy, mul(i, rz, vz)));
-        const double al3 = mul(i, 3.0, mul(i, rv, y2));
-        const double w1x = fma(-al3, rx, vx), w1y = fma(-al3, ry, vy), w1z = fma(-al3, rz, vz);
-        c.a[0] = fma(q, rx, c.a[0]); c.a[1] = fma(q, ry, c.a[1]); c.a[2] = fma(q, rz, c.a[2]);
-        c.j[0] = fma(q, w1x, c.j[0]); c.j[1] = fma(q, w1y, c.j[1]); c.j[2] = fma(q, w1z, c.j[2]);
+    static __device__ __forceinline__ void interact(const I &i, const J &jj, bool self, Acc &c) {
+        pair<true>(i, jj, self, c);
     }
-    // pot-only pair term (energy diagnostics)
+    // 4th-order pair term (Makino & Aarseth 1992): A0 = q r, A1 = q (v - 3 alpha r)
+    static __device__ __forceinline__ void interact4(const I &i, const J &jj, bool self, Acc &c) {
+        pair<false>(i, jj, self, c);
+    }
+    static __device__ __forceinline__ void finish(const I &i, const Acc &c, double o[10]) {
+        // a velocity that is not finite takes jerk and snap with it, an
+        // acceleration the snap (as v - 3 alpha r and the rest would)
+        const double nan = __hiloint2double(0x7ff80000, 0);
+        const bool bad_v = max(c.fv, i.ev) >= kFxBad, bad_a = bad_v || max(c.fa, i.ea) >= kFxBad;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            o[k] = c.a[k];
+            o[3 + k] = bad_v ? nan : c.j[k];
+            o[6 + k] = bad_a ? nan : c.s[k];
+        }
+        o[9] = -(c.p + ((double)c.pf.hi + (double)c.pf.lo));
+    }
+};
+
+// ========================================================= FP64 potential
+// The potential alone (energy diagnostics), from the FP64 records.
+template <>
+struct Prec<kPrecPot> {
+    using J = J64;
+    static constexpr int kPerRec = 1;
+    struct I {
+        double x[3];
+    };
+    struct Acc {
+        double p;
+    };
+    static __device__ __forceinline__ I load_i(const J *jarr, int64_t k) {
+        const J e = jarr[k];
+        return I{{e.q[0].x, e.q[0].y, e.q[1].x}};
+    }
+    static __device__ __forceinline__ void zero(Acc &c) { c.p = 0.0; }
     static __device__ __forceinline__ void interact_pot(const I &i, const J &jj, bool self,
                                                         double eps2, Acc &c) {
         const double2 q0 = jj.q[0], q1 = jj.q[1];
@@ -182,18 +231,10 @@ struct Prec<NB_FP64> {
         m = self ? 0.0 : m;
         c.p = fma(m, rsqrt_f64(r2), c.p);
     }
-    static __device__ __forceinline__ void finish(const Acc &c, const double *, int, double o[10]) {
+    static __device__ __forceinline__ void finish(const Acc &c, double o[10]) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            o[k] = c.a[k];
-            o[3 + k] = c.j[k];
-            o[6 + k] = c.s[k];
-        }
-#if NB_FP64_POT_FF
-        o[9] = -(c.p + ((double)c.pf.hi + (double)c.pf.lo));
-#else
+        for (int k = 0; k < 9; ++k) o[k] = 0.0;
         o[9] = -c.p;
-#endif
     }
 };
 
@@ -850,7 +891,6 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
 #pragma unroll
         for (int q = 0; q < 10; ++q) t64[q * t64st] = 0.0;
         const double eps2 = d.eps2;
-        const float eps2f = (float)eps2;
         const float2 eps2f2 = d.eps2_hi2;
         const ff2 eps2ff2{d.eps2_hi2, d.eps2_lo2};
 
@@ -907,20 +947,20 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
                         T::interact(me, tl[k], jbase + 2 * k == ji, jbase + 2 * k + 1 == ji,
                                     eps2ff2, acc);
                 } else if constexpr (uses_order4_terms(MODE)) {
-#pragma unroll kEvalUnroll
+#pragma unroll 1
                     for (int k = jsub; k < kTJ; k += gl)
-                        T::interact4(me, tl[k], jbase + k == ji, eps2, eps2f, acc);
+                        T::interact4(me, tl[k], jbase + k == ji, acc);
                 } else {
-#pragma unroll kEvalUnroll
+#pragma unroll 1
                     for (int k = jsub; k < kTJ; k += gl)
-                        T::interact(me, tl[k], jbase + k == ji, eps2, eps2f, acc);
+                        T::interact(me, tl[k], jbase + k == ji, acc);
                 }
                 if constexpr (P == NB_FP32 || P == NB_FP32X) {
                     if ((tt - tb + 1) % kFp32FlushTiles == 0) T::flush(acc, t64, t64st);
                     else T::tile_done(acc);
                 } else if constexpr (P == NB_EX && MODE != kModePot) {
                     T::tile_done(acc);
-                } else if constexpr (P == NB_FP64 && NB_FP64_POT_FF && MODE != kModePot) {
+                } else if constexpr (P == NB_FP64) {
                     T::tile_done(acc);
                 }
             }
@@ -948,7 +988,9 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
         }
 
         double o[10];
-        T::finish(acc, t64, t64st, o);
+        if constexpr (P == NB_FP64) T::finish(me, acc, o);
+        else if constexpr (P == kPrecPot) T::finish(acc, o);
+        else T::finish(acc, t64, t64st, o);
         // lanes sharing an i: butterfly sum (fixed order)
         for (int w = gl >> 1; w >= 1; w >>= 1) {
 #pragma unroll

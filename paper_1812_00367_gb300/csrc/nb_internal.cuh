@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/nb.h"
+#include "nb_fixed.cuh"
 
 namespace nb {
 
@@ -25,7 +26,7 @@ constexpr int kTJ = 64;        // j-particles per shared-memory tile
 #define NB_EVAL_MIN_BLOCKS 4  // resident evaluation CTAs per SM the compiler must allow
 #endif
 #ifndef NB_EVAL_UNROLL
-#define NB_EVAL_UNROLL 2      // j-loop unrolling of the FP64 / FP32 evaluation
+#define NB_EVAL_UNROLL 2      // j-loop unrolling of the FP32 evaluation
 #endif
 #ifndef NB_EX_LAZY
 // 1: the EX evaluation keeps its sums and intermediate products unnormalised
@@ -33,13 +34,6 @@ constexpr int kTJ = 64;        // j-particles per shared-memory tile
 // Measured: 1.126x the pair rate at N = 65536, and the same maximum errors
 // against FP64 at N = 2^20 (Kroupa masses, eps = 1e-5) to two digits.
 #define NB_EX_LAZY 1
-#endif
-#ifndef NB_FP64_ALL_FMA
-// 1: the FP64 evaluation issues its products and differences as FMAs with
-// run-time -0.0 / -1.0 operands.  On GB300, DADD and DMUL run at 84 % of the
-// DFMA instruction rate (nb_probe_fma_peak modes 5, 6 vs 0), and this form
-// measured 5.9 % faster for the whole pair evaluation.
-#define NB_FP64_ALL_FMA 1
 #endif
 // FP32 evaluation: its own ring depth, residency and place of the FP64
 // chunk totals (registers, or shared memory when NB_FP32_T64_SMEM)
@@ -78,34 +72,49 @@ constexpr uint32_t kErrIndex = 4u;   // a caller-given index outside its cluster
 // wait budget of a bounded device-side wait, nanoseconds
 constexpr unsigned long long kWaitBudgetNs = 2000000000ull;
 
+// Tag of the potential-only evaluation (FP64, energy diagnostics) beside the
+// nb_precision values.
+constexpr int kPrecPot = 64;
+
 // ------------------------------------------------------------ packed j-data
-#ifndef NB_FP64_POT_FF
-// 1: the FP64 pair terms sum the potential in float-float on the FP32 pipe
-// (m y from the mass's float pair and y's bits; renormalised every term, a
-// j-tile's sum added to an FP64 total), one DFMA fewer per pair: measured
-// +1.5 % FP64 pair rate, potential within 1e-12 of the oracle at N = 2^20
-// (the j record grows from 80 to 96 bytes)
-#define NB_FP64_POT_FF 1
-#endif
-// FP64: x, y, z, m, vx, vy, vz, ax, ay, az as five 16-byte pairs (and, with
-// NB_FP64_POT_FF, the mass as a float pair).
+// FP64 values (energy diagnostics, nb_predict's output): x, y, z, m, vx, vy,
+// vz, ax, ay, az as five 16-byte pairs.
 struct alignas(16) J64 {
     double2 q[5];  // (x,y) (z,m) (vx,vy) (vz,ax) (ay,az)
-#if NB_FP64_POT_FF
-    float2 mf;     // (m_hi, m_lo)
-    float2 pad_;
-#endif
 };
-// Fill the record's float-pair mass (no-op without NB_FP64_POT_FF).
-__host__ __device__ inline void j64_set_mass_split(J64 &w, double m) {
-#if NB_FP64_POT_FF
+// FP64 evaluation: the position as doubles, velocity and acceleration as
+// block fixed-point vectors (component k is w[k] 2^(e - 60), nb_fixed.cuh),
+// the mass as a 63-bit integer (|m| = mm 2^(em - 62)) and as a float pair.
+struct alignas(16) JFX {
+    double x[3];
+    uint64_t mm;
+    int64_t v[3], a[3];
+    float2 mf;      // (m_hi, m_lo) for the potential
+    int32_t eva;    // exponents: ev in the low half, ea in the high half
+    int32_t ems;    // 2 em + (m < 0)
+};
+static_assert(sizeof(JFX) == 96, "JFX layout");
+__device__ __forceinline__ int jfx_ev(const JFX &j) { return (int)(short)j.eva; }
+__device__ __forceinline__ int jfx_ea(const JFX &j) { return j.eva >> 16; }
+__device__ __forceinline__ int jfx_em(const JFX &j) { return j.ems >> 1; }
+__device__ __forceinline__ uint32_t jfx_sign(const JFX &j) { return (uint32_t)j.ems << 31; }
+__device__ __forceinline__ JFX jfx_pack(const double x[3], const double v[3], const double a[3],
+                                        double m) {
+    JFX w;
+    const Fx3 fv = fx_pack(v[0], v[1], v[2]), fa = fx_pack(a[0], a[1], a[2]);
+    for (int k = 0; k < 3; ++k) {
+        w.x[k] = x[k];
+        w.v[k] = fv.w[k];
+        w.a[k] = fa.w[k];
+    }
+    int em;
+    uint32_t sign;
+    fx_pack_mass(m, w.mm, em, sign);
     const float hi = (float)m;
     w.mf = make_float2(hi, (float)(m - (double)hi));
-    w.pad_ = make_float2(0.f, 0.f);
-#else
-    (void)w;
-    (void)m;
-#endif
+    w.eva = (int32_t)(((uint32_t)fa.e << 16) | ((uint32_t)fv.e & 0xffffu));
+    w.ems = 2 * em + (int32_t)(sign >> 31);
+    return w;
 }
 // EX and FP32X: 80 bytes per particle (hi/lo single pairs), stored as records of two
 // particles whose values interleave like the FP32 records below: value f of
@@ -179,8 +188,8 @@ struct Dev {
     // state (caller-owned), SoA [3][n]
     double *m, *x, *v, *a, *j, *s, *c, *t, *dt, *pot;
     // predicted j-arrays
-    void *jarr;        // precision-specific (J64 / JEX (EX, FP32X) / J32)
-    J64 *jarr64;       // FP64 copy (energy, nb_predict output); == jarr for FP64
+    void *jarr;        // precision-specific (JFX / JEX (EX, FP32X) / J32)
+    J64 *jarr64;       // FP64 copy (energy, nb_predict output)
     // select
     double *chunk_min;
     int32_t *chunk_cnt;
@@ -220,6 +229,11 @@ struct Dev {
     // read them as parameters, where converting eps2 in the kernel costs
     // FP64-pipe conversions wherever the compiler re-forms the values.
     float2 eps2_hi2, eps2_lo2;
+    // eps^2 = eps_x 2^(2 E - 58), eps_x in [2^58, 2^60], and its block's
+    // exponent field (E + 1023) << 20 (nb_fixed.cuh); both 0 for eps = 0
+    uint64_t eps_x;
+    uint32_t eps_emin;
+    FxK fxk;  // {1, 2} as run-time values (nb_fixed.cuh)
 };
 
 // eps^2 and its float-float pair (host side; every context and launch).
@@ -229,6 +243,8 @@ inline void set_eps2(Dev &d, double eps) {
     const float lo = (float)(d.eps2 - (double)hi);
     d.eps2_hi2 = make_float2(hi, hi);
     d.eps2_lo2 = make_float2(lo, lo);
+    fx_eps2(d.eps2, d.eps_x, d.eps_emin);
+    d.fxk = FxK{1, 2};
 }
 
 // How one evaluation launch obtains its work.
@@ -391,83 +407,6 @@ __device__ __forceinline__ float rsqrt_sfu(float x) {
 __device__ __forceinline__ float2 rsqrt_sfu(float2 x) {
     return make_float2(rsqrt_sfu(x.x), rsqrt_sfu(x.y));
 }
-#ifndef NB_FP64_RSQRT3
-// 1: the FP64 pair terms take 1/sqrt from rsqrt_f64_3 (three FP64
-// operations, the seed refined on the FP32 and integer pipes) instead of
-// rsqrt_f64_fma (five)
-#define NB_FP64_RSQRT3 1
-#endif
-
-// 1/sqrt(x) for a positive normal double x, with three FP64 operations.
-//  - x = 2^(2m) x', x' in [1, 4): an exact exponent shift (integer pipe).
-//  - x' as a float pair xh + xl (24 + 23 significant bits) from its bits:
-//    xh truncated (integer pipe), xl an integer of 23 bits turned into a
-//    float by the 2^23 bias trick (one FP32 subtraction) and scaled.
-//  - y0 = SFU 1/sqrt(xh); residual e = 1 - x' y0^2 from exact FP32 products
-//    (1 - u is exact by Sterbenz, u = xh y0^2 lying within 2^-21 of 1);
-//    c = y0 e (1/2 + 3e/8), the third-order step of the binomial series of
-//    (1 - e)^{-1/2}, so y0 + c is within about 2^-44 of 1/sqrt(x').
-//  - Y = y0 + c rounded to 30 significant bits and assembled as a double on
-//    the integer pipe (its exponent renormalised when the correction crosses
-//    a power of two), Y/2 by an exponent decrement.
-//  - One Newton step in FP64: y' = Y + (Y/2)(1 - x' Y^2); with
-//    |1 - x' Y^2| < 2^-28 its truncation error (3/8)(1 - x' Y^2)^2 is below
-//    2^-57, and the roundings of Y^2 and the last FMA stay near 1 ulp.
-//  - y = 2^-m y' (integer pipe, exact).
-__device__ __forceinline__ double rsqrt_f64_3(double x, double neg_zero) {
-    const int hx = __double2hiint(x), lx = __double2loint(x);
-    const int m = ((((unsigned)hx >> 20) & 0x7ff) - 1023) >> 1;  // floor(exponent / 2)
-    const int hxp = hx - (m << 21);                              // x' = 2^-2m x
-    const int exp_p = (hxp >> 20) - 1023;                        // 0 or 1
-    const double xp = __hiloint2double(hxp, lx);
-    const float xh =
-        __int_as_float((int)__funnelshift_l((unsigned)lx, (unsigned)(hxp - 0x38000000), 3));
-    const float l23 = __fsub_rn(__int_as_float(0x4B000000 | (((unsigned)lx >> 6) & 0x7FFFFFu)),
-                                8388608.0f);                     // next 23 bits, exact
-    const float xl = __fmul_rn(l23, __int_as_float((127 - 46 + exp_p) << 23));
-    const float y0 = rsqrt_sfu(xh);
-    const float p = __fmul_rn(y0, y0);
-    const float pe = __fmaf_rn(y0, y0, -p);
-    const float u = __fmul_rn(xh, p);
-    float ue = __fmaf_rn(xh, p, -u);
-    ue = __fmaf_rn(xh, pe, ue);
-    ue = __fmaf_rn(xl, p, ue);
-    const float e = __fsub_rn(__fsub_rn(1.0f, u), ue);
-    const float c = __fmul_rn(__fmul_rn(y0, e), __fmaf_rn(e, 0.375f, 0.5f));
-    // Y = y0 + c in units of 2^(ey - 29), ey the exponent of y0 (-1 or 0)
-    const int yb = __float_as_int(y0);
-    int ey = ((yb >> 23) & 0xff) - 127;
-    const float cs = __fmaf_rn(c, __int_as_float((127 + 29 - ey) << 23), 12582912.0f);
-    int M = (((yb & 0x7FFFFF) | 0x800000) << 6) + (__float_as_int(cs) - 0x4B400000);
-    if (M >= (1 << 30)) {
-        M >>= 1;
-        ey += 1;
-    } else if (M < (1 << 29)) {
-        M <<= 1;
-        ey -= 1;
-    }
-    const int frac = M - (1 << 29);
-    const int hy = ((ey + 1023) << 20) | (frac >> 9);
-    const int ly = (frac & 0x1FF) << 23;
-    const double Y = __hiloint2double(hy, ly);
-    const double Yh = __hiloint2double(hy - (1 << 20), ly);
-    const double Y2 = fma_rn_f64(Y, Y, neg_zero);
-    const double e2 = fma(-xp, Y2, 1.0);
-    const double yp = fma(Yh, e2, Y);
-    return __hiloint2double(__double2hiint(yp) - (m << 20), __double2loint(yp));
-}
-
-// 2x by adding one to the exponent field on the integer pipe (exact for
-// normal x whose double does not overflow).  Zero, subnormal, infinite and NaN
-// inputs are returned unchanged (a subnormal is then off by a factor two, at
-// the 1e-308 level; a NaN stays NaN).
-__device__ __forceinline__ double twice_int(double x) {
-    const int hi = __double2hiint(x);
-    const int ex = hi & 0x7ff00000;
-    const bool ok = ex != 0 && ex < 0x7fe00000;
-    return __hiloint2double(ok ? hi + 0x00100000 : hi, __double2loint(x));
-}
-
 // --------------------------------------------- packed two-lane FP32 (f32x2)
 // sm_100 and later execute FP32 add / multiply / FMA on a pair of floats in
 // one instruction (PTX add/sub/mul/fma.rn.f32x2): the same per-lane IEEE
@@ -701,21 +640,6 @@ __device__ __forceinline__ ffT<T> rsqrt_ff(ffT<T> r2) {
     const T corr = o_mul(o_mul(y0, e), o_fma(e, o_cst(y0, 0.375f), o_cst(y0, 0.5f)));
     if constexpr (NB_EX_LAZY) return ffT<T>{y0, corr};
     else return ff_renorm(y0, corr);
-}
-
-// A positive double y in [2^-74, 2^127] as a float pair, from its bits with
-// no FP64 instruction and no int-to-float conversion: hi = the top 24
-// significant bits (truncated), lo = the next 23 bits, an integer turned
-// into a float by the 2^23 bias trick (exact) and scaled by 2^(E - 1069)
-// (the remaining 6 bits dropped: the pair holds y to 2^-47).
-__device__ __forceinline__ ff ff_from_pos_double(double y) {
-    const int hi = __double2hiint(y);
-    const int lo = __double2loint(y);
-    const float yh = __int_as_float((int)__funnelshift_l((unsigned)lo, (unsigned)(hi - 0x38000000), 3));
-    const float scale = __int_as_float(((hi & 0x7ff00000) - (942 << 20)) << 3);  // 2^(E - 1069)
-    const float l23 = __fsub_rn(__int_as_float(0x4B000000 | (((unsigned)lo >> 6) & 0x7FFFFFu)),
-                                8388608.0f);
-    return ff{yh, __fmul_rn(l23, scale)};
 }
 
 // a.b, unnormalised (hi + lo with every error term in lo)

@@ -299,14 +299,16 @@ __global__ void __launch_bounds__(kSelTPB) k_predict(const Dev d, int also64, in
         predict_particle(d, i, tn, xp, vp, ap);
         const double m = d.m[i];
         const int64_t jx = jo + (i - off);
-        if (d.precision == NB_FP64 || also64) {
+        if (d.precision == NB_FP64) {
+            reinterpret_cast<JFX *>(d.jarr)[jx] = jfx_pack(xp, vp, ap, m);
+        }
+        if (also64) {
             J64 w;
             w.q[0] = make_double2(xp[0], xp[1]);
             w.q[1] = make_double2(xp[2], m);
             w.q[2] = make_double2(vp[0], vp[1]);
             w.q[3] = make_double2(vp[2], ap[0]);
             w.q[4] = make_double2(ap[1], ap[2]);
-            j64_set_mass_split(w, m);
             d.jarr64[jx] = w;
         }
         if (d.precision == NB_EX || d.precision == NB_FP32X) {
@@ -349,9 +351,11 @@ __global__ void k_pad(const Dev d) {
         w.q[0] = make_double2(far, far);
         w.q[1] = make_double2(far, 0.0);
         w.q[2] = w.q[3] = w.q[4] = make_double2(0.0, 0.0);
-        j64_set_mass_split(w, 0.0);
         d.jarr64[jx] = w;
-        if (d.precision == NB_EX || d.precision == NB_FP32X) {
+        if (d.precision == NB_FP64) {
+            const double x[3] = {far, far, far}, z[3] = {0.0, 0.0, 0.0};
+            reinterpret_cast<JFX *>(d.jarr)[jx] = jfx_pack(x, z, z, 0.0);
+        } else if (d.precision == NB_EX || d.precision == NB_FP32X) {
             float w[kJEXVals] = {};
             w[0] = w[1] = w[2] = (float)far;
             jpair_store<kJEXVals>(d.jarr, jx, w);

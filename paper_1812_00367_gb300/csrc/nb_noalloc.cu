@@ -23,7 +23,7 @@ constexpr int64_t kNaMaxN = 32768;       // particles (and active entries) per c
 constexpr int64_t kNaMaxItems = 256;     // work items that keep split partial sums
 constexpr int64_t kNaMaxTiles = kNaMaxN / 4 + 64;  // i-tiles (at least 4 i per tile)
 
-constexpr size_t kNaJarrBytes = (size_t)kNaMaxN * sizeof(J64);
+constexpr size_t kNaJarrBytes = (size_t)kNaMaxN * sizeof(JFX);
 constexpr size_t kNaPartBytes = (size_t)kNaMaxItems * 10 * kTPB * sizeof(double);
 constexpr size_t kNaTileBytes = (size_t)kNaMaxTiles * sizeof(int32_t);
 constexpr size_t kNaOffJarr = 0;
@@ -47,33 +47,27 @@ struct DevSlot {
 std::mutex g_na_mutex;
 DevSlot g_na_slots[128];
 
-// Pack the caller's [10][n] predicted values into J64 entries (96 bytes:
-// position, mass, velocity, acceleration and the mass as a float pair), pad to
-// whole 64-particle tiles with zero-mass particles far away, clear the tile
+// Pack the caller's [10][n] predicted values into the FP64 evaluation's
+// records (JFX, 96 bytes), pad to whole 64-particle tiles with zero-mass particles far away, clear the tile
 // counters and the error word, and write the one-cluster offsets.
 __global__ void k_na_prepare(unsigned char *base, const double *jp, int64_t n, int64_t npad,
                              int64_t tiles) {
-    J64 *jarr = reinterpret_cast<J64 *>(base + kNaOffJarr);
+    JFX *jarr = reinterpret_cast<JFX *>(base + kNaOffJarr);
     int32_t *tc = reinterpret_cast<int32_t *>(base + kNaOffTile);
     NaAux *aux = reinterpret_cast<NaAux *>(base + kNaOffAux);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t i = i0; i < npad; i += stride) {
-        J64 w;
+        double x[3] = {1.0e6, 1.0e6, 1.0e6}, v[3] = {0.0, 0.0, 0.0}, a[3] = {0.0, 0.0, 0.0}, m = 0.0;
         if (i < n) {
-            w.q[0] = make_double2(jp[0 * n + i], jp[1 * n + i]);
-            w.q[1] = make_double2(jp[2 * n + i], jp[9 * n + i]);
-            w.q[2] = make_double2(jp[3 * n + i], jp[4 * n + i]);
-            w.q[3] = make_double2(jp[5 * n + i], jp[6 * n + i]);
-            w.q[4] = make_double2(jp[7 * n + i], jp[8 * n + i]);
-            j64_set_mass_split(w, jp[9 * n + i]);
-        } else {
-            w.q[0] = make_double2(1.0e6, 1.0e6);
-            w.q[1] = make_double2(1.0e6, 0.0);
-            w.q[2] = w.q[3] = w.q[4] = make_double2(0.0, 0.0);
-            j64_set_mass_split(w, 0.0);
+            for (int k = 0; k < 3; ++k) {
+                x[k] = jp[k * n + i];
+                v[k] = jp[(3 + k) * n + i];
+                a[k] = jp[(6 + k) * n + i];
+            }
+            m = jp[9 * n + i];
         }
-        jarr[i] = w;
+        jarr[i] = jfx_pack(x, v, a, m);
     }
     for (int64_t k = i0; k < tiles; k += stride) tc[k] = 0;
     if (i0 == 0) {
@@ -170,7 +164,6 @@ extern "C" nb_status nb_evaluate_noalloc(const double *jpred, int64_t n, double 
     d.offsets = aux->offsets;
     d.jofs = aux->jofs;
     d.jarr = slot.base + kNaOffJarr;
-    d.jarr64 = reinterpret_cast<J64 *>(slot.base + kNaOffJarr);
     d.partial = reinterpret_cast<double *>(slot.base + kNaOffPart);
     d.partial_cap = kNaMaxItems * 10 * kTPB;  // doubles
     d.tile_cnt = reinterpret_cast<int32_t *>(slot.base + kNaOffTile);

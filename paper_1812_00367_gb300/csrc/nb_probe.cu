@@ -224,12 +224,19 @@ extern "C" nb_status nb_selftest_wait_timeout(double budget_seconds, void *strea
 
 // ------------------------------------------------ reciprocal square roots
 namespace {
-__global__ void k_rsqrt(int which, const double *x, double *y, int64_t n, double neg_zero) {
+__global__ void k_rsqrt(int which, const double *x, double *y, int64_t n, double neg_zero,
+                        nb::FxK K) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
          k += (int64_t)gridDim.x * blockDim.x) {
         const double v = x[k];
         if (which == 0) {
-            y[k] = NB_FP64_RSQRT3 ? nb::rsqrt_f64_3(v, neg_zero) : nb::rsqrt_f64_fma(v, neg_zero);
+            // the pair terms' root of r^2 + eps^2 with r = 0, eps^2 = x
+            uint64_t eps_x;
+            uint32_t emin;
+            nb::fx_eps2(v, eps_x, emin);
+            const nb::FxS zero[3] = {{0, 0}, {0, 0}, {0, 0}};
+            const nb::FxRoot t = nb::fx_root(zero, (int)(emin >> 20) - 1023, eps_x, emin, K);
+            y[k] = nb::fx_to_double((int64_t)(t.y >> 1), -61 - t.g + 1023);
         } else if (which == 2) {
             y[k] = nb::rsqrt_f64_fma(v, neg_zero);
         } else {
@@ -249,6 +256,7 @@ extern "C" nb_status nb_probe_rsqrt(int32_t which, const double *x, double *y, i
     if (n < 0 || (n > 0 && (!x || !y))) return NB_EINVAL;
     if (n == 0) return NB_OK;
     const int blocks = (int)std::min<int64_t>((n + 255) / 256, 4096);
-    k_rsqrt<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(which, x, y, n, -0.0);
+    k_rsqrt<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(which, x, y, n, -0.0,
+                                                                      nb::FxK{1, 2});
     return cudaGetLastError() == cudaSuccess ? NB_OK : NB_ECUDA;
 }
