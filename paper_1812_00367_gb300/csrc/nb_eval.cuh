@@ -190,46 +190,64 @@ struct Prec<NB_FP64> {
         pair<false>(i, jj, self, c);
     }
     static __device__ __forceinline__ void finish(const I &i, const Acc &c, double o[10]) {
-        // a velocity that is not finite takes jerk and snap with it, an
-        // acceleration the snap (as v - 3 alpha r and the rest would)
+        // what is not finite spreads as in doubles: a position (seen in the
+        // acceleration, its differences are doubles) takes every sum, a
+        // velocity jerk and snap, an acceleration the snap
         const double nan = __hiloint2double(0x7ff80000, 0);
-        const bool bad_v = max(c.fv, i.ev) >= kFxBad, bad_a = bad_v || max(c.fa, i.ea) >= kFxBad;
+        const bool bad_x = !(isfinite(c.a[0]) && isfinite(c.a[1]) && isfinite(c.a[2]));
+        const bool bad_v = bad_x || max(c.fv, i.ev) >= kFxBad, bad_a = bad_v || max(c.fa, i.ea) >= kFxBad;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            o[k] = c.a[k];
+            o[k] = bad_x ? nan : c.a[k];
             o[3 + k] = bad_v ? nan : c.j[k];
             o[6 + k] = bad_a ? nan : c.s[k];
         }
-        o[9] = -(c.p + ((double)c.pf.hi + (double)c.pf.lo));
+        o[9] = bad_x ? nan : -(c.p + ((double)c.pf.hi + (double)c.pf.lo));
     }
 };
 
 // ========================================================= FP64 potential
-// The potential alone (energy diagnostics), from the FP64 records.
+// The potential alone (energy diagnostics), from the FP64 records: the root on
+// the integer pipes as in the FP64 pair terms, four FP64 instructions a pair
+// (differences and m y; 12 before).  Bound: the FP64 pipe (64 of 77 SM clocks
+// per warp of pairs).  Energy of N = 65536: 32.9 ms (1.31e11 pairs/s) against
+// 92.9 ms with the root and the products in doubles.
 template <>
 struct Prec<kPrecPot> {
     using J = J64;
     static constexpr int kPerRec = 1;
     struct I {
-        double x[3];
+        double x[3], m1;
+        uint64_t eps_x;
+        uint32_t emin;
+        FxK K;
     };
     struct Acc {
         double p;
     };
+    static __device__ __forceinline__ void prepare(I &i, const Dev &d) {
+        i.m1 = d.neg_one;
+        i.eps_x = d.eps_x;
+        i.emin = d.eps_emin;
+        i.K = d.fxk;
+    }
     static __device__ __forceinline__ I load_i(const J *jarr, int64_t k) {
         const J e = jarr[k];
-        return I{{e.q[0].x, e.q[0].y, e.q[1].x}};
+        I r;
+        r.x[0] = e.q[0].x;
+        r.x[1] = e.q[0].y;
+        r.x[2] = e.q[1].x;
+        return r;
     }
     static __device__ __forceinline__ void zero(Acc &c) { c.p = 0.0; }
-    static __device__ __forceinline__ void interact_pot(const I &i, const J &jj, bool self,
-                                                        double eps2, Acc &c) {
+    static __device__ __forceinline__ void interact_pot(const I &i, const J &jj, bool self, Acc &c) {
         const double2 q0 = jj.q[0], q1 = jj.q[1];
-        const double rx = q0.x - i.x[0], ry = q0.y - i.x[1], rz = q1.x - i.x[2];
-        double r2 = fma(rx, rx, fma(ry, ry, fma(rz, rz, eps2)));
-        double m = q1.y;
-        r2 = self ? 1.0 : r2;
-        m = self ? 0.0 : m;
-        c.p = fma(m, rsqrt_f64(r2), c.p);
+        const double r[3] = {fma_rn_f64(i.x[0], i.m1, q0.x), fma_rn_f64(i.x[1], i.m1, q0.y),
+                             fma_rn_f64(i.x[2], i.m1, q1.x)};
+        const Fx3 R = fx_decode(r, i.emin);
+        const FxS Rs[3] = {fx_split(R.w[0]), fx_split(R.w[1]), fx_split(R.w[2])};
+        const FxRoot t = fx_root(Rs, R.e, i.eps_x, i.emin, i.K);
+        c.p = fma(self ? 0.0 : q1.y, fx_root_to_double(t, R.e), c.p);
     }
     static __device__ __forceinline__ void finish(const Acc &c, double o[10]) {
 #pragma unroll
@@ -882,7 +900,7 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
             if (bad) atomicOr(d.err, kErrIndex);  // caller-given index outside the cluster
         }
         typename T::I me = T::load_i(jc, ji);
-        if constexpr (P == NB_FP64) T::prepare(me, d);
+        if constexpr (P == NB_FP64 || P == kPrecPot) T::prepare(me, d);
         typename T::Acc acc;
         T::zero(acc);
         double t64r[EvalCfg<P>::t64_smem ? 1 : 10];
@@ -890,7 +908,6 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
         constexpr int t64st = EvalCfg<P>::t64_smem ? kTPB : 1;
 #pragma unroll
         for (int q = 0; q < 10; ++q) t64[q * t64st] = 0.0;
-        const double eps2 = d.eps2;
         const float2 eps2f2 = d.eps2_hi2;
         const ff2 eps2ff2{d.eps2_hi2, d.eps2_lo2};
 
@@ -914,7 +931,7 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
                 const int64_t jbase = tt * kTJ;
                 if constexpr (MODE == kModePot) {
                     for (int k = jsub; k < kTJ; k += gl)
-                        T::interact_pot(me, tl[k], jbase + k == ji, eps2, acc);
+                        T::interact_pot(me, tl[k], jbase + k == ji, acc);
                 } else if constexpr (P == NB_FP32 && uses_order4_terms(MODE)) {
                     // record k holds particles 2k and 2k + 1 of the tile
 #pragma unroll kEvalUnroll

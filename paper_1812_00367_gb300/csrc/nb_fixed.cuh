@@ -373,6 +373,15 @@ NB_HD FxRoot fx_root(const FxS R[3], int e, uint64_t eps_x, uint32_t emin_field,
     return o;
 }
 
+// 1/sqrt(r^2 + eps^2) as a double; no number when r (block exponent e) is not
+// finite.
+NB_HD double fx_root_to_double(const FxRoot &t, int e) {
+    const uint64_t m = (t.y + 0x200) >> 10;  // leading one at bit 52
+    uint32_t hi = (uint32_t)(m >> 32) + ((uint32_t)(1023 - 1 - t.g) << 20);
+    hi = e >= 1024 ? 0x7ff80000u : hi;
+    return fx_bits2d(hi, (uint32_t)m);
+}
+
 // q = |m| y^3, with the sign put back, as a double.
 NB_HD double fx_q(const FxRoot &t, uint64_t mm, int em, uint32_t sign, bool zero, FxK K) {
     const uint64_t y3 = fx_mulhi_u(t.y, t.y2, K);  // y^3 in units of 2^(-58 - 3 g)

@@ -357,34 +357,20 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 }
 
 // ---------------------------------------------------------------- FP64 rsqrt
-// 1/sqrt(r2) for r2 in [2^-126, 2^128).  Seed: the exponent and top 20
-// mantissa bits of r2 are moved into an FP32 word with integer operations,
-// the SFU gives rsqrt.approx, and the result is moved back the same way
-// (relative seed error below 2^-19).  One third-order step
-//   y = y0 (1 + e/2 + 3 e^2/8),  e = 1 - r2 y0^2
-// (the binomial series of (1 - e)^{-1/2}) leaves a truncation error of about
-// (5/16) e^3 < 2^-55; y0 has 21 significant bits, so y0^2 is exact.  Five FP64
-// operations, none of them on the seed.
-__device__ __forceinline__ double rsqrt_f64(double r2) {
-    const int hi = __double2hiint(r2);
-    const float f = __int_as_float((hi - 0x38000000) << 3);
-    float yf;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(f));
-    const double y0 = __hiloint2double((__float_as_int(yf) >> 3) + 0x38000000, 0);
-    const double y2 = y0 * y0;
-    const double e = fma(-r2, y2, 1.0);
-    const double p = fma(e, 0.375, 0.5);
-    const double t = y0 * e;
-    return fma(t, p, y0);
-}
-
-// The same with its two products issued as FMAs against a run-time -0.0
-// (x*y + (-0) == x*y, signed zeros included): every instruction is a DFMA.
 __device__ __forceinline__ double fma_rn_f64(double a, double b, double c) {
     double r;
     asm("fma.rn.f64 %0, %1, %2, %3;" : "=d"(r) : "d"(a), "d"(b), "d"(c));
     return r;
 }
+// 1/sqrt(r2) for r2 in [2^-126, 2^128) in five FP64 operations (measured
+// beside the pair terms' own root, nb_probe_rsqrt).  Seed: the exponent and
+// top 20 mantissa bits of r2 are moved into an FP32 word with integer
+// operations, the SFU gives rsqrt.approx, and the result is moved back the
+// same way (relative seed error below 2^-19).  One third-order step
+//   y = y0 (1 + e/2 + 3 e^2/8),  e = 1 - r2 y0^2
+// (the binomial series of (1 - e)^{-1/2}) leaves a truncation error of about
+// (5/16) e^3 < 2^-55; y0 has 21 significant bits, so y0^2 is exact.  Products
+// are FMAs against a run-time -0.0 (x*y + (-0) == x*y, signed zeros included).
 __device__ __forceinline__ double rsqrt_f64_fma(double r2, double neg_zero) {
     const int hi = __double2hiint(r2);
     const float f = __int_as_float((hi - 0x38000000) << 3);

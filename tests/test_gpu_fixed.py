@@ -89,7 +89,7 @@ def _evaluate_predicted(nb, m, x, v, a, eps):
     return out.cpu().numpy()
 
 
-def test_nonfinite_velocity_and_acceleration(nb):
+def test_nonfinite_position_velocity_and_acceleration(nb):
     n = 130
     m, x, v = ic.plummer(n, seed=6)
     a = np.random.default_rng(6).normal(size=(n, 3))
@@ -98,8 +98,25 @@ def test_nonfinite_velocity_and_acceleration(nb):
     out = _evaluate_predicted(nb, m, x, bad, a, 1e-3)
     assert np.isfinite(out[0:3]).all() and np.isfinite(out[9]).all()
     assert np.isnan(out[3:9]).all()
+    bad = x.copy()
+    bad[7, 0] = np.nan
+    assert np.isnan(_evaluate_predicted(nb, m, bad, v, a, 1e-3)).all()
     bad = a.copy()
     bad[100, 2] = np.inf
     out = _evaluate_predicted(nb, m, x, v, bad, 1e-3)
     assert np.isfinite(out[0:6]).all() and np.isfinite(out[9]).all()
     assert not np.isfinite(out[6:9]).any()
+
+
+@pytest.mark.parametrize("eps", [1e-4, 0.0, 2.0])
+@pytest.mark.parametrize("n", [1, 2, 65, 1000])
+def test_potential_parity(nb, oracle, n, eps):
+    """The potential-only evaluation behind the energies, all particles."""
+    m, x, v = ic.plummer(max(n, 2), seed=n)
+    m, x, v = m[:n], x[:n], v[:n]
+    a = np.zeros((n, 3))
+    sim = nb.Simulation(m, x, v, eps=eps, keep_state=True)
+    _, epot, _, _ = sim.energy(0.0)
+    sim.close()
+    ref = 0.5 * float(np.sum(m * oracle.force(m, x, v, a, eps)[3]))
+    assert abs(epot - ref) <= 1e-13 * abs(ref)
