@@ -232,17 +232,18 @@ void plan_direct(const nb_ctx *ctx, int cluster, int32_t n_active, int &gl, int 
                  int &streamk, int64_t jtiles = -1) {
     const int b = 31 - __builtin_clz((unsigned)std::max(n_active, 1));
     const PlanEntry e = ctx->table[b];
-    gl = e.gl;
-    tiles = (int)cdiv(n_active, kTPB / gl);
     const int64_t ncl = ctx->h_offsets[cluster + 1] - ctx->h_offsets[cluster];
     const int64_t ntj = jtiles >= 0 ? jtiles : cdiv(ncl, kTJ);  // j-tiles evaluated
+    gl = ctx->p.flags & NB_NO_STREAMK ? e.gl : sk_lanes(e.gl, n_active, ntj, ctx->grid_eval,
+                                                       ctx->p.precision);
+    tiles = (int)cdiv(n_active, kTPB / gl);
     streamk = !(ctx->p.flags & NB_NO_STREAMK) &&
               sk_use(tiles, kTPB / gl, ntj, ctx->grid_eval, ctx->d.partial_cap) ? 1 : 0;
     if (streamk) {
         split = 1;
         return;
     }
-    int64_t S = choose_split(tiles, ntj, e.target_items, ctx->grid_eval);
+    int64_t S = choose_split(tiles, ntj, e.target_items, ctx->grid_eval, ctx->p.precision);
     const int64_t per_item = 10LL * (kTPB / gl);  // partial doubles per item
     if (S > 1 && (int64_t)tiles * S * per_item > ctx->d.partial_cap)
         S = std::max<int64_t>(1, ctx->d.partial_cap / (per_item * tiles));

@@ -750,6 +750,48 @@ struct SmemLayout {
     int fail;
 };
 
+// Sums over the gl lanes that share an i, by recursive halving: at each step a
+// lane keeps half of its values and hands the other half to its partner, so
+// ten values over 32 lanes take 12 additions and 12 exchanges a lane where a
+// butterfly on every value takes 50 of each (an FP64 addition is 16 SM clocks
+// a warp: 12,800 against 3,000 clocks for the 16 resident warps).  Every sum is
+// the butterfly's: own + partner at distances gl / 2, ..., 1.
+struct LaneSums {
+    int off, lim, n;  // the lane holds the sums off .. min(off + n, lim) - 1
+    // element q of the lane's i goes to dst[q * st]
+    __device__ __forceinline__ void store(const double o[10], double *dst, int st) const {
+#pragma unroll
+        for (int k = 0; k < 10; ++k)
+            if (k < n && off + k < lim) dst[(off + k) * st] = o[k];
+    }
+};
+template <int N>
+__device__ __forceinline__ void halve_lanes(double *o, LaneSums &s, int w, int jsub) {
+    constexpr int H = (N + 1) / 2;  // the lower lane keeps H values, the upper N - H
+    const bool up = (jsub & w) != 0;
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+        const double hi = H + k < N ? o[H + k] : 0.0;
+        const double keep = N == 1 ? o[0] : (up ? hi : o[k]), give = N == 1 ? o[0] : (up ? o[k] : hi);
+        o[k] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+    }
+    s.n = H;
+    if (N == 1) s.lim = up ? s.off : s.lim;  // both hold it: one writes
+    else if (up) s.off += H;
+    else s.lim = min(s.lim, s.off + H);
+}
+// Not inlined: inlined, it changed the register allocation of the pair loops
+// (FP32 2 % slower).
+static __device__ __noinline__ LaneSums reduce_lanes(double *o, int gl, int jsub) {
+    LaneSums s{0, 10, 10};
+    if (gl >= 2) halve_lanes<10>(o, s, gl >> 1, jsub);
+    if (gl >= 4) halve_lanes<5>(o, s, gl >> 2, jsub);
+    if (gl >= 8) halve_lanes<3>(o, s, gl >> 3, jsub);
+    if (gl >= 16) halve_lanes<2>(o, s, gl >> 4, jsub);
+    if (gl >= 32) halve_lanes<1>(o, s, gl >> 5, jsub);
+    return s;
+}
+
 __device__ __forceinline__ int find_cluster(const ClusterPlan *plan, int nc, int64_t item) {
     int lo = 0, hi = nc - 1;  // largest c with plan[c].item0 <= item
     while (lo < hi) {
@@ -1008,15 +1050,13 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
         if constexpr (P == NB_FP64) T::finish(me, acc, o);
         else if constexpr (P == kPrecPot) T::finish(acc, o);
         else T::finish(acc, t64, t64st, o);
-        // lanes sharing an i: butterfly sum (fixed order)
-        for (int w = gl >> 1; w >= 1; w >>= 1) {
-#pragma unroll
-            for (int q = 0; q < 10; ++q) o[q] += __shfl_xor_sync(0xffffffffu, o[q], w);
-        }
+        // lanes sharing an i: after this, the lane holds the sums q in
+        // [held.off, held.lim) of its i in o[0 ..]
+        const LaneSums held = reduce_lanes(o, R.gl, tid & (R.gl - 1));
 
         // ---- epilogue: the piece's bookkeeping comes back from shared memory
         const int tile = R.tile, A = R.A, split = R.split;
-        const int Ti = kTPB / gl;
+        const int Ti = kTPB / R.gl, ilane_e = tid / R.gl;
         const int64_t ntj = R.ntj;
         const bool sk = R.sk;
         // pieces of this i-tile: split items, or the CTAs whose ranges meet it
@@ -1038,21 +1078,31 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
             if (sk) return ((sk_first + s) * sk_maxp + (s == 0 ? sk_loc0 : 0)) * (10 * Ti);
             return pslot0 + ((int64_t)tile * split + s) * (10 * Ti);
         };
-        if (npieces == 1) {
-            if (valid && jsub == 0) {
+        if (npieces == 1 && Ti == kTPB) {
+            const int il = tile * Ti + tid;
+            if (il < A) {
                 bool bad;
-                const int il = tile * Ti + ilane;
                 const int64_t gi = i_of(il, bad);
                 if (!bad) finalize_one<P, MODE>(d, L, c, gi, il, o);
+            }
+        } else if (npieces == 1) {
+            // one thread per i gathers its ten sums
+            held.store(o, S.red + ilane_e, Ti);
+            __syncthreads();
+            const int il = tile * Ti + tid;
+            if (tid < Ti && il < A) {
+                double sum[10];
+#pragma unroll
+                for (int q = 0; q < 10; ++q) sum[q] = S.red[q * Ti + tid];
+                bool bad;
+                const int64_t gi = i_of(il, bad);
+                if (!bad) finalize_one<P, MODE>(d, L, c, gi, il, sum);
             }
         } else {
             // this CTA's piece of the tile
             double *part = d.partial + (sk ? piece_slot((int64_t)blockIdx.x - sk_first)
                                            : pslot0 + R.local * (int64_t)(10 * Ti));
-            if (jsub == 0) {
-#pragma unroll
-                for (int q = 0; q < 10; ++q) part[q * Ti + ilane] = o[q];
-            }
+            held.store(o, part + ilane_e, Ti);
             __threadfence();
             __syncthreads();
             if (tid == 0) {
@@ -1064,36 +1114,49 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
                 // Last CTA of this i-tile: add the partials of its pieces for
                 // every (i, q) pair in two fixed-order levels.  Level 1: thread
                 // (p, r) sums the r-th contiguous group of pieces of pair p in
-                // piece order; level 2 adds the R group sums in group order.  The
-                // order depends only on (pieces, valid i count), so results are
-                // reproducible.
+                // piece order; level 2 adds the Rg group sums in group order.
+                // The order depends only on the pieces and the tile's width, so
+                // results are reproducible and the same for every i.  Groups of
+                // eight pieces (more when S.red would overflow): a tile of few
+                // i's may have hundreds of pieces, and a chain of that many
+                // loads and additions in a handful of threads took longer than
+                // the pairs themselves.
                 __threadfence();
                 const int nv = min(Ti, A - tile * Ti);     // valid i in this tile
                 const int npair = nv * 10;
-                const int Rg = max(1, kTPB / npair);
+                const int Rg = min((npieces + 7) / 8, kTPB / Ti);
                 for (int w = tid; w < npair * Rg; w += kTPB) {
                     const int p = w % npair, r = w / npair;
                     const int q = p / nv, il = p % nv;
                     const int s0 = (int)((int64_t)npieces * r / Rg), s1 = (int)((int64_t)npieces * (r + 1) / Rg);
+                    // pieces at a fixed stride (the first of a stream-K tile
+                    // sits elsewhere), eight loads in flight
+                    const int64_t stride = (sk ? sk_maxp : (int64_t)1) * (10 * Ti);
+                    const double *base = d.partial + piece_slot(0) + q * Ti + il;
+                    const double *rest = base - (sk ? sk_loc0 : (int64_t)0) * (10 * Ti);
                     double acc2 = 0.0;
-                    if (sk) {
-                        for (int sp = s0; sp < s1; ++sp) acc2 += __ldcg(d.partial + piece_slot(sp) + q * Ti + il);
-                    } else {
-                        const double *base = d.partial + piece_slot(0);
-#pragma unroll 4
-                        for (int sp = s0; sp < s1; ++sp) acc2 += __ldcg(base + (int64_t)sp * (10 * Ti) + q * Ti + il);
+                    for (int sp = s0; sp < s1; sp += 8) {
+                        double t[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            t[u] = sp + u < s1 ? __ldcg(sp + u == 0 ? base : rest + (sp + u) * stride) : 0.0;
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            if (sp + u < s1) acc2 += t[u];
                     }
                     S.red[r * npair + p] = acc2;
+                }
+                __syncthreads();
+                for (int p = tid; p < npair; p += kTPB) {
+                    double a2 = S.red[p];
+                    for (int r = 1; r < Rg; ++r) a2 += S.red[r * npair + p];
+                    S.red[p] = a2;
                 }
                 __syncthreads();
                 if (tid < nv) {
                     double sum[10];
 #pragma unroll
-                    for (int q = 0; q < 10; ++q) {
-                        double a2 = 0.0;
-                        for (int r = 0; r < Rg; ++r) a2 += S.red[r * npair + q * nv + tid];
-                        sum[q] = a2;
-                    }
+                    for (int q = 0; q < 10; ++q) sum[q] = S.red[q * nv + tid];
                     const int il = tile * Ti + tid;
                     bool bad;
                     const int64_t g2 = i_of(il, bad);

@@ -312,6 +312,33 @@ __host__ __device__ inline bool sk_use(int64_t tiles, int64_t Ti, int64_t ntj, i
     return G * sk_max_pieces(U, G, ntj) * 10 * Ti <= partial_cap;
 }
 
+// Lanes per i of a single cluster's launch: the table's choice for the
+// active-set size, doubled while the launch has fewer units than stream-K
+// wants (few active particles, or a small cluster) and an even share still
+// gives every lane of the grid kLanesMinPairs pairs: below that the epilogue
+// of the extra pieces costs more than the idle SMs.  The share a lane needs
+// falls with the cost of a pair.  Measured (us, one evaluation, table's lanes
+// -> these): N = A = 1024 FP64 128 -> 59, EX 59 -> 47; N = A = 256 FP64 64 -> 15;
+// FP32, N = A = 1024, 21 -> 37 if its lanes were doubled too.
+__host__ __device__ constexpr int sk_min_pairs(int precision) {
+    return precision == NB_FP64 ? 0 : precision == NB_EX ? 8 : precision == NB_FP32X ? 32 : 64;
+}
+__host__ __device__ inline int sk_lanes(int gl, int64_t A, int64_t ntj, int64_t G, int precision) {
+    if (A * ntj * kTJ < (int64_t)sk_min_pairs(precision) * G * kTPB) return gl;
+    while (gl < 32 && cdiv(A, kTPB / gl) * ntj < kStreamKMinUnits * G) gl *= 2;
+    return gl;
+}
+// Most j-ranges a launch is split into: at least kMinTilesPerItem j-tiles
+// each; the FP64 terms, whose pairs cost most, go down to one tile while that
+// makes no more than 64 ranges.  Measured (us, FP64, N = 1024, A = 1): 20 ->
+// 14; N = 4096, A = 2: 21 -> 15; with one tile everywhere N = 65536, A = 2 rose
+// from 29 to 37.
+__host__ __device__ inline int64_t split_max(int64_t ntj, int precision) {
+    const int64_t s = ntj / kMinTilesPerItem > 1 ? ntj / kMinTilesPerItem : 1;
+    const int64_t fine = ntj < 64 ? ntj : 64;
+    return precision == NB_FP64 && s < fine ? fine : s;
+}
+
 // Number of j-ranges (split S) for `tiles` i-tiles over a cluster of `ntj`
 // j-tiles.  Start from the bucket's target item count; keep at least
 // kMinTilesPerItem j-tiles per item; for `grid` resident CTAs, take the
@@ -320,8 +347,8 @@ __host__ __device__ inline bool sk_use(int64_t tiles, int64_t Ti, int64_t ntj, i
 // result depends on this cluster alone, so a cluster's plan (and therefore
 // its rounding) is the same in a batch as on its own.
 __host__ __device__ inline int64_t choose_split(int64_t tiles, int64_t ntj, int64_t target,
-                                                int64_t grid) {
-    const int64_t smax = ntj / kMinTilesPerItem > 1 ? ntj / kMinTilesPerItem : 1;
+                                                int64_t grid, int precision = NB_EX) {
+    const int64_t smax = split_max(ntj, precision);
     int64_t s0 = cdiv(target, tiles > 0 ? tiles : 1);
     s0 = s0 < 1 ? 1 : (s0 > smax ? smax : s0);
     if (grid <= 0) return s0;

@@ -222,17 +222,19 @@ __global__ void __launch_bounds__(kPlanTPB) k_plan(const Dev d, int mode_init, i
                 const int64_t ncl = d.offsets[c + 1] - d.offsets[c];
                 const int A = mode_init ? (int)ncl : d.nact[c];
                 if (A > 0) {
-                    const PlanEntry e = d.table[31 - __clz(A)];
-                    tiles = cdiv(A, kTPB / e.gl);
+                    PlanEntry e = d.table[31 - __clz(A)];
                     const long long ntj = cdiv(ncl, kTJ);
-                    if (d.n_clusters == 1 && !d.streamk_off &&
+                    const bool single = d.n_clusters == 1 && !d.streamk_off;
+                    if (single) e.gl = sk_lanes(e.gl, A, ntj, d.grid_eval, d.precision);
+                    tiles = cdiv(A, kTPB / e.gl);
+                    if (single &&
                         sk_use(tiles, kTPB / e.gl, ntj, d.grid_eval, d.partial_cap)) {
                         // one cluster, enough work: stream-K ranges (one "item")
                         items = 1;
                         pl = ClusterPlan{e.gl, 1, (int)tiles, A, 0, 0, 0, 1, 0};
                     } else {
                         const long long S =
-                            fallback ? 1 : choose_split(tiles, ntj, e.target_items, d.grid_eval);
+                            fallback ? 1 : choose_split(tiles, ntj, e.target_items, d.grid_eval, d.precision);
                         items = tiles * S;
                         pl = ClusterPlan{e.gl, (int)S, (int)tiles, A, 0, 0, 0, 0, 0};
                     }

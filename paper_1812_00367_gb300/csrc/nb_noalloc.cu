@@ -130,10 +130,11 @@ extern "C" nb_status nb_evaluate_noalloc(const double *jpred, int64_t n, double 
         slot = g_na_slots[dev];
     }
     // plan: lanes per i from the active-set size, splits within the arena
-    const int gl = n_active < 64 ? 32 : (n_active < 1024 ? 8 : (n_active < 4096 ? 2 : 1));
-    const int tiles = (int)cdiv(n_active, kTPB / gl);
     const int64_t ntj = cdiv(n, kTJ);
-    int64_t split = choose_split(tiles, ntj, 8LL * slot.grid, slot.grid);
+    const int gl = sk_lanes(n_active < 64 ? 32 : (n_active < 1024 ? 8 : (n_active < 4096 ? 2 : 1)),
+                            n_active, ntj, slot.grid, NB_FP64);
+    const int tiles = (int)cdiv(n_active, kTPB / gl);
+    int64_t split = choose_split(tiles, ntj, 8LL * slot.grid, slot.grid, NB_FP64);
     const int64_t per_item = 10LL * (kTPB / gl);         // partial doubles per item
     const int64_t cap = kNaMaxItems * 10LL * kTPB;        // arena partial doubles
     if (split > 1 && (int64_t)tiles * split * per_item > cap)
