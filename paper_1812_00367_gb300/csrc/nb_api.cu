@@ -437,8 +437,10 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
 
     int64_t *d_offs = nullptr, *d_jofs = nullptr, *d_cb = nullptr, *d_ce = nullptr;
     int32_t *d_ccl = nullptr, *d_cc0 = nullptr;
-    size_t jbytes = p->precision == NB_FP64 ? sizeof(JFX)
-                    : (p->precision == NB_FP32 ? sizeof(J32) : sizeof(JEX));  // EX, FP32X
+    // bytes per particle (the single-precision records hold two; clusters are
+    // padded to whole tiles, so nj is even)
+    const size_t jbytes = p->precision == NB_FP64 ? sizeof(JFX)
+                          : (p->precision == NB_FP32 ? sizeof(J32P) : sizeof(JEXP)) / 2;  // EX, FP32X
 #define ALLOC(ptr, cnt)                                                                      \
     do {                                                                                     \
         cudaError_t ee = dalloc(ctx, &(ptr), (cnt));                                         \

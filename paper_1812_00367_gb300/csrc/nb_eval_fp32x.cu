@@ -18,9 +18,11 @@ cudaError_t launch_eval_fp32x(const Dev &d, int mode, const EvalLaunch &L, int g
     }
 }
 
+// At most 4 CTAs per SM: the grid cuts a launch into its pieces, and the FP32
+// sums' rounding follows the pieces.
 int occupancy_fp32x(int mode) {
-    if (is_order4_mode(mode)) return occupancy_t<NB_FP32X, kModeStep4>();
-    return occupancy_t<NB_FP32X, kModeStep>();
+    const int b = is_order4_mode(mode) ? occupancy_t<NB_FP32X, kModeStep4>() : occupancy_t<NB_FP32X, kModeStep>();
+    return b < 4 ? b : 4;
 }
 
 }  // namespace nb

@@ -116,40 +116,40 @@ __device__ __forceinline__ JFX jfx_pack(const double x[3], const double v[3], co
     w.ems = 2 * em + (int32_t)(sign >> 31);
     return w;
 }
-// EX and FP32X: 80 bytes per particle (hi/lo single pairs), stored as records of two
-// particles whose values interleave like the FP32 records below: value f of
-// lane l of record r is float r * 40 + 2 f + l, f in the order
+// EX and FP32X: records of two particles whose values interleave like the FP32
+// records below: value f of lane l of a record is its float 2 f + l, f in the
+// order
 //   xh, yh, zh, mh, xl, yl, zl, ml, vxh, vyh, vzh, axh, vxl, vyl, vzl, axl,
 //   ayh, azh, ayl, azl
 // so q[k] of a record holds (value 2k of lanes 0, 1; value 2k + 1 of lanes 0, 1).
-struct alignas(16) JEX {  // one particle's share of the array (sizing only)
-    float4 q[5];
-};
+// The last 16 bytes are padding: lanes that share an i read records side by
+// side, and at a stride of 176 bytes eight of them meet 32 different banks (at
+// 160 bytes pairs of them collide).
 struct alignas(16) JEXP {  // a record of two particles
-    float4 q[10];
+    float4 q[11];
 };
 constexpr int kJEXVals = 20;
-// FP32: 64 bytes per particle, stored as records of two particles whose
-// values interleave, so that one 16-byte shared-memory load gives two
-// two-lane operands of the packed FP32 arithmetic.  Value f of lane l (the
-// particle's index parity) of record r is float r * 32 + 2 f + l, f in the
-// order xh, yh, zh, m, xl, yl, zl, ax, vxh, vyh, vzh, ay, vxl, vyl, vzl, az:
+// FP32: records of two particles whose values interleave, so that one 16-byte
+// shared-memory load gives two two-lane operands of the packed FP32
+// arithmetic.  Value f of lane l (the particle's index parity) of a record is
+// its float 2 f + l, f in the order
+// xh, yh, zh, m, xl, yl, zl, ax, vxh, vyh, vzh, ay, vxl, vyl, vzl, az:
 //   q[0] = (xh0, xh1, yh0, yh1)  q[1] = (zh0, zh1, m0, m1)
 //   q[2] = (xl0, xl1, yl0, yl1)  q[3] = (zl0, zl1, ax0, ax1)
 //   q[4] = (vxh0, vxh1, vyh0, vyh1)  q[5] = (vzh0, vzh1, ay0, ay1)
 //   q[6] = (vxl0, vxl1, vyl0, vyl1)  q[7] = (vzl0, vzl1, az0, az1)
-struct alignas(16) J32 {  // one particle's share of the array (sizing only)
-    float4 q[4];
-};
+// and 16 bytes of padding: at 128 bytes every record of a warp's lanes starts
+// in the same bank (8 lanes an i: 8-fold conflicts; FP32, N = 16384, A = 1000:
+// 240 us, with the padding 66 us).
 struct alignas(16) J32P {  // a record of two particles
-    float4 q[8];
+    float4 q[9];
 };
 constexpr int kJ32Vals = 16;
-// Write particle jx's NV values (the orders above) into a two-particle
-// record array (FP32: NV = 16, EX: NV = 20).
-template <int NV>
+// Write particle jx's NV values (the orders above) into an array of
+// two-particle records Rec (FP32: NV = 16, EX: NV = 20).
+template <class Rec, int NV>
 __device__ __forceinline__ void jpair_store(void *jarr, int64_t jx, const float v[NV]) {
-    float *p = reinterpret_cast<float *>(jarr) + (jx >> 1) * (2 * NV) + (jx & 1);
+    float *p = reinterpret_cast<float *>(reinterpret_cast<Rec *>(jarr) + (jx >> 1)) + (jx & 1);
 #pragma unroll
     for (int f = 0; f < NV; ++f) p[2 * f] = v[f];
 }
@@ -188,7 +188,7 @@ struct Dev {
     // state (caller-owned), SoA [3][n]
     double *m, *x, *v, *a, *j, *s, *c, *t, *dt, *pot;
     // predicted j-arrays
-    void *jarr;        // precision-specific (JFX / JEX (EX, FP32X) / J32)
+    void *jarr;        // precision-specific (JFX / JEXP (EX, FP32X) / J32P)
     J64 *jarr64;       // FP64 copy (energy, nb_predict output)
     // select
     double *chunk_min;

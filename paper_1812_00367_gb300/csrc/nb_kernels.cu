@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(kSelTPB) k_predict(const Dev d, int also64, in
             const float w[kJEXVals] = {xh[0], xh[1], xh[2], mh, xl[0], xl[1], xl[2], ml,
                                        vh[0], vh[1], vh[2], ah[0], vl[0], vl[1], vl[2], al[0],
                                        ah[1], ah[2], al[1], al[2]};
-            jpair_store<kJEXVals>(d.jarr, jx, w);
+            jpair_store<JEXP, kJEXVals>(d.jarr, jx, w);
         } else if (d.precision == NB_FP32) {
             float xh[3], xl[3], vh[3], vl[3];
             for (int q = 0; q < 3; ++q) {
@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(kSelTPB) k_predict(const Dev d, int also64, in
                                        xl[0], xl[1], xl[2], __double2float_rn(ap[0]),
                                        vh[0], vh[1], vh[2], __double2float_rn(ap[1]),
                                        vl[0], vl[1], vl[2], __double2float_rn(ap[2])};
-            jpair_store<kJ32Vals>(d.jarr, jx, w);
+            jpair_store<J32P, kJ32Vals>(d.jarr, jx, w);
         }
     }
 }
@@ -360,11 +360,11 @@ __global__ void k_pad(const Dev d) {
         } else if (d.precision == NB_EX || d.precision == NB_FP32X) {
             float w[kJEXVals] = {};
             w[0] = w[1] = w[2] = (float)far;
-            jpair_store<kJEXVals>(d.jarr, jx, w);
+            jpair_store<JEXP, kJEXVals>(d.jarr, jx, w);
         } else if (d.precision == NB_FP32) {
             float w[kJ32Vals] = {};
             w[0] = w[1] = w[2] = (float)far;
-            jpair_store<kJ32Vals>(d.jarr, jx, w);
+            jpair_store<J32P, kJ32Vals>(d.jarr, jx, w);
         }
     }
 }
