@@ -6,6 +6,7 @@
 // round trips.  Kernel launches go to the caller's stream.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -71,9 +72,9 @@ struct nb_ctx {
     std::vector<PlanEntry> table;
     PlanEntry *d_table = nullptr;
     cudaGraphExec_t g_step = nullptr;    // one block step
-    cudaGraphExec_t g_multi = nullptr;   // kMultiSteps block steps + busy readback
-    int32_t *h_busy = nullptr;           // pinned
-    double *h_tend = nullptr;            // pinned
+    cudaGraphExec_t g_multi = nullptr;   // kMultiSteps block steps, a look ahead and its readback
+    Ctl *d_ctl = nullptr;
+    Ctl *h_ctl = nullptr;                // pinned: [0] read back, [1] written to the device
     std::string err;
     // launch accounting and evaluation timing (NB_TIME_EVAL)
     int64_t launches = 0;
@@ -145,13 +146,16 @@ nb_status upload_table(nb_ctx *ctx) {
     return NB_OK;
 }
 
-nb_status check_device_error(nb_ctx *ctx) {
-    uint32_t err = 0;
-    NB_CU(ctx, cudaMemcpy(&err, ctx->d.err, sizeof(err), cudaMemcpyDeviceToHost));
+nb_status error_status(nb_ctx *ctx, uint32_t err) {
     if (err & kErrTimeout) return fail(ctx, NB_ETIMEOUT, "device: a bounded wait timed out");
     if (err & kErrIndex) return fail(ctx, NB_EINVAL, "device: an active index lies outside its cluster");
     if (err & kErrNonFinite) return fail(ctx, NB_ENONFINITE, "device: non-finite value in the state");
     return NB_OK;
+}
+nb_status check_device_error(nb_ctx *ctx) {
+    uint32_t err = 0;
+    NB_CU(ctx, cudaMemcpy(&err, ctx->d.err, sizeof(err), cudaMemcpyDeviceToHost));
+    return error_status(ctx, err);
 }
 
 constexpr int kKernelsPerStep = 5;
@@ -160,7 +164,7 @@ constexpr int kKernelsPerStep = 5;
 // event pair timing its evaluation launch (-1: none).
 cudaError_t enqueue_step(nb_ctx *ctx, cudaStream_t st, int slot) {
     cudaError_t e;
-    if ((e = launch_select_min(ctx->d, st)) != cudaSuccess) return e;
+    if ((e = launch_select_min(ctx->d, 0, st)) != cudaSuccess) return e;
     // the compaction, the planner and the predictor all need only pass 1's
     // t_next and counts: three graph branches, joined before the evaluation
     if ((e = cudaEventRecord(ctx->fork, st)) != cudaSuccess) return e;
@@ -195,34 +199,38 @@ void harvest_events(nb_ctx *ctx, int first, int count) {
     }
 }
 
-nb_status build_graphs(nb_ctx *ctx) {
-    if (ctx->g_step) return NB_OK;
-    for (int which = 0; which < 2; ++which) {
-        cudaGraph_t g = nullptr;
-        NB_CU(ctx, cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = cudaSuccess;
-        const int steps = which == 0 ? 1 : kMultiSteps;
-        const bool timed = !ctx->ev.empty();
-        for (int k = 0; k < steps && e == cudaSuccess; ++k)
-            e = enqueue_step(ctx, ctx->cap_stream, !timed ? -1 : (which == 0 ? kMultiSteps : k));
-        if (e == cudaSuccess && which == 1)
-            e = cudaMemcpyAsync(ctx->h_busy, ctx->d.busy, sizeof(int32_t), cudaMemcpyDeviceToHost,
-                                ctx->cap_stream);
-        cudaError_t e2 = cudaStreamEndCapture(ctx->cap_stream, &g);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "capture");
-        if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "cudaStreamEndCapture");
-        cudaGraphExec_t ex = nullptr;
-        e = cudaGraphInstantiate(&ex, g, 0);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaGraphInstantiate");
-        (which == 0 ? ctx->g_step : ctx->g_multi) = ex;
+// One block step (which = 0); or kMultiSteps of them, then selection pass 1
+// once more, which tells whether another step is due, and the control block's
+// readback (which = 1): a run that ends with a batch stops there instead of
+// replaying an idle batch (14-22 us a step).
+nb_status build_graph(nb_ctx *ctx, int which) {
+    cudaGraphExec_t &ex = which == 0 ? ctx->g_step : ctx->g_multi;
+    if (ex) return NB_OK;
+    cudaGraph_t g = nullptr;
+    NB_CU(ctx, cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
+    cudaError_t e = cudaSuccess;
+    const int steps = which == 0 ? 1 : kMultiSteps;
+    const bool timed = !ctx->ev.empty();
+    for (int k = 0; k < steps && e == cudaSuccess; ++k)
+        e = enqueue_step(ctx, ctx->cap_stream, !timed ? -1 : (which == 0 ? kMultiSteps : k));
+    if (e == cudaSuccess && which == 1) e = launch_select_min(ctx->d, 1, ctx->cap_stream);
+    if (e == cudaSuccess && which == 1)
+        e = cudaMemcpyAsync(ctx->h_ctl, ctx->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->cap_stream);
+    cudaError_t e2 = cudaStreamEndCapture(ctx->cap_stream, &g);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "capture");
+    if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "cudaStreamEndCapture");
+    e = cudaGraphInstantiate(&ex, g, 0);
+    cudaGraphDestroy(g);
+    if (e != cudaSuccess) {
+        ex = nullptr;
+        return cuda_fail(ctx, e, "cudaGraphInstantiate");
     }
     return NB_OK;
 }
 
 nb_status set_tend(nb_ctx *ctx, double t_end) {
-    *ctx->h_tend = t_end;
-    NB_CU(ctx, cudaMemcpyAsync(ctx->d.t_end, ctx->h_tend, sizeof(double), cudaMemcpyHostToDevice,
+    ctx->h_ctl[1].t_end = t_end;
+    NB_CU(ctx, cudaMemcpyAsync(&ctx->d_ctl->t_end, &ctx->h_ctl[1].t_end, sizeof(double), cudaMemcpyHostToDevice,
                                ctx->stream));
     return NB_OK;
 }
@@ -319,8 +327,7 @@ void nb_free(nb_ctx *ctx) {
     if (ctx->g_step) cudaGraphExecDestroy(ctx->g_step);
     if (ctx->g_multi) cudaGraphExecDestroy(ctx->g_multi);
     for (void *q : ctx->allocs) cudaFree(q);
-    if (ctx->h_busy) cudaFreeHost(ctx->h_busy);
-    if (ctx->h_tend) cudaFreeHost(ctx->h_tend);
+    if (ctx->h_ctl) cudaFreeHost(ctx->h_ctl);
     for (cudaEvent_t ev : ctx->ev) cudaEventDestroy(ev);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->cap_side) cudaStreamDestroy(ctx->cap_side);
@@ -376,8 +383,7 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->join2, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->join, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_busy, sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_tend, sizeof(double));
+    if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_ctl, 2 * sizeof(Ctl));
     if (e != cudaSuccess) {
         nb_status s = cuda_fail(nullptr, e, "nb_init: setup");
         nb_free(ctx);
@@ -474,12 +480,13 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
     ALLOC(d.partial, ctx->cap_items * 10 * kTPB);
     const int64_t max_tiles = n + n_clusters + 1;
     ALLOC(d.tile_cnt, max_tiles);
-    ALLOC(d.ctr_steps, 1);
-    ALLOC(d.ctr_inter, 1);
-    ALLOC(d.ctr_underflow, 1);
-    ALLOC(d.err, 1);
-    ALLOC(d.busy, 1);
-    ALLOC(d.t_end, 1);
+    ALLOC(ctx->d_ctl, 1);
+    d.ctr_steps = &ctx->d_ctl->steps;
+    d.ctr_inter = &ctx->d_ctl->inter;
+    d.ctr_underflow = &ctx->d_ctl->underflow;
+    d.err = &ctx->d_ctl->err;
+    d.busy = &ctx->d_ctl->busy;
+    d.t_end = &ctx->d_ctl->t_end;
     ALLOC(d.pot_tmp, n);
     ALLOC(d.energy_part, (int64_t)n_chunks * 8);
 #undef ALLOC
@@ -519,11 +526,7 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
     up(d_cc0, cluster_chunk0.data(), cluster_chunk0.size() * sizeof(int32_t));
     up(ctx->d_table, ctx->table.data(), kBuckets * sizeof(PlanEntry));
     if (ok && cudaMemsetAsync(d.tile_cnt, 0, max_tiles * sizeof(int32_t), s0) != cudaSuccess) ok = false;
-    if (ok && cudaMemsetAsync(d.ctr_steps, 0, sizeof(unsigned long long), s0) != cudaSuccess) ok = false;
-    if (ok && cudaMemsetAsync(d.ctr_inter, 0, sizeof(double), s0) != cudaSuccess) ok = false;
-    if (ok && cudaMemsetAsync(d.ctr_underflow, 0, sizeof(unsigned long long), s0) != cudaSuccess) ok = false;
-    if (ok && cudaMemsetAsync(d.err, 0, sizeof(uint32_t), s0) != cudaSuccess) ok = false;
-    if (ok && cudaMemsetAsync(d.busy, 0, sizeof(int32_t), s0) != cudaSuccess) ok = false;
+    if (ok && cudaMemsetAsync(ctx->d_ctl, 0, sizeof(Ctl), s0) != cudaSuccess) ok = false;
     if (ok && cudaMemsetAsync(d.sel_ctr, 0, sizeof(unsigned int), s0) != cudaSuccess) ok = false;
     // the chunk tables live in pageable host vectors: finish the copies here
     if (ok && cudaStreamSynchronize(s0) != cudaSuccess) ok = false;
@@ -609,7 +612,7 @@ nb_status nb_correct_and_timestep(nb_ctx *ctx, int32_t cluster, const int32_t *a
 
 nb_status nb_step(nb_ctx *ctx, double *t_next_out, int32_t *n_active_out) {
     if (!ctx) return fail(nullptr, NB_EINVAL, "nb_step: NULL context");
-    nb_status s = build_graphs(ctx);
+    nb_status s = build_graph(ctx, 0);
     if (s != NB_OK) return s;
     if ((s = set_tend(ctx, INFINITY)) != NB_OK) return s;
     NB_CU(ctx, cudaGraphLaunch(ctx->g_step, ctx->stream));
@@ -641,49 +644,37 @@ nb_status nb_run(nb_ctx *ctx, double t_end, int64_t max_block_steps, int64_t *bl
                  double *interactions_out) {
     if (!ctx) return fail(nullptr, NB_EINVAL, "nb_run: NULL context");
     if (std::isnan(t_end)) return fail(ctx, NB_EINVAL, "nb_run: t_end is NaN");
-    nb_status s = build_graphs(ctx);
+    nb_status s = NB_OK;
+    if (max_block_steps < 0 || max_block_steps >= kMultiSteps) s = build_graph(ctx, 1);
+    if (s == NB_OK && max_block_steps >= 0 && max_block_steps % kMultiSteps) s = build_graph(ctx, 0);
     if (s != NB_OK) return s;
-    unsigned long long steps0 = 0;
-    double inter0 = 0.0;
-    NB_CU(ctx, cudaStreamSynchronize(ctx->stream));
-    NB_CU(ctx, cudaMemcpy(&steps0, ctx->d.ctr_steps, sizeof(steps0), cudaMemcpyDeviceToHost));
-    NB_CU(ctx, cudaMemcpy(&inter0, ctx->d.ctr_inter, sizeof(inter0), cudaMemcpyDeviceToHost));
+    auto read_ctl = [&]() -> cudaError_t {  // the control block as of now, in h_ctl[0]
+        cudaError_t e = cudaMemcpyAsync(ctx->h_ctl, ctx->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->stream);
+        return e != cudaSuccess ? e : cudaStreamSynchronize(ctx->stream);
+    };
+    NB_CU(ctx, read_ctl());
+    const unsigned long long steps0 = ctx->h_ctl->steps;
+    const double inter0 = ctx->h_ctl->inter;
     if ((s = set_tend(ctx, t_end)) != NB_OK) return s;
-    int64_t done_batches = 0;
+    int64_t done = 0;
     while (true) {
-        const int64_t left = max_block_steps < 0 ? INT64_MAX : max_block_steps - done_batches;
+        const int64_t left = max_block_steps < 0 ? INT64_MAX : max_block_steps - done;
         if (left <= 0) break;
         const bool multi = left >= kMultiSteps;
-        if (multi) {
-            NB_CU(ctx, cudaGraphLaunch(ctx->g_multi, ctx->stream));
-            done_batches += kMultiSteps;
-            ctx->launches += (int64_t)kKernelsPerStep * kMultiSteps;
-        } else {
-            NB_CU(ctx, cudaGraphLaunch(ctx->g_step, ctx->stream));
-            NB_CU(ctx, cudaMemcpyAsync(ctx->h_busy, ctx->d.busy, sizeof(int32_t),
-                                       cudaMemcpyDeviceToHost, ctx->stream));
-            done_batches += 1;
-            ctx->launches += kKernelsPerStep;
-        }
-        NB_CU(ctx, cudaStreamSynchronize(ctx->stream));
+        NB_CU(ctx, cudaGraphLaunch(multi ? ctx->g_multi : ctx->g_step, ctx->stream));
+        done += multi ? kMultiSteps : 1;
+        ctx->launches += multi ? (int64_t)kKernelsPerStep * kMultiSteps + 1 : kKernelsPerStep;
+        if (multi) NB_CU(ctx, cudaStreamSynchronize(ctx->stream));
+        else NB_CU(ctx, read_ctl());
         if (multi) harvest_events(ctx, 0, kMultiSteps);
         else harvest_events(ctx, kMultiSteps, 1);
-        if (*ctx->h_busy == 0) break;
         // a device-side failure stops time from advancing: never spin on it
-        if ((s = check_device_error(ctx)) != NB_OK) {
-            set_tend(ctx, INFINITY);
-            return s;
-        }
+        if ((s = error_status(ctx, ctx->h_ctl->err)) != NB_OK) return s;
+        if (ctx->h_ctl->busy == 0) break;
     }
-    if ((s = set_tend(ctx, INFINITY)) != NB_OK) return s;
-    unsigned long long steps1 = 0;
-    double inter1 = 0.0;
-    NB_CU(ctx, cudaStreamSynchronize(ctx->stream));
-    NB_CU(ctx, cudaMemcpy(&steps1, ctx->d.ctr_steps, sizeof(steps1), cudaMemcpyDeviceToHost));
-    NB_CU(ctx, cudaMemcpy(&inter1, ctx->d.ctr_inter, sizeof(inter1), cudaMemcpyDeviceToHost));
-    if (block_steps_out) *block_steps_out = (int64_t)(steps1 - steps0);
-    if (interactions_out) *interactions_out = inter1 - inter0;
-    return check_device_error(ctx);
+    if (block_steps_out) *block_steps_out = (int64_t)(ctx->h_ctl->steps - steps0);
+    if (interactions_out) *interactions_out = ctx->h_ctl->inter - inter0;
+    return error_status(ctx, ctx->h_ctl->err);
 }
 
 nb_status nb_energy(nb_ctx *ctx, int32_t cluster, double t, double *ekin, double *epot, double P[3],

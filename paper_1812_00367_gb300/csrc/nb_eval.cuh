@@ -109,7 +109,7 @@ struct Prec<NB_FP64> {
         const ff mff = ff{self ? 0.f : jj.mf.x, self ? 0.f : jj.mf.y};
         c.pf = ff_add(c.pf, ff_mul_lazy(mff, ff{yh, yl}));
     }
-    // End of a j-tile: the tile's float-pair potential joins the FP64 total.
+    // After 64 pairs: their float-pair potential joins the FP64 total.
     static __device__ __forceinline__ void tile_done(Acc &c) {
         c.p += (double)c.pf.hi + (double)c.pf.lo;
         c.pf = ff{0.f, 0.f};
@@ -1010,8 +1010,11 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
                 if constexpr (P == NB_FP32 || P == NB_FP32X) {
                     if ((tt - tb + 1) % kFp32FlushTiles == 0) T::flush(acc, t64, t64st);
                     else T::tile_done(acc);
-                } else if constexpr (P == NB_EX || P == NB_FP64) {
+                } else if constexpr (P == NB_EX) {
                     T::tile_done(acc);
+                } else if constexpr (P == NB_FP64) {
+                    // every 64 pairs of the lane (four FP64 operations)
+                    if (((int)(tt - tb + 1) & (gl - 1)) == 0) T::tile_done(acc);
                 }
             }
             if (!ok) S.fail = 1;

@@ -58,7 +58,8 @@ constexpr int kTJ = 64;        // j-particles per shared-memory tile
 constexpr int kStages = NB_EVAL_STAGES;  // TMA pipeline depth
 constexpr int kEvalUnroll = NB_EVAL_UNROLL;
 constexpr int kChunk = 2048;   // particles per select / predict chunk
-constexpr int kSelTPB = 256;   // threads per select / predict CTA
+constexpr int kSelTPB = 256;   // threads per select CTA
+constexpr int kPredTPB = 64;   // threads per predict CTA
 constexpr int kPlanTPB = 1024; // threads of the single planning CTA
 constexpr int kBuckets = 32;   // active-set size buckets (floor log2 A)
 constexpr int kFp32FlushTiles = 32;  // FP32 path: j-tiles summed in FP32 before
@@ -234,6 +235,16 @@ struct Dev {
     uint64_t eps_x;
     uint32_t eps_emin;
     FxK fxk;  // {1, 2} as run-time values (nb_fixed.cuh)
+};
+
+// The small values host and device exchange, in one block: the host reads it
+// with one copy.
+struct Ctl {
+    double t_end;       // clusters whose next block time exceeds it stay idle
+    int32_t busy;       // clusters active in the last plan, or whether a step is due
+    uint32_t err;       // device error word
+    unsigned long long steps, underflow;  // counters
+    double inter;
 };
 
 // eps^2 and its float-float pair (host side; every context and launch).
@@ -777,7 +788,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 
 // ------------------------------------------------------------ launchers
 // (implemented in the kernel translation units)
-cudaError_t launch_select_min(const Dev &d, cudaStream_t st);
+cudaError_t launch_select_min(const Dev &d, int look, cudaStream_t st);
 cudaError_t launch_select_compact(const Dev &d, double unused, cudaStream_t st);
 cudaError_t launch_predict(const Dev &d, int also64, int use_fixed_t, double t_fixed,
                            cudaStream_t st);

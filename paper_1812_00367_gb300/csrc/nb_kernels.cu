@@ -40,17 +40,50 @@ struct SumI {
 };
 
 // -------------------------------------------------------------- select pass 1
-__global__ void __launch_bounds__(kSelTPB) k_select_min(const Dev d) {
+// Latency is all there is: a particle's two values are loaded once, all of a
+// thread's side by side, and stay in registers for the count (a loop of single
+// loads over two passes took 8-12 us a launch for any size).
+constexpr int kSelPer = kChunk / kSelTPB;  // particles per thread
+
+__device__ __forceinline__ void load_next_times(const Dev &d, int64_t b, int64_t e, double v[kSelPer]) {
+    double t[kSelPer], dt[kSelPer];
+#pragma unroll
+    for (int u = 0; u < kSelPer; ++u) {
+        const int64_t i = b + threadIdx.x + u * kSelTPB;
+        t[u] = i < e ? d.t[i] : INFINITY;
+        dt[u] = i < e ? d.dt[i] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < kSelPer; ++u) v[u] = t[u] + dt[u];
+}
+
+__global__ void __launch_bounds__(kSelTPB) k_select_min(const Dev d, int look) {
     __shared__ double smd[kSelTPB / 32];
     __shared__ int smi[kSelTPB / 32];
     const int k = blockIdx.x;
     const int64_t b = d.chunk_begin[k], e = d.chunk_end[k];
-    double mn = INFINITY;
-    for (int64_t i = b + threadIdx.x; i < e; i += blockDim.x) mn = fmin(mn, d.t[i] + d.dt[i]);
+    double v[kSelPer];
+    load_next_times(d, b, e, v);
+    double mn = v[0];
+#pragma unroll
+    for (int u = 1; u < kSelPer; ++u) mn = fmin(mn, v[u]);
     mn = block_reduce(mn, MinOp(), smd);
     int cnt = 0;
-    for (int64_t i = b + threadIdx.x; i < e; i += blockDim.x) cnt += (d.t[i] + d.dt[i] == mn);
+#pragma unroll
+    for (int u = 0; u < kSelPer; ++u)
+        cnt += (b + threadIdx.x + u * kSelTPB < e) && v[u] == mn;
     cnt = block_reduce(cnt, SumI(), smi);
+    if (gridDim.x == 1) {  // one chunk, so one cluster: nothing to combine
+        const bool any = mn <= *d.t_end && cnt > 0;
+        if (threadIdx.x == 0) {
+            d.chunk_min[0] = mn;
+            d.chunk_cnt[0] = cnt;
+            d.tnext[0] = mn;
+            d.nact[0] = any ? cnt : 0;
+            if (look) *d.busy = any ? 1 : 0;
+        }
+        return;
+    }
     __shared__ int last;
     if (threadIdx.x == 0) {
         d.chunk_min[k] = mn;
@@ -77,6 +110,7 @@ __global__ void __launch_bounds__(kSelTPB) k_select_min(const Dev d) {
     if (threadIdx.x == 0) n_mid = n_large = 0;
     __syncthreads();
     const double t_end = *d.t_end;
+    int any = 0;  // this thread saw an active cluster
     for (int c = threadIdx.x; c < d.n_clusters; c += blockDim.x) {
         const int k0 = d.cluster_chunk0[c], k1 = d.cluster_chunk0[c + 1];
         if (k1 - k0 > kSelWarp) {
@@ -100,6 +134,7 @@ __global__ void __launch_bounds__(kSelTPB) k_select_min(const Dev d) {
             if (__ldcg(&d.chunk_min[kk]) == tn) total += __ldcg(&d.chunk_cnt[kk]);
         d.tnext[c] = tn;
         d.nact[c] = tn <= t_end ? total : 0;
+        any |= tn <= t_end && total > 0;
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
@@ -118,6 +153,7 @@ __global__ void __launch_bounds__(kSelTPB) k_select_min(const Dev d) {
             d.tnext[c] = tn;
             d.nact[c] = tn <= t_end ? total : 0;
         }
+        any |= tn <= t_end && total > 0;
     }
     const int nl = n_large < kSelLarge ? n_large : kSelLarge;
     for (int q = 0; q < nl; ++q) {
@@ -134,14 +170,18 @@ __global__ void __launch_bounds__(kSelTPB) k_select_min(const Dev d) {
             d.tnext[c] = tn;
             d.nact[c] = tn <= t_end ? total : 0;
         }
+        any |= tn <= t_end && total > 0;
     }
     if (threadIdx.x == 0) *d.sel_ctr = 0u;  // ready for the next pass
+    if (look) {
+        any = __syncthreads_or(any);
+        if (threadIdx.x == 0) *d.busy = any;
+    }
 }
 
 // -------------------------------------------------------------- select pass 2
 __global__ void __launch_bounds__(kSelTPB) k_select_compact(const Dev d) {
     __shared__ int smi[kSelTPB / 32];
-    __shared__ int warp_cnt[kSelTPB / 32];
     const int k = blockIdx.x;
     const int c = d.chunk_cluster[k];
     const int k0 = d.cluster_chunk0[c];
@@ -155,21 +195,33 @@ __global__ void __launch_bounds__(kSelTPB) k_select_compact(const Dev d) {
     const int64_t b = d.chunk_begin[k], e = d.chunk_end[k];
     int32_t *out = d.active + d.offsets[c] + before;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int base = 0;
-    for (int64_t i0 = b; i0 < e; i0 += blockDim.x) {
-        const int64_t i = i0 + threadIdx.x;
-        const bool f = (i < e) && (d.t[i] + d.dt[i] == tn);
-        const unsigned bal = __ballot_sync(0xffffffffu, f);
-        if (lane == 0) warp_cnt[warp] = __popc(bal);
-        __syncthreads();
-        int wbase = base;
-        for (int w = 0; w < warp; ++w) wbase += warp_cnt[w];
-        int round = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) round += warp_cnt[w];
-        if (f) out[wbase + __popc(bal & ((1u << lane) - 1u))] = (int32_t)i;
-        base += round;
-        __syncthreads();
+    double v[kSelPer];
+    load_next_times(d, b, e, v);
+    // active particles of each (round, warp) in index order: round u holds the
+    // particles b + u kSelTPB + thread
+    __shared__ int cnt[kSelPer][kSelTPB / 32];
+    unsigned bal[kSelPer];
+#pragma unroll
+    for (int u = 0; u < kSelPer; ++u) {
+        bal[u] = __ballot_sync(0xffffffffu, (b + threadIdx.x + u * kSelTPB < e) && v[u] == tn);
+        if (lane == 0) cnt[u][warp] = __popc(bal[u]);
     }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int run = 0;
+        for (int q = 0; q < kSelPer * (kSelTPB / 32); ++q) {
+            int &x = cnt[q / (kSelTPB / 32)][q % (kSelTPB / 32)];
+            const int y = x;
+            x = run;
+            run += y;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kSelPer; ++u)
+        if ((bal[u] >> lane) & 1u)
+            out[cnt[u][warp] + __popc(bal[u] & ((1u << lane) - 1u))] =
+                (int32_t)(b + threadIdx.x + u * kSelTPB);
 }
 
 // --------------------------------------------------------------------- plan
@@ -201,6 +253,25 @@ __device__ __forceinline__ double block_sum_d(double v, double *sm) {
     return r;
 }
 
+// One cluster's lanes per i, i-tiles and split (or stream-K ranges); unsplit:
+// the partial sums of its splits do not fit the scratch.
+__device__ __forceinline__ ClusterPlan plan_cluster(const Dev &d, int64_t ncl, int A, bool unsplit,
+                                                    long long &items) {
+    PlanEntry e = d.table[31 - __clz(A)];
+    const long long ntj = cdiv(ncl, kTJ);
+    const bool single = d.n_clusters == 1 && !d.streamk_off;
+    if (single) e.gl = sk_lanes(e.gl, A, ntj, d.grid_eval, d.precision);
+    const long long tiles = cdiv(A, kTPB / e.gl);
+    if (single && sk_use(tiles, kTPB / e.gl, ntj, d.grid_eval, d.partial_cap)) {
+        // one cluster, enough work: stream-K ranges (one "item")
+        items = 1;
+        return ClusterPlan{e.gl, 1, (int)tiles, A, 0, 0, 0, 1, 0};
+    }
+    const long long S = unsplit ? 1 : choose_split(tiles, ntj, e.target_items, d.grid_eval, d.precision);
+    items = tiles * S;
+    return ClusterPlan{e.gl, (int)S, (int)tiles, A, 0, 0, 0, 0, 0};
+}
+
 // One CTA.  Per cluster: A -> bucket floor(log2 A) -> (gl, target items) ->
 // i-tiles and split S (clamped to the cluster's j-tiles); exclusive scans
 // give each cluster its first item and first tile.  If the items that need
@@ -210,6 +281,26 @@ __global__ void __launch_bounds__(kPlanTPB) k_plan(const Dev d, int mode_init, i
     __shared__ long long s_l[kPlanTPB];
     __shared__ double s_d[kPlanTPB];
     const int tid = threadIdx.x;
+    if (d.n_clusters == 1) {  // no scans over clusters
+        if (tid == 0) {
+            const int64_t ncl = d.offsets[1] - d.offsets[0];
+            const int A = mode_init ? (int)ncl : d.nact[0];
+            long long items = 0;
+            ClusterPlan pl{1, 1, 0, 0, 0, 0, 0, 0, 0};
+            if (A > 0) pl = plan_cluster(d, ncl, A, false, items);
+            if (pl.split > 1 && items * 10 * (kTPB / pl.gl) > d.partial_cap)
+                pl = plan_cluster(d, ncl, A, true, items);
+            d.plan[0] = pl;
+            *d.n_items = items;
+            *d.item_ctr = 0ull;
+            *d.busy = A > 0 ? 1 : 0;
+            if (count && !mode_init && A > 0) {
+                *d.ctr_steps += 1ull;
+                *d.ctr_inter += (double)A * (double)(ncl - 1);
+            }
+        }
+        return;
+    }
     for (int fallback = 0; fallback < 2; ++fallback) {
         long long carry_items = 0, carry_tiles = 0, carry_slots = 0;
         double inter = 0.0, busy = 0.0;
@@ -222,22 +313,8 @@ __global__ void __launch_bounds__(kPlanTPB) k_plan(const Dev d, int mode_init, i
                 const int64_t ncl = d.offsets[c + 1] - d.offsets[c];
                 const int A = mode_init ? (int)ncl : d.nact[c];
                 if (A > 0) {
-                    PlanEntry e = d.table[31 - __clz(A)];
-                    const long long ntj = cdiv(ncl, kTJ);
-                    const bool single = d.n_clusters == 1 && !d.streamk_off;
-                    if (single) e.gl = sk_lanes(e.gl, A, ntj, d.grid_eval, d.precision);
-                    tiles = cdiv(A, kTPB / e.gl);
-                    if (single &&
-                        sk_use(tiles, kTPB / e.gl, ntj, d.grid_eval, d.partial_cap)) {
-                        // one cluster, enough work: stream-K ranges (one "item")
-                        items = 1;
-                        pl = ClusterPlan{e.gl, 1, (int)tiles, A, 0, 0, 0, 1, 0};
-                    } else {
-                        const long long S =
-                            fallback ? 1 : choose_split(tiles, ntj, e.target_items, d.grid_eval, d.precision);
-                        items = tiles * S;
-                        pl = ClusterPlan{e.gl, (int)S, (int)tiles, A, 0, 0, 0, 0, 0};
-                    }
+                    pl = plan_cluster(d, ncl, A, fallback != 0, items);
+                    tiles = pl.tiles;
                     my_inter = (double)A * (double)(ncl - 1);
                 }
             }
@@ -285,18 +362,21 @@ __device__ __forceinline__ void split_ff(double x, float &hi, float &lo) {
     lo = __double2float_rn(x - (double)hi);
 }
 
-__global__ void __launch_bounds__(kSelTPB) k_predict(const Dev d, int also64, int use_fixed,
-                                                     double t_fixed) {
-    // kChunk / kSelTPB CTAs per chunk: one particle per thread, all SMs busy
-    constexpr int kSub = kChunk / kSelTPB;
+// One particle per thread in CTAs of two warps: the ~50 FP64 operations of a
+// particle take 16 SM clocks a warp each, so a small system's warps are spread
+// over the SMs (N = 1024: 7.6 -> 5.8 us a launch).
+__global__ void __launch_bounds__(kPredTPB) k_predict(const Dev d, int also64, int use_fixed,
+                                                      double t_fixed) {
+    constexpr int kSub = kChunk / kPredTPB;
     const int k = blockIdx.x / kSub;
     const int c = d.chunk_cluster[k];
     if (!use_fixed && d.nact[c] == 0) return;  // idle cluster this step
     const double tn = use_fixed ? t_fixed : d.tnext[c];
     const int64_t off = d.offsets[c];
     const int64_t jo = d.jofs[c];
-    const int64_t b = d.chunk_begin[k] + (int64_t)(blockIdx.x % kSub) * kSelTPB, e = d.chunk_end[k];
-    for (int64_t i = b + threadIdx.x; i < e && i < b + kSelTPB; i += blockDim.x) {
+    const int64_t b = d.chunk_begin[k] + (int64_t)(blockIdx.x % kSub) * kPredTPB, e = d.chunk_end[k];
+    const int64_t i = b + threadIdx.x;
+    if (i < e) {
         double xp[3], vp[3], ap[3];
         predict_particle(d, i, tn, xp, vp, ap);
         const double m = d.m[i];
@@ -448,8 +528,8 @@ __global__ void __launch_bounds__(kSelTPB) k_unpack64(const Dev d, double *out) 
 }
 
 // ---------------------------------------------------------------- launchers
-cudaError_t launch_select_min(const Dev &d, cudaStream_t st) {
-    k_select_min<<<d.n_chunks, kSelTPB, 0, st>>>(d);
+cudaError_t launch_select_min(const Dev &d, int look, cudaStream_t st) {
+    k_select_min<<<d.n_chunks, kSelTPB, 0, st>>>(d, look);
     return cudaGetLastError();
 }
 cudaError_t launch_select_compact(const Dev &d, double, cudaStream_t st) {
@@ -469,7 +549,7 @@ cudaError_t launch_unpack64(const Dev &d, double *out, cudaStream_t st) {
 }
 cudaError_t launch_predict(const Dev &d, int also64, int use_fixed, double t_fixed,
                            cudaStream_t st) {
-    k_predict<<<d.n_chunks * (kChunk / kSelTPB), kSelTPB, 0, st>>>(d, also64, use_fixed, t_fixed);
+    k_predict<<<d.n_chunks * (kChunk / kPredTPB), kPredTPB, 0, st>>>(d, also64, use_fixed, t_fixed);
     return cudaGetLastError();
 }
 cudaError_t launch_pad(const Dev &d, cudaStream_t st) {
