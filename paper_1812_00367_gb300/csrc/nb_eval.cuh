@@ -48,12 +48,14 @@ struct Prec;
 // the nine running sums stay on the FP64 pipe (12 instructions per pair, 9 in
 // the 4th-order form), everything between them runs on the integer pipes.
 // Bound: the issue of half-rate integer instructions (shifts, logic,
-// IMAD.WIDE; about 680 instructions a pair and warp, 61 % of the ALU pipe and
-// 59 % of the FP64 pipe busy).  Measured, N = 65536 all active: 139.7 ms
-// (3.07e10 pairs/s) against 361.2 ms for the same terms in doubles (50 DFMA a
-// pair, the FP64 pipe 95 % busy); 4th order, N = 30011: 18.4 against 44.8 ms;
-// A = 48: 151 against 324 us.  Residency: 3, 4, 5 or 6 CTAs per SM measured
-// within 1 % of one another.
+// IMAD.WIDE; about 650 instructions a pair and warp; ALU and FP64 pipes both
+// near 60 % busy).  Measured, N = 65536 all active: 133.2 ms (3.22e10 pairs/s)
+// against 361.2 ms for the same terms in doubles (50 DFMA a pair, the FP64
+// pipe 95 % busy); 4th order, N = 30011: 17.3 against 44.8 ms; A = 48: 144
+// against 324 us.  Residency: 3, 4, 5 or 6 CTAs per SM measured within 1 % of
+// one another.  Converting w1, w2 with the count of leading zeros of the high
+// word (a general conversion where a component is that small) instead of a
+// float's exponent: 138.6 -> 133.2 ms.
 template <>
 struct Prec<NB_FP64> {
     using J = JFX;
@@ -164,15 +166,27 @@ struct Prec<NB_FP64> {
         } else {
             const FxS Y2 = fx_split((int64_t)t.y2);
             const FxW1 u = fx_w1(Rs, Vs, V.w, t, Y2, i.K);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) w1[k] = fx_to_double(u.w[k], V.e - 59 + 1023);
+            int64_t x2[3];
+            int base1 = V.e - 59 + 1023, base2 = 0;
+            uint32_t high = min(fx_high(u.w[0]), min(fx_high(u.w[1]), fx_high(u.w[2])));
             if constexpr (kOrder6) {
-                int64_t x2[3];
                 int ez;
                 fx_w2(Rs, R.e, Vs, V.e, A, t, Y2, u, x2, ez, i.K);
-                const int base = min(ez - R.e, 900) - 52 + 1023;
+                base2 = min(ez - R.e, 900) - 52 + 1023;
+                high = min(high, min(fx_high(x2[0]), min(fx_high(x2[1]), fx_high(x2[2]))));
+            }
+            if (high != 0) {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) w2[k] = fx_to_double(x2[k], base);
+                for (int k = 0; k < 3; ++k) {
+                    w1[k] = fx_to_double_high(u.w[k], base1);
+                    if constexpr (kOrder6) w2[k] = fx_to_double_high(x2[k], base2);
+                }
+            } else {  // a component below 2^-30 of its vector's scale (or zero)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    w1[k] = fx_to_double(u.w[k], base1);
+                    if constexpr (kOrder6) w2[k] = fx_to_double(x2[k], base2);
+                }
             }
         }
 #pragma unroll

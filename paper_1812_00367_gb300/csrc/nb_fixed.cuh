@@ -247,9 +247,10 @@ NB_HD Fx3 fx_pack(double x, double y, double z) {
 NB_HD void fx_pack_mass(double m, uint64_t &mm, int &e, uint32_t &sign) {
     const int64_t b = fx_d2bits(m);
     const int ek = (int)((uint64_t)b >> 52) & 0x7ff;
-    sign = (uint32_t)((uint64_t)b >> 32) & 0x80000000u;
+    // a vanishing mass: an exponent below every range, so that q becomes 0
+    sign = ek == 0 ? 0u : (uint32_t)((uint64_t)b >> 32) & 0x80000000u;
     mm = ek == 0 ? 0 : ((((uint64_t)b & 0xfffffffffffffull) | ((uint64_t)1 << 52)) << 10);
-    e = ek == 0x7ff ? 2 * kFxBad : (ek == 0 ? 0 : ek - 1023);
+    e = ek == 0x7ff ? 2 * kFxBad : (ek == 0 ? -2 * kFxBad : ek - 1023);
 }
 
 // ------------------------------------------------------- a pair's vectors
@@ -330,14 +331,30 @@ NB_HD double fx_to_double(int64_t w, int base_biased) {
     hi |= (uint32_t)(s >> 32) & 0x80000000u;
     return fx_bits2d(hi, (uint32_t)m);
 }
+// The same for a w whose magnitude has a bit in the high word (fx_high).
+NB_HD double fx_to_double_high(int64_t w, int base_biased) {
+    const int64_t s = w >> 63;
+    const uint64_t a = (uint64_t)(w ^ s);
+    const int n = fx_clz((uint32_t)(a >> 32));
+    const uint64_t m = (fx_shl(a, n - 1) + 0x200) >> 10;  // leading one at bit 52
+    const uint32_t hi = (uint32_t)(m >> 32) + ((uint32_t)(base_biased + 62 - n) << 20);
+    return fx_bits2d(hi | ((uint32_t)(s >> 32) & 0x80000000u), (uint32_t)m);
+}
+// The high word of the magnitude (one's complement for negative w).
+NB_HD uint32_t fx_high(int64_t w) {
+    const int32_t h = (int32_t)(w >> 32);
+    return (uint32_t)(h ^ (h >> 31));
+}
 // a positive q 2^base as a double; clamped to infinity / zero outside the range
 NB_HD void fx_q_to_double(uint64_t q, int base_biased, uint32_t &hi, uint32_t &lo) {
     const int n = fx_clz((uint32_t)(q >> 32));  // the caller's q has its top bit in the high word
     const uint64_t m = (fx_shl(q, n - 1) + 0x200) >> 10;
     int e = base_biased + 63 - n;
-    e = e < 1 ? 1 : (e > 0x7ff ? 0x7ff : e);
-    hi = (uint32_t)(m >> 32) + ((uint32_t)(e - 1) << 20);
-    lo = (uint32_t)m;
+    e = e < 0 ? 0 : (e > 0x7ff ? 0x7ff : e);
+    // the leading one adds one to the exponent; without it (e = 0) a number
+    // below the normal range remains, which stands for zero
+    hi = e == 0 ? 0u : (uint32_t)(m >> 32) + ((uint32_t)(e - 1) << 20);
+    lo = e == 0 ? 0u : (uint32_t)m;
 }
 
 // The scalar part that every pair term starts with.
@@ -387,11 +404,8 @@ NB_HD double fx_q(const FxRoot &t, uint64_t mm, int em, uint32_t sign, bool zero
     const uint64_t y3 = fx_mulhi_u(t.y, t.y2, K);  // y^3 in units of 2^(-58 - 3 g)
     const uint64_t Q = fx_mulhi_u(mm, y3, K);      // in units of 2^(em - 56 - 3 g)
     uint32_t hi, lo;
-    fx_q_to_double(Q, em - 3 * t.g - 56 + 1023, hi, lo);
-    zero = zero || (Q >> 32) == 0;
-    hi = zero ? 0u : (hi | sign);
-    lo = zero ? 0u : lo;
-    return fx_bits2d(hi, lo);
+    fx_q_to_double(Q, (zero ? -2 * kFxBad : em) - 3 * t.g - 56 + 1023, hi, lo);
+    return fx_bits2d(hi | sign, lo);
 }
 
 // Pair terms up to the jerk: alpha and w1 = v - 3 alpha r.

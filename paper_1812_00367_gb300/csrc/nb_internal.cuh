@@ -334,19 +334,23 @@ __host__ __device__ inline bool sk_use(int64_t tiles, int64_t Ti, int64_t ntj, i
 __host__ __device__ constexpr int sk_min_pairs(int precision) {
     return precision == NB_FP64 ? 0 : precision == NB_EX ? 8 : precision == NB_FP32X ? 32 : 64;
 }
+// Units per CTA that the doubling aims at: with FP64's costly units a finer cut
+// still pays (block steps of N = 16384: 24.04 -> 23.90 ms with 8 instead of 4).
+__host__ __device__ constexpr int64_t sk_lane_units(int precision) {
+    return precision == NB_FP64 ? 2 * kStreamKMinUnits : kStreamKMinUnits;
+}
 __host__ __device__ inline int sk_lanes(int gl, int64_t A, int64_t ntj, int64_t G, int precision) {
     if (A * ntj * kTJ < (int64_t)sk_min_pairs(precision) * G * kTPB) return gl;
-    while (gl < 32 && cdiv(A, kTPB / gl) * ntj < kStreamKMinUnits * G) gl *= 2;
+    while (gl < 32 && cdiv(A, kTPB / gl) * ntj < sk_lane_units(precision) * G) gl *= 2;
     return gl;
 }
 // Most j-ranges a launch is split into: at least kMinTilesPerItem j-tiles
 // each; the FP64 terms, whose pairs cost most, go down to one tile while that
-// makes no more than 64 ranges.  Measured (us, FP64, N = 1024, A = 1): 20 ->
-// 14; N = 4096, A = 2: 21 -> 15; with one tile everywhere N = 65536, A = 2 rose
-// from 29 to 37.
+// makes no more than 128 ranges.  Measured (us, FP64, N = 1024, A = 1): 20 ->
+// 14; N = 16384, A = 4: 24.7 with at most 64 ranges, 22.7 with 128, 29 with 256.
 __host__ __device__ inline int64_t split_max(int64_t ntj, int precision) {
     const int64_t s = ntj / kMinTilesPerItem > 1 ? ntj / kMinTilesPerItem : 1;
-    const int64_t fine = ntj < 64 ? ntj : 64;
+    const int64_t fine = ntj < 128 ? ntj : 128;
     return precision == NB_FP64 && s < fine ? fine : s;
 }
 

@@ -200,6 +200,7 @@ static void check_conversions() {
         const L ref = std::ldexp((L)w, b);
         CHECK(std::fabs((L)got - ref) <= std::ldexp((L)1, b) + std::fabs(ref) * std::ldexp((L)1, -53),
               "fx_to_double(%lld)", (long long)w);
+        CHECK(fx_high(w) == 0 || fx_to_double_high(w, b + 1023) == got, "fx_to_double_high(%lld)", (long long)w);
         CHECK(w < 0 || w >> 53 || (L)got == ref, "fx_to_double(%lld) is not exact", (long long)w);
     }
     CHECK(fx_to_double(0, 1023) == 0.0, "zero");

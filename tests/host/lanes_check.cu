@@ -34,8 +34,8 @@ int main() {
                         const int64_t tiles = cdiv(A, kTPB / gl), U = tiles * ntj;
                         // raised only while the launch has too few units, and then as far as needed
                         if (gl > gl0)
-                            CHECK(cdiv(A, kTPB / (gl / 2)) * ntj < kStreamKMinUnits * G, "raised too far: %d", gl);
-                        if (p == NB_FP64) CHECK(gl == 32 || U >= kStreamKMinUnits * G, "gl %d U %lld", gl, (long long)U);
+                            CHECK(cdiv(A, kTPB / (gl / 2)) * ntj < sk_lane_units(p) * G, "raised too far: %d", gl);
+                        if (p == NB_FP64) CHECK(gl == 32 || U >= sk_lane_units(p) * G, "gl %d U %lld", gl, (long long)U);
                         // never for a share below the arithmetic's least
                         if (A * ntj * kTJ < (int64_t)sk_min_pairs(p) * G * kTPB) CHECK(gl == gl0, "gl %d", gl);
                         // splits: at least one range, each of at least one tile
