@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "nb_internal.cuh"
+#include "nb_sym.cuh"
 
 namespace nb {
 cudaError_t launch_eval_fp64(const Dev &, int, const EvalLaunch &, int, cudaStream_t);
@@ -69,6 +70,9 @@ struct nb_ctx {
     int sm_count = 0;
     int grid_eval = 0, grid_pot = 0;
     int64_t cap_items = 0;
+    SymLaunch sym{};                     // each pair once: whole-cluster evaluations
+    bool sym_force = false, sym_pot = false;
+    int sym_grid[8] = {};                // by evaluation mode
     std::vector<PlanEntry> table;
     PlanEntry *d_table = nullptr;
     cudaGraphExec_t g_step = nullptr;    // one block step
@@ -258,7 +262,8 @@ void plan_direct(const nb_ctx *ctx, int cluster, int32_t n_active, int &gl, int 
     split = (int)S;
 }
 nb_status eval_direct(nb_ctx *ctx, int cluster, const int32_t *active, int32_t n_active, double *out,
-                      int gl, int split, int tiles, int streamk, int32_t jt0 = 0, int32_t jt1 = 0) {
+                      int gl, int split, int tiles, int streamk, int32_t jt0 = 0, int32_t jt1 = 0,
+                      const int *gate = nullptr) {
     EvalLaunch L{};
     L.direct = 1;
     L.cluster = cluster;
@@ -271,10 +276,68 @@ nb_status eval_direct(nb_ctx *ctx, int cluster, const int32_t *active, int32_t n
     L.streamk = streamk;
     L.jt0 = jt0;
     L.jt1 = jt1;
+    L.gate = gate;
     const int64_t items = (int64_t)tiles * split;
     // stream-K ranges were cut for the whole persistent grid
     const int grid = streamk ? ctx->grid_eval : (int)std::min<int64_t>(items, ctx->grid_eval);
     NB_CU(ctx, launch_eval(ctx->d, ctx->d.order == 4 ? kModeOut4 : kModeOut, L, grid, ctx->stream));
+    return NB_OK;
+}
+
+// The whole cluster by itself, each pair once (nb_sym.cu).  active: the
+// caller's list, checked on the device to be every particle in order (*gate is
+// 0 then, and the evaluation that follows with that gate does nothing); NULL:
+// known to be.
+nb_status eval_sym(nb_ctx *ctx, const Dev &d, int mode, const int32_t *active, double *out) {
+    SymLaunch L = ctx->sym;
+    L.out = out;
+    NB_CU(ctx, cudaMemsetAsync(L.gate, 0, 2 * sizeof(int), ctx->stream));
+    if (active) NB_CU(ctx, launch_sym_check(active, ctx->n, 0, L.gate, ctx->stream));
+    NB_CU(ctx, launch_sym(d, mode, L, ctx->sym_grid[mode], ctx->stream));
+    return NB_OK;
+}
+
+// Whether whole-cluster evaluations take each pair once, and their scratch: one
+// cluster of enough particles (N >= 7,800 or so) whose columns' partial sums
+// stay within kSymMaxBytes (N <= 113,000 for the FP64 terms, 357,000 for the
+// potential).  NB_NO_STREAMK keeps the split-item sums everywhere.
+nb_status setup_sym(nb_ctx *ctx) {
+    if (ctx->nc != 1 || (ctx->p.flags & NB_NO_STREAMK)) return NB_OK;
+    SymLaunch &L = ctx->sym;
+    const int64_t ntj = cdiv(ctx->n, kTJ), units = sym_units(ntj);
+    const bool order4 = ctx->d.order == 4;
+    auto usable = [&](int mode) {
+        ctx->sym_grid[mode] = sym_resident(mode) * ctx->sm_count;
+        return ctx->sym_grid[mode] > 0 && units >= kSymMinUnits * ctx->sym_grid[mode];
+    };
+    ctx->sym_force = ctx->p.precision == NB_FP64 && units * kSymUnitBytes <= kSymMaxBytes &&
+                     (order4 ? usable(kModeOut4) && usable(kModeInit4)
+                             : usable(kModeOut) && usable(kModeInit1) && usable(kModeInit2));
+    ctx->sym_pot = units * kSymUnitBytes / 10 <= kSymMaxBytes && usable(kModePot);
+    if (!ctx->sym_force && !ctx->sym_pot) return NB_OK;
+    L.cluster = 0;
+    L.ntj = (int32_t)ntj;
+    L.n = ctx->n;
+    L.units = units;
+    const int64_t grid = 8LL * ctx->sm_count;  // at least any mode's
+    if (dalloc(ctx, &L.jpart, (size_t)(units * kTJ * (ctx->sym_force ? 10 : 1))) != cudaSuccess ||
+        dalloc(ctx, &L.ipart, (size_t)((sym_rows(ntj) + grid) * 10 * kTPB)) != cudaSuccess ||
+        dalloc(ctx, &L.gate, 2) != cudaSuccess) {
+        cudaGetLastError();  // no room: the one-sided evaluation does without
+        ctx->sym_force = ctx->sym_pot = false;
+        return NB_OK;
+    }
+    L.bad = L.gate + 1;
+    return NB_OK;
+}
+
+// The potential of every particle on the FP64 predicted state.
+nb_status eval_potential(nb_ctx *ctx) {
+    if (ctx->sym_pot) return eval_sym(ctx, ctx->d_pot, kModePot, nullptr, nullptr);
+    NB_CU(ctx, launch_plan_ex(ctx->d_pot, 1, 0, ctx->stream));
+    EvalLaunch L{};
+    L.identity = 1;
+    NB_CU(ctx, launch_eval(ctx->d_pot, kModePot, L, ctx->grid_pot, ctx->stream));
     return NB_OK;
 }
 
@@ -285,10 +348,15 @@ nb_status startup(nb_ctx *ctx) {
     const bool order4 = ctx->d.order == 4;
     for (int pass = 0; pass < (order4 ? 1 : 2); ++pass) {
         NB_CU(ctx, launch_predict(ctx->d, 0, 1, 0.0, ctx->stream));
-        NB_CU(ctx, launch_plan_ex(ctx->d, 1, 0, ctx->stream));
         EvalLaunch L{};
         L.identity = 1;
         const int mode = order4 ? kModeInit4 : (pass == 0 ? kModeInit1 : kModeInit2);
+        if (ctx->sym_force) {
+            const nb_status s = eval_sym(ctx, ctx->d, mode, nullptr, nullptr);
+            if (s != NB_OK) return s;
+            continue;
+        }
+        NB_CU(ctx, launch_plan_ex(ctx->d, 1, 0, ctx->stream));
         NB_CU(ctx, launch_eval(ctx->d, mode, L, ctx->grid_eval, ctx->stream));
     }
     return NB_OK;
@@ -502,6 +570,11 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
     ctx->d_pot.precision = NB_FP64;
     ctx->d_pot.grid_eval = ctx->grid_pot;
 
+    if (nb_status ss = setup_sym(ctx); ss != NB_OK) {
+        g_init_err = ctx->err;
+        nb_free(ctx);
+        return ss;
+    }
     default_table(ctx);
     if (p->flags & NB_TIME_EVAL) {
         ctx->ev.resize(2 * (kMultiSteps + 1));
@@ -568,7 +641,13 @@ nb_status nb_evaluate(nb_ctx *ctx, int32_t cluster, const int32_t *active, int32
     if (!active || !out_ajs) return fail(ctx, NB_EINVAL, "nb_evaluate: NULL pointer");
     int gl, split, tiles, streamk;
     plan_direct(ctx, cluster, n_active, gl, split, tiles, streamk);
-    return eval_direct(ctx, cluster, active, n_active, out_ajs, gl, split, tiles, streamk);
+    const int *gate = nullptr;
+    if (ctx->sym_force && n_active == ctx->n) {
+        const nb_status s = eval_sym(ctx, ctx->d, ctx->d.order == 4 ? kModeOut4 : kModeOut, active, out_ajs);
+        if (s != NB_OK) return s;
+        gate = ctx->sym.gate;  // any other list of n entries
+    }
+    return eval_direct(ctx, cluster, active, n_active, out_ajs, gl, split, tiles, streamk, 0, 0, gate);
 }
 
 nb_status nb_evaluate_range(nb_ctx *ctx, int32_t cluster, const int32_t *active, int32_t n_active,
@@ -683,10 +762,7 @@ nb_status nb_energy(nb_ctx *ctx, int32_t cluster, double t, double *ekin, double
     if (cluster < -1 || cluster >= ctx->nc) return fail(ctx, NB_EINVAL, "nb_energy: bad cluster");
     if (!std::isfinite(t)) return fail(ctx, NB_EINVAL, "nb_energy: t not finite");
     NB_CU(ctx, launch_predict(ctx->d, 1, 1, t, ctx->stream));
-    NB_CU(ctx, launch_plan_ex(ctx->d_pot, 1, 0, ctx->stream));
-    EvalLaunch Lz{};
-    Lz.identity = 1;
-    NB_CU(ctx, launch_eval(ctx->d_pot, kModePot, Lz, ctx->grid_pot, ctx->stream));
+    if (nb_status sp = eval_potential(ctx); sp != NB_OK) return sp;
     const int64_t b = cluster < 0 ? 0 : ctx->h_offsets[cluster];
     const int64_t e = cluster < 0 ? ctx->n : ctx->h_offsets[cluster + 1];
     NB_CU(ctx, launch_energy(ctx->d, b, e, 0, ctx->stream));
@@ -708,10 +784,7 @@ nb_status nb_energy_all(nb_ctx *ctx, double t, double *out) {
     if (!ctx) return fail(nullptr, NB_EINVAL, "nb_energy_all: NULL context");
     if (!out || !std::isfinite(t)) return fail(ctx, NB_EINVAL, "nb_energy_all: NULL out or bad t");
     NB_CU(ctx, launch_predict(ctx->d, 1, 1, t, ctx->stream));
-    NB_CU(ctx, launch_plan_ex(ctx->d_pot, 1, 0, ctx->stream));
-    EvalLaunch Lz{};
-    Lz.identity = 1;
-    NB_CU(ctx, launch_eval(ctx->d_pot, kModePot, Lz, ctx->grid_pot, ctx->stream));
+    if (nb_status sp = eval_potential(ctx); sp != NB_OK) return sp;
     NB_CU(ctx, launch_energy(ctx->d, 0, ctx->n, 0, ctx->stream));
     std::vector<double> part((size_t)ctx->d.n_chunks * 8);
     NB_CU(ctx, cudaMemcpyAsync(part.data(), ctx->d.energy_part, part.size() * sizeof(double),

@@ -103,22 +103,26 @@ struct Prec<NB_FP64> {
     // potential term m y in float-float, renormalised every term (|lo| stays
     // below half an ulp of hi): a 64-term tile sum is good to ~2^-45, and
     // tiles add up in FP64
-    static __device__ __forceinline__ void pot_term(const J &jj, bool self, const FxRoot &t, Acc &c) {
+    static __device__ __forceinline__ void pot_term(float2 m, const FxRoot &t, ff &sum) {
         // y = Y 2^(-62 - g) as 24 + 24 bits
         const float s1 = __int_as_float((127 - 23 - t.g) << 23);
         const float yh = __fmul_rn((float)(uint32_t)(t.y >> 39), s1);
         const float yl = __fmul_rn((float)((uint32_t)(t.y >> 15) & 0xffffffu), __fmul_rn(s1, 5.9604644775390625e-08f));
-        const ff mff = ff{self ? 0.f : jj.mf.x, self ? 0.f : jj.mf.y};
-        c.pf = ff_add(c.pf, ff_mul_lazy(mff, ff{yh, yl}));
+        sum = ff_add(sum, ff_mul_lazy(ff{m.x, m.y}, ff{yh, yl}));
     }
     // After 64 pairs: their float-pair potential joins the FP64 total.
     static __device__ __forceinline__ void tile_done(Acc &c) {
         c.p += (double)c.pf.hi + (double)c.pf.lo;
         c.pf = ff{0.f, 0.f};
     }
+    // What a pair's sums are formed from: y, r, w1, w2 (w2 in the 6th-order form).
+    struct Terms {
+        FxRoot t;
+        double r[3], w1[3], w2[3];
+    };
     template <bool kOrder6>
-    static __device__ __forceinline__ void pair(const I &i, const J &jj, bool self, Acc &c) {
-        double r[3];
+    static __device__ __forceinline__ void terms(const I &i, const J &jj, Acc &c, Terms &o) {
+        double (&r)[3] = o.r, (&w1)[3] = o.w1, (&w2)[3] = o.w2;
 #pragma unroll
         for (int k = 0; k < 3; ++k) r[k] = fma_rn_f64(i.x[k], i.m1, jj.x[k]);
         const int evj = jfx_ev(jj);
@@ -130,9 +134,7 @@ struct Prec<NB_FP64> {
             Rs[k] = fx_split(R.w[k]);
             Vs[k] = fx_split(V.w[k]);
         }
-        const FxRoot t = fx_root(Rs, R.e, i.eps_x, i.emin, i.K);
-        pot_term(jj, self, t, c);
-        const double q = fx_q(t, jj.mm, jfx_em(jj), jfx_sign(jj), self, i.K);
+        const FxRoot t = o.t = fx_root(Rs, R.e, i.eps_x, i.emin, i.K);
         c.fv = max(c.fv, evj);
         Fx3 A;
         if constexpr (kOrder6) {
@@ -140,7 +142,6 @@ struct Prec<NB_FP64> {
             c.fa = max(c.fa, eaj);
             A = fx_diff_norm(jj.a, eaj, i.a, i.ea);
         }
-        double w1[3], w2[3];
         if (fx_inside(r, i.emin)) {
             // r below the softening's scale (and the pair i == j): its block
             // would carry too few bits, so alpha, beta, w1 and w2 are formed
@@ -189,11 +190,22 @@ struct Prec<NB_FP64> {
                 }
             }
         }
+    }
+    template <bool kOrder6>
+    static __device__ __forceinline__ void pair(const I &i, const J &jj, bool self, Acc &c) {
+        Terms o;
+        terms<kOrder6>(i, jj, c, o);
+        pot_term(self ? make_float2(0.f, 0.f) : jj.mf, o.t, c.pf);
+        const double q = fx_q(fx_y3(o.t, i.K), o.t.g, jj.mm, jfx_em(jj), jfx_sign(jj), self, i.K);
+        add<kOrder6>(q, o, c);
+    }
+    template <bool kOrder6>
+    static __device__ __forceinline__ void add(double q, const Terms &o, Acc &c) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            c.a[k] = fma(q, r[k], c.a[k]);
-            c.j[k] = fma(q, w1[k], c.j[k]);
-            if constexpr (kOrder6) c.s[k] = fma(q, w2[k], c.s[k]);
+            c.a[k] = fma(q, o.r[k], c.a[k]);
+            c.j[k] = fma(q, o.w1[k], c.j[k]);
+            if constexpr (kOrder6) c.s[k] = fma(q, o.w2[k], c.s[k]);
         }
     }
     static __device__ __forceinline__ void interact(const I &i, const J &jj, bool self, Acc &c) {
@@ -254,14 +266,17 @@ struct Prec<kPrecPot> {
         return r;
     }
     static __device__ __forceinline__ void zero(Acc &c) { c.p = 0.0; }
-    static __device__ __forceinline__ void interact_pot(const I &i, const J &jj, bool self, Acc &c) {
+    static __device__ __forceinline__ double root(const I &i, const J &jj) {
         const double2 q0 = jj.q[0], q1 = jj.q[1];
         const double r[3] = {fma_rn_f64(i.x[0], i.m1, q0.x), fma_rn_f64(i.x[1], i.m1, q0.y),
                              fma_rn_f64(i.x[2], i.m1, q1.x)};
         const Fx3 R = fx_decode(r, i.emin);
         const FxS Rs[3] = {fx_split(R.w[0]), fx_split(R.w[1]), fx_split(R.w[2])};
         const FxRoot t = fx_root(Rs, R.e, i.eps_x, i.emin, i.K);
-        c.p = fma(self ? 0.0 : q1.y, fx_root_to_double(t, R.e), c.p);
+        return fx_root_to_double(t, R.e);
+    }
+    static __device__ __forceinline__ void interact_pot(const I &i, const J &jj, bool self, Acc &c) {
+        c.p = fma(self ? 0.0 : jj.q[1].y, root(i, jj), c.p);
     }
     static __device__ __forceinline__ void finish(const Acc &c, double o[10]) {
 #pragma unroll
@@ -891,6 +906,7 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
     SmemLayout<P> &S = *reinterpret_cast<SmemLayout<P> *>(smem_raw);
     PieceRec &R = S.pc;
     const int tid = threadIdx.x;
+    if (L.gate && *L.gate == 0) return;  // done by the form that takes each pair once
 
     // Work: a stream-K launch (one cluster) gives CTA k the unit range
     // [U k / G, U (k+1) / G) and walks it piece by piece (one piece per i-tile

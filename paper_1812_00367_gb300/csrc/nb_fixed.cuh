@@ -399,12 +399,13 @@ NB_HD double fx_root_to_double(const FxRoot &t, int e) {
     return fx_bits2d(hi, (uint32_t)m);
 }
 
+// y^3 in units of 2^(-58 - 3 g)
+NB_HD uint64_t fx_y3(const FxRoot &t, FxK K) { return fx_mulhi_u(t.y, t.y2, K); }
 // q = |m| y^3, with the sign put back, as a double.
-NB_HD double fx_q(const FxRoot &t, uint64_t mm, int em, uint32_t sign, bool zero, FxK K) {
-    const uint64_t y3 = fx_mulhi_u(t.y, t.y2, K);  // y^3 in units of 2^(-58 - 3 g)
-    const uint64_t Q = fx_mulhi_u(mm, y3, K);      // in units of 2^(em - 56 - 3 g)
+NB_HD double fx_q(uint64_t y3, int g, uint64_t mm, int em, uint32_t sign, bool zero, FxK K) {
+    const uint64_t Q = fx_mulhi_u(mm, y3, K);  // in units of 2^(em - 56 - 3 g)
     uint32_t hi, lo;
-    fx_q_to_double(Q, (zero ? -2 * kFxBad : em) - 3 * t.g - 56 + 1023, hi, lo);
+    fx_q_to_double(Q, (zero ? -2 * kFxBad : em) - 3 * g - 56 + 1023, hi, lo);
     return fx_bits2d(hi | sign, lo);
 }
 

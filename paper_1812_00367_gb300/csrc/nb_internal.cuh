@@ -271,6 +271,7 @@ struct EvalLaunch {
     double *out;        // direct mode output [10][n_active]
     int32_t streamk;    // direct mode: stream-K ranges instead of split items
     int32_t jt0, jt1;   // direct mode: j-tiles [jt0, jt1) of the cluster (jt1 = 0: all)
+    const int *gate;    // run only while *gate != 0 (NULL: always)
 };
 
 // Out/Step/Init1/Init2: 6th-order pair terms (a, jerk, snap); the *4 modes

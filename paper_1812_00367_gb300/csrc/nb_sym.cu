@@ -1,0 +1,320 @@
+// nb_sym.cu -- the evaluation of a whole cluster by itself (every particle
+// active), each pair once.
+//
+// Of a pair's terms only the mass and the sign differ between its two members
+// (r, v, a change sign together; y, alpha, beta do not), so the all-active
+// sums need half the pair terms: i's share is q_j (r, w1, w2), j's is
+// -q_i (r, w1, w2).  Rows are i-tiles of 128 particles (one per thread), columns
+// j-tiles of 64; row I meets the columns from 2 I on.  The first two are the
+// row's own particles and are summed one-sided as in k_eval; in the others lane
+// l of a warp starts at particle l of the tile and walks round it, so that the
+// lanes always hold different j's, and adds j's share into its warp's sums in
+// shared memory.
+//
+// Bound: the FP64 pipe and the issue of integer instructions together (6th
+// order: 21 DFMA a pair for both members, 336 SM clocks a warp, against 2 x 192,
+// and half of the integer work).  Measured, one-sided -> each pair once: N =
+// 65536 6th order 133.2 -> 90.4 ms (98 ms at 2 or 3 CTAs per SM), N = 10007 3.3
+// -> 2.3 ms, 4th order N = 30011 17.3 -> 13.4 ms, potential N = 65536 32.0 ->
+// 20.0 ms (FP64 pipe 85 % busy).  Padding the records against two-fold bank
+// conflicts measured the same.
+//
+// Order of the sums: units (row, column) are cut into equal ranges over a fixed
+// grid (as stream-K); each range leaves one partial per row it touches and each
+// unit one per column particle, in slots of its own; k_sym_reduce adds them in
+// row order.  No atomics: results are reproducible.  A column's partials take
+// 5 KB a unit (1.3 GB at N = 65536), so the form is used up to kSymMaxBytes.
+#include "nb_eval.cuh"
+#include "nb_sym.cuh"
+
+namespace nb {
+namespace {
+
+// values per particle in the partials: sums first, the potential last
+template <int MODE>
+constexpr int sym_nv() {
+    return MODE == kModePot ? 1 : (uses_order4_terms(MODE) ? 7 : 10);
+}
+// place of value v in the ten sums
+template <int MODE>
+__device__ __forceinline__ int sym_q(int v) {
+    return v == sym_nv<MODE>() - 1 ? 9 : v;
+}
+
+template <int P, int MODE>
+struct SymSmem {
+    typename Prec<P>::J tile[kStages][kTJ];
+    double jsum[kTPB / 32][sym_nv<MODE>()][kTJ];  // per warp
+    uint64_t bar[kStages];
+    long long u, u_end;  // next unit, end of the CTA's range
+    long long tb, te;    // columns of the current piece
+    int row, flag, fail;
+};
+
+// Both members' shares of one pair.
+template <int MODE>
+__device__ __forceinline__ void sym_pair(const Prec<NB_FP64>::I &i, const JFX &own, const JFX &jj, bool valid,
+                                         Prec<NB_FP64>::Acc &c, double (*js)[kTJ], int k) {
+    using T = Prec<NB_FP64>;
+    constexpr bool k6 = !uses_order4_terms(MODE);
+    T::Terms o;
+    T::terms<k6>(i, jj, c, o);
+    T::pot_term(jj.mf, o.t, c.pf);
+    const uint64_t y3 = fx_y3(o.t, i.K);
+    T::add<k6>(fx_q(y3, o.t.g, jj.mm, jfx_em(jj), jfx_sign(jj), false, i.K), o, c);
+    // -q_i: the sign bit turned
+    const double nq = fx_q(y3, o.t.g, own.mm, jfx_em(own), jfx_sign(own) ^ 0x80000000u, !valid, i.K);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        js[q][k] = fma(nq, o.r[q], js[q][k]);
+        js[3 + q][k] = fma(nq, o.w1[q], js[3 + q][k]);
+        if constexpr (k6) js[6 + q][k] = fma(nq, o.w2[q], js[6 + q][k]);
+    }
+    double &pj = js[sym_nv<MODE>() - 1][k];  // the float pair of j's potential
+    ff p{__int_as_float(__double2hiint(pj)), __int_as_float(__double2loint(pj))};
+    T::pot_term(valid ? own.mf : make_float2(0.f, 0.f), o.t, p);
+    pj = __hiloint2double(__float_as_int(p.hi), __float_as_int(p.lo));
+}
+__device__ __forceinline__ void sym_pot(const Prec<kPrecPot>::I &i, double mi, const J64 &jj,
+                                        Prec<kPrecPot>::Acc &c, double (*js)[kTJ], int k) {
+    const double y = Prec<kPrecPot>::root(i, jj);
+    c.p = fma(jj.q[1].y, y, c.p);
+    js[0][k] = fma(mi, y, js[0][k]);
+}
+
+template <int P, int MODE>
+__global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L) {
+    using T = Prec<P>;
+    using J = typename T::J;
+    constexpr int NV = sym_nv<MODE>();
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    SymSmem<P, MODE> &S = *reinterpret_cast<SymSmem<P, MODE> *>(smem_raw);
+    if (L.gate && *L.gate != 0) return;  // not the whole cluster in order
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const J *jc = reinterpret_cast<const J *>(d.jarr) + d.jofs[L.cluster];
+    if (tid == 0) {
+        for (int s = 0; s < kStages; ++s) mbar_init(&S.bar[s], 1);
+        S.fail = 0;
+        fence_mbar_init();
+        S.u = sk_begin(L.units, gridDim.x, blockIdx.x);
+        S.u_end = sk_begin(L.units, gridDim.x, blockIdx.x + 1);
+    }
+    uint32_t phase = 0, pending = 0;  // as in k_eval
+    for (;;) {
+        if (tid == 0) {
+            S.row = -1;
+            if (S.u < S.u_end) {
+                const int row = sym_row(S.u, L.ntj);
+                const long long first = sym_first(row, L.ntj);
+                S.row = row;
+                S.tb = 2LL * row + (S.u - first);
+                S.te = min((long long)L.ntj, S.tb + (S.u_end - S.u));
+            }
+        }
+        __syncthreads();
+        if (S.row < 0) break;
+        const int row = S.row;
+        const int64_t tb = S.tb, te = S.te;
+        const int64_t il = (int64_t)row * kTPB + tid;
+        const bool valid = il < L.n;
+        typename T::I me = T::load_i(jc, valid ? il : 0);
+        T::prepare(me, d);
+        const J own = jc[valid ? il : 0];
+        typename T::Acc acc;
+        T::zero(acc);
+        if (tid == 0) {
+            for (int s = 0; s < kStages && tb + s < te; ++s) {
+                mbar_expect_tx(&S.bar[s], kTJ * sizeof(J));
+                tma_load_1d(&S.tile[s][0], jc + (tb + s) * kTJ, kTJ * sizeof(J), &S.bar[s]);
+                pending |= 1u << s;
+            }
+        }
+        bool ok = true;
+        for (int64_t tt = tb; tt < te; ++tt) {
+            const int s = (int)((tt - tb) % kStages);
+            if (ok) ok = mbar_wait_bounded(&S.bar[s], (phase >> s) & 1u);
+            phase ^= 1u << s;
+            const J *tl = &S.tile[s][0];
+            const bool own_cols = tt < 2LL * row + 2;  // uniform over the CTA
+            if (ok && own_cols) {
+                const int js = (int)min(max(il - tt * kTJ, (int64_t)-1), (int64_t)kTJ);
+                tile_pairs<P, MODE, true>(d, me, tl, js, 0, 1, acc);
+            } else if (ok) {
+                double (*js)[kTJ] = S.jsum[warp];
+#pragma unroll
+                for (int q = 0; q < NV; ++q) js[q][lane] = js[q][lane + 32] = 0.0;
+                __syncwarp();
+#pragma unroll 1
+                for (int k0 = 0; k0 < kTJ; ++k0) {
+                    const int k = (lane + k0) & (kTJ - 1);
+                    if constexpr (P == kPrecPot) sym_pot(me, valid ? own.q[1].y : 0.0, tl[k], acc, js, k);
+                    else sym_pair<MODE>(me, own, tl[k], valid, acc, js, k);
+                    __syncwarp();  // the next lane takes this j over
+                }
+            }
+            if constexpr (P == NB_FP64) T::tile_done(acc);
+            if (!ok) S.fail = 1;
+            __syncthreads();
+            if (S.fail) break;
+            if (tid == 0) {
+                pending &= ~(1u << s);
+                if (tt + kStages < te) {
+                    mbar_expect_tx(&S.bar[s], kTJ * sizeof(J));
+                    tma_load_1d(&S.tile[s][0], jc + (tt + kStages) * kTJ, kTJ * sizeof(J), &S.bar[s]);
+                    pending |= 1u << s;
+                }
+            }
+            if (!own_cols) {  // the warps' sums of the tile's particles, in warp order
+                double *out = L.jpart + (S.u + (tt - tb)) * (int64_t)(NV * kTJ);
+                for (int e = tid; e < NV * kTJ; e += kTPB) {
+                    const int q = e / kTJ, k = e % kTJ;
+                    double sum = 0.0;
+#pragma unroll
+                    for (int w = 0; w < kTPB / 32; ++w) {
+                        const double v = S.jsum[w][q][k];
+                        if (P == NB_FP64 && q == NV - 1)
+                            sum += (double)__int_as_float(__double2hiint(v)) + (double)__int_as_float(__double2loint(v));
+                        else
+                            sum += v;
+                    }
+                    out[e] = sum;
+                }
+                __syncthreads();
+            }
+        }
+        if (S.fail) {
+            if (tid == 0) {
+                atomicOr(d.err, kErrTimeout);
+                for (int s = 0; s < kStages; ++s)
+                    if (pending & (1u << s)) (void)mbar_wait_bounded(&S.bar[s], (phase >> s) & 1u);
+            }
+            return;
+        }
+        double o[10];
+        if constexpr (P == NB_FP64) {
+            T::finish(me, acc, o);
+            // a velocity or acceleration that is not finite spoils every other
+            // particle's sums: the reduction is told
+            const int bad = max(acc.fv, me.ev) >= kFxBad ? 3 : (max(acc.fa, me.ea) >= kFxBad ? 2 : 0);
+            if (bad) atomicOr(L.bad, bad);
+        } else {
+            T::finish(acc, o);
+        }
+        double *part = L.ipart + ((int64_t)row + blockIdx.x) * (10 * kTPB) + tid;
+#pragma unroll
+        for (int q = 0; q < 10; ++q) part[q * kTPB] = o[q];
+        __syncthreads();
+        if (tid == 0) S.u += S.te - S.tb;
+    }
+}
+
+// One j-tile's particles: the pieces of their own row, then the shares from the
+// rows above, in row order.
+constexpr int kSymRedTPB = 320;
+template <int P, int MODE>
+__global__ void __launch_bounds__(kSymRedTPB) k_sym_reduce(const Dev d, const SymLaunch L, int grid_sym) {
+    constexpr int NV = sym_nv<MODE>();
+    __shared__ double sums[10][kTJ];
+    if (L.gate && *L.gate != 0) return;
+    const int tile = blockIdx.x, row = tile / 2, il0 = (tile & 1) * kTJ;
+    const long long u0 = sym_first(row, L.ntj), u1 = sym_first(row + 1, L.ntj);
+    const long long k0 = sk_owner(L.units, grid_sym, u0), k1 = sk_owner(L.units, grid_sym, u1 - 1);
+    for (int e = threadIdx.x; e < NV * kTJ; e += kSymRedTPB) {
+        const int v = e / kTJ, k = e % kTJ, q = sym_q<MODE>(v);
+        double sum = 0.0;
+        for (long long c = k0; c <= k1; ++c)
+            sum += __ldcs(L.ipart + (row + c) * (10 * kTPB) + q * kTPB + il0 + k);
+        double above = 0.0;
+        for (int r = 0; r < row; r += 8) {
+            double t[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x)
+                t[x] = r + x < row ? __ldcs(L.jpart + (sym_first(r + x, L.ntj) + (tile - 2LL * (r + x))) *
+                                                          (int64_t)(NV * kTJ) + e)
+                                   : 0.0;
+#pragma unroll
+            for (int x = 0; x < 8; ++x) above += t[x];
+        }
+        // the potential's shares are sums of m y, its sum carries the sign
+        sums[q][k] = q == 9 ? sum - above : sum + above;
+    }
+    __syncthreads();
+    const int64_t il = (int64_t)tile * kTJ + threadIdx.x;
+    if (threadIdx.x < kTJ && il < L.n) {
+        double o[10];
+        const double nan = __hiloint2double(0x7ff80000, 0);
+        const int bad = P == NB_FP64 ? *L.bad : 0;
+#pragma unroll
+        for (int q = 0; q < 10; ++q) {
+            const bool here = MODE == kModePot ? q == 9 : (!uses_order4_terms(MODE) || q < 6 || q == 9);
+            o[q] = here ? sums[q][threadIdx.x] : 0.0;
+        }
+        if constexpr (P == NB_FP64) {
+            const bool bad_x = !(isfinite(o[0]) && isfinite(o[1]) && isfinite(o[2]));
+#pragma unroll
+            for (int q = 0; q < 10; ++q)
+                if (bad_x || (q >= 3 && q < 6 && (bad & 1)) || (q >= 6 && q < 9 && bad)) o[q] = nan;
+        }
+        EvalLaunch E{};
+        E.out = L.out;
+        E.n_active = (int32_t)L.n;
+        finalize_one<P, MODE>(d, E, L.cluster, d.offsets[L.cluster] + il, (int)il, o);
+    }
+}
+
+// Whether active is off, off + 1, ..., off + n - 1 (gate stays 0).
+__global__ void k_sym_check(const int32_t *active, int64_t n, int64_t off, int *gate) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < n && active[i] != off + i) atomicOr(gate, 1);
+}
+
+template <int P, int MODE>
+cudaError_t go(const Dev &d, const SymLaunch &L, int grid, cudaStream_t st) {
+    constexpr size_t smem = sizeof(SymSmem<P, MODE>);
+    k_sym<P, MODE><<<grid, kTPB, smem, st>>>(d, L);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_sym_reduce<P, MODE><<<L.ntj, kSymRedTPB, 0, st>>>(d, L, grid);
+    return cudaGetLastError();
+}
+template <int P, int MODE>
+int resident() {  // CTAs per SM, after raising the shared-memory limit
+    constexpr int smem = (int)sizeof(SymSmem<P, MODE>);
+    int b = 0;
+    if (cudaFuncSetAttribute(k_sym<P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sym<P, MODE>, kTPB, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return b;
+}
+}  // namespace
+
+cudaError_t launch_sym_check(const int32_t *active, int64_t n, int64_t off, int *gate, cudaStream_t st) {
+    k_sym_check<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(active, n, off, gate);
+    return cudaGetLastError();
+}
+cudaError_t launch_sym(const Dev &d, int mode, const SymLaunch &L, int grid, cudaStream_t st) {
+    switch (mode) {
+    case kModeOut: return go<NB_FP64, kModeOut>(d, L, grid, st);
+    case kModeOut4: return go<NB_FP64, kModeOut4>(d, L, grid, st);
+    case kModeInit1: return go<NB_FP64, kModeInit1>(d, L, grid, st);
+    case kModeInit2: return go<NB_FP64, kModeInit2>(d, L, grid, st);
+    case kModeInit4: return go<NB_FP64, kModeInit4>(d, L, grid, st);
+    case kModePot: return go<kPrecPot, kModePot>(d, L, grid, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+int sym_resident(int mode) {
+    switch (mode) {
+    case kModeOut: return resident<NB_FP64, kModeOut>();
+    case kModeOut4: return resident<NB_FP64, kModeOut4>();
+    case kModeInit1: return resident<NB_FP64, kModeInit1>();
+    case kModeInit2: return resident<NB_FP64, kModeInit2>();
+    case kModeInit4: return resident<NB_FP64, kModeInit4>();
+    case kModePot: return resident<kPrecPot, kModePot>();
+    default: return 0;
+    }
+}
+
+}  // namespace nb

@@ -83,7 +83,7 @@ static Term fixed(const Pair &p) {
         Vs[k] = fx_split(V.w[k]);
     }
     const FxRoot t = fx_root(Rs, R.e, eps_x, emin, K);
-    const double q = fx_q(t, mm, em, sign, false, K);
+    const double q = fx_q(fx_y3(t, K), t.g, mm, em, sign, false, K);
     double w1[3], w2[3];
     if (fx_inside(r, emin)) {
         double v[3], a[3];
@@ -232,22 +232,23 @@ static void check_conversions() {
     uint32_t sg;
     int e;
     fx_pack_mass(0.0, mm, e, sg);
-    CHECK(fx_q(t, mm, e, sg, false, K) == 0.0, "massless");
+    CHECK(fx_q(fx_y3(t, K), t.g, mm, e, sg, false, K) == 0.0, "massless");
     fx_pack_mass(1.0, mm, e, sg);
-    CHECK(fx_q(t, mm, e, sg, true, K) == 0.0, "excluded");
-    CHECK(fx_q(t, mm, e, sg, false, K) > 0.0, "mass 1");
+    CHECK(fx_q(fx_y3(t, K), t.g, mm, e, sg, true, K) == 0.0, "excluded");
+    CHECK(fx_q(fx_y3(t, K), t.g, mm, e, sg, false, K) > 0.0, "mass 1");
     fx_pack_mass(-1.0, mm, e, sg);
-    CHECK(fx_q(t, mm, e, sg, false, K) < 0.0, "mass -1");
+    CHECK(fx_q(fx_y3(t, K), t.g, mm, e, sg, false, K) < 0.0, "mass -1");
     for (double bad : {inf, nan}) {
         fx_pack_mass(bad, mm, e, sg);
-        CHECK(!std::isfinite(fx_q(t, mm, e, sg, false, K)), "mass %g", bad);
+        CHECK(!std::isfinite(fx_q(fx_y3(t, K), t.g, mm, e, sg, false, K)), "mass %g", bad);
     }
     // coincident particles without softening: no finite q
     const double zero[3] = {0, 0, 0};
     const Fx3 Z = fx_decode(zero, 0);
     const FxS Zs[3] = {fx_split(Z.w[0]), fx_split(Z.w[1]), fx_split(Z.w[2])};
     fx_pack_mass(1.0, mm, e, sg);
-    CHECK(!std::isfinite(fx_q(fx_root(Zs, Z.e, 0, 0, K), mm, e, sg, false, K)), "r = 0, eps = 0");
+    const FxRoot z0 = fx_root(Zs, Z.e, 0, 0, K);
+    CHECK(!std::isfinite(fx_q(fx_y3(z0, K), z0.g, mm, e, sg, false, K)), "r = 0, eps = 0");
 }
 
 int main() {
