@@ -299,18 +299,18 @@ nb_status eval_sym(nb_ctx *ctx, const Dev &d, int mode, const int32_t *active, d
 
 // Whether whole-cluster evaluations take each pair once, and their scratch: one
 // cluster of enough particles (N >= 7,800 or so) whose columns' partial sums
-// stay within kSymMaxBytes (N <= 113,000 for the FP64 terms, 357,000 for the
-// potential).  NB_NO_STREAMK keeps the split-item sums everywhere.
+// stay within kSymMaxBytes (N <= 113,000 for the pair terms of FP64 and EX,
+// 357,000 for the potential).  NB_NO_STREAMK keeps the split-item sums everywhere.
 nb_status setup_sym(nb_ctx *ctx) {
     if (ctx->nc != 1 || (ctx->p.flags & NB_NO_STREAMK)) return NB_OK;
     SymLaunch &L = ctx->sym;
     const int64_t ntj = cdiv(ctx->n, kTJ), units = sym_units(ntj);
     const bool order4 = ctx->d.order == 4;
     auto usable = [&](int mode) {
-        ctx->sym_grid[mode] = sym_resident(mode) * ctx->sm_count;
+        ctx->sym_grid[mode] = sym_resident(ctx->p.precision, mode) * ctx->sm_count;
         return ctx->sym_grid[mode] > 0 && units >= kSymMinUnits * ctx->sym_grid[mode];
     };
-    ctx->sym_force = ctx->p.precision == NB_FP64 && units * kSymUnitBytes <= kSymMaxBytes &&
+    ctx->sym_force = (ctx->p.precision == NB_FP64 || ctx->p.precision == NB_EX) && units * kSymUnitBytes <= kSymMaxBytes &&
                      (order4 ? usable(kModeOut4) && usable(kModeInit4)
                              : usable(kModeOut) && usable(kModeInit1) && usable(kModeInit2));
     ctx->sym_pot = units * kSymUnitBytes / 10 <= kSymMaxBytes && usable(kModePot);

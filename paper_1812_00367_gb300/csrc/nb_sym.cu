@@ -4,7 +4,8 @@
 // Of a pair's terms only the mass and the sign differ between its two members
 // (r, v, a change sign together; y, alpha, beta do not), so the all-active
 // sums need half the pair terms: i's share is q_j (r, w1, w2), j's is
-// -q_i (r, w1, w2).  Rows are i-tiles of 128 particles (one per thread), columns
+// -q_i (r, w1, w2).  For the FP64 and EX terms (the sums of the FP32 ones keep
+// their order of additions) and the potential.  Rows are i-tiles of 128 particles (one per thread), columns
 // j-tiles of 64; row I meets the columns from 2 I on.  The first two are the
 // row's own particles and are summed one-sided as in k_eval; in the others lane
 // l of a warp starts at particle l of the tile and walks round it, so that the
@@ -16,7 +17,9 @@
 // and half of the integer work).  Measured, one-sided -> each pair once: N =
 // 65536 6th order 133.2 -> 90.4 ms (98 ms at 2 or 3 CTAs per SM), N = 10007 3.3
 // -> 2.3 ms, 4th order N = 30011 17.3 -> 13.4 ms, potential N = 65536 32.0 ->
-// 20.0 ms (FP64 pipe 85 % busy).  Padding the records against two-fold bank
+// 20.0 ms (FP64 pipe 85 % busy); EX, bound by its packed FP32 operations (about
+// 620 a pair for both members instead of 2 x 500), N = 65536 62.5 -> 42.9 ms, 4th
+// order N = 30011 7.7 -> 5.6 ms.  Padding the records against two-fold bank
 // conflicts measured the same.
 //
 // Order of the sums: units (row, column) are cut into equal ranges over a fixed
@@ -43,8 +46,11 @@ __device__ __forceinline__ int sym_q(int v) {
 
 template <int P, int MODE>
 struct SymSmem {
-    typename Prec<P>::J tile[kStages][kTJ];
-    double jsum[kTPB / 32][sym_nv<MODE>()][kTJ];  // per warp
+    typename Prec<P>::J tile[kStages][kTJ / Prec<P>::kPerRec];
+    // per warp: the sums of the tile's particles, one double each (FP64: the
+    // potential as a float pair in its bits), EX: hi and lo of a record's two
+    // particles in the room of two doubles
+    alignas(16) double jsum[kTPB / 32][sym_nv<MODE>()][kTJ];
     uint64_t bar[kStages];
     long long u, u_end;  // next unit, end of the CTA's range
     long long tb, te;    // columns of the current piece
@@ -75,6 +81,57 @@ __device__ __forceinline__ void sym_pair(const Prec<NB_FP64>::I &i, const JFX &o
     T::pot_term(valid ? own.mf : make_float2(0.f, 0.f), o.t, p);
     pj = __hiloint2double(__float_as_int(p.hi), __float_as_int(p.lo));
 }
+// EX: one record, two pairs.
+__device__ __forceinline__ void sym_add_ex(float4 *sum, ff2 a, ff2 b) {
+    float4 v = *sum;  // (hi, hi, lo, lo) of the record's two particles
+    ff2 acc{lo2(v), hi2(v)};
+    ff_fma_acc_lazy(acc, a, b);
+    *sum = make_float4(acc.hi.x, acc.hi.y, acc.lo.x, acc.lo.y);
+}
+template <int MODE>
+__device__ __forceinline__ void sym_pair(const Prec<NB_EX>::I &i, ff2 nmi, const JEXP &jj, ff2 eps2,
+                                         Prec<NB_EX>::Acc &c, float4 (*js)[kTJ / 2], int k) {
+    using T = Prec<NB_EX>;
+    constexpr bool k6 = !uses_order4_terms(MODE);
+    ff2 r[3], v[3], a[3];
+    T::rel(i, jj, r, v);
+    const ff2 m{hi2(jj.q[1]), hi2(jj.q[3])};
+    const ff2 y = rsqrt_ff(k6 ? ff_dot3_add_lazy(r, r, eps2) : ff_dot3_add(r, r, eps2));
+    const ff2 y2 = ff_sqr_lazy(y);
+    const ff2 my = ff_mul_lazy(m, y), myi = ff_mul_lazy(nmi, y);  // m_j y, -m_i y
+    ff_add_lazy(c.p, my);
+    {
+        float4 &p = js[sym_nv<MODE>() - 1][k];
+        ff2 acc{lo2(p), hi2(p)};
+        ff_add_lazy(acc, myi);
+        p = make_float4(acc.hi.x, acc.hi.y, acc.lo.x, acc.lo.y);
+    }
+    const ff2 q = ff_mul_lazy(my, y2), nq = ff_mul_lazy(myi, y2);
+    const ff2 al = ff_mul_lazy(k6 ? ff_dot3_lazy(r, v) : ff_dot3(r, v), y2);
+    const ff2 al3 = ff_mul_f_lazy(al, f2s(3.0f));
+    ff2 be3, al6;
+    if constexpr (k6) {
+        a[0] = ff_sub(ff2{hi2(jj.q[5]), hi2(jj.q[7])}, i.a[0]);
+        a[1] = ff_sub(ff2{lo2(jj.q[8]), lo2(jj.q[9])}, i.a[1]);
+        a[2] = ff_sub(ff2{hi2(jj.q[8]), hi2(jj.q[9])}, i.a[2]);
+        const ff2 ze = ff_mul_lazy(ff_dot3x2_lazy(v, v, r, a), y2);
+        be3 = ff_mul_f_lazy(ff_sum_lazy(ff_sqr_lazy(al), ze), f2s(3.0f));
+        al6 = ff2{add2(al3.hi, al3.hi), add2(al3.lo, al3.lo)};  // exact
+    }
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        const ff2 w1 = ff_fnma_lazy(al3, r[t], v[t]);
+        ff_fma_acc_lazy(c.a[t], q, r[t]);
+        sym_add_ex(&js[t][k], nq, r[t]);
+        ff_fma_acc_lazy(c.j[t], q, w1);
+        sym_add_ex(&js[3 + t][k], nq, w1);
+        if constexpr (k6) {
+            const ff2 w2 = ff_fnma_lazy(be3, r[t], ff_fnma_lazy(al6, w1, a[t]));
+            ff_fma_acc_lazy(c.s[t], q, w2);
+            sym_add_ex(&js[6 + t][k], nq, w2);
+        }
+    }
+}
 __device__ __forceinline__ void sym_pot(const Prec<kPrecPot>::I &i, double mi, const J64 &jj,
                                         Prec<kPrecPot>::Acc &c, double (*js)[kTJ], int k) {
     const double y = Prec<kPrecPot>::root(i, jj);
@@ -87,11 +144,12 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
     using T = Prec<P>;
     using J = typename T::J;
     constexpr int NV = sym_nv<MODE>();
+    constexpr int kRecs = kTJ / T::kPerRec;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     SymSmem<P, MODE> &S = *reinterpret_cast<SymSmem<P, MODE> *>(smem_raw);
     if (L.gate && *L.gate != 0) return;  // not the whole cluster in order
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const J *jc = reinterpret_cast<const J *>(d.jarr) + d.jofs[L.cluster];
+    const J *jc = reinterpret_cast<const J *>(d.jarr) + d.jofs[L.cluster] / T::kPerRec;
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) mbar_init(&S.bar[s], 1);
         S.fail = 0;
@@ -118,14 +176,19 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
         const int64_t il = (int64_t)row * kTPB + tid;
         const bool valid = il < L.n;
         typename T::I me = T::load_i(jc, valid ? il : 0);
-        T::prepare(me, d);
-        const J own = jc[valid ? il : 0];
+        if constexpr (P != NB_EX) T::prepare(me, d);
+        const J own = jc[(valid ? il : 0) / T::kPerRec];
+        ff2 nmi{f2s(0.f), f2s(0.f)};  // EX: -m_i
+        if constexpr (P == NB_EX) {
+            const float *f = reinterpret_cast<const float *>(&own) + (il & 1);
+            if (valid) nmi = ff2{f2s(-f[2 * 3]), f2s(-f[2 * 7])};
+        }
         typename T::Acc acc;
         T::zero(acc);
         if (tid == 0) {
             for (int s = 0; s < kStages && tb + s < te; ++s) {
-                mbar_expect_tx(&S.bar[s], kTJ * sizeof(J));
-                tma_load_1d(&S.tile[s][0], jc + (tb + s) * kTJ, kTJ * sizeof(J), &S.bar[s]);
+                mbar_expect_tx(&S.bar[s], kRecs * sizeof(J));
+                tma_load_1d(&S.tile[s][0], jc + (tb + s) * kRecs, kRecs * sizeof(J), &S.bar[s]);
                 pending |= 1u << s;
             }
         }
@@ -145,22 +208,25 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
                 for (int q = 0; q < NV; ++q) js[q][lane] = js[q][lane + 32] = 0.0;
                 __syncwarp();
 #pragma unroll 1
-                for (int k0 = 0; k0 < kTJ; ++k0) {
-                    const int k = (lane + k0) & (kTJ - 1);
-                    if constexpr (P == kPrecPot) sym_pot(me, valid ? own.q[1].y : 0.0, tl[k], acc, js, k);
+                for (int k0 = 0; k0 < kRecs; ++k0) {
+                    const int k = (lane + k0) & (kRecs - 1);
+                    if constexpr (P == NB_EX)
+                        sym_pair<MODE>(me, nmi, tl[k], ff2{d.eps2_hi2, d.eps2_lo2}, acc,
+                                       reinterpret_cast<float4(*)[kTJ / 2]>(js), k);
+                    else if constexpr (P == kPrecPot) sym_pot(me, valid ? own.q[1].y : 0.0, tl[k], acc, js, k);
                     else sym_pair<MODE>(me, own, tl[k], valid, acc, js, k);
                     __syncwarp();  // the next lane takes this j over
                 }
             }
-            if constexpr (P == NB_FP64) T::tile_done(acc);
+            if constexpr (P != kPrecPot) T::tile_done(acc);
             if (!ok) S.fail = 1;
             __syncthreads();
             if (S.fail) break;
             if (tid == 0) {
                 pending &= ~(1u << s);
                 if (tt + kStages < te) {
-                    mbar_expect_tx(&S.bar[s], kTJ * sizeof(J));
-                    tma_load_1d(&S.tile[s][0], jc + (tt + kStages) * kTJ, kTJ * sizeof(J), &S.bar[s]);
+                    mbar_expect_tx(&S.bar[s], kRecs * sizeof(J));
+                    tma_load_1d(&S.tile[s][0], jc + (tt + kStages) * kRecs, kRecs * sizeof(J), &S.bar[s]);
                     pending |= 1u << s;
                 }
             }
@@ -171,6 +237,11 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
                     double sum = 0.0;
 #pragma unroll
                     for (int w = 0; w < kTPB / 32; ++w) {
+                        if constexpr (P == NB_EX) {
+                            const float *f = reinterpret_cast<const float *>(&S.jsum[w][q][0]) + 4 * (k >> 1) + (k & 1);
+                            sum += (double)f[0] + (double)f[2];
+                            continue;
+                        }
                         const double v = S.jsum[w][q][k];
                         if (P == NB_FP64 && q == NV - 1)
                             sum += (double)__int_as_float(__double2hiint(v)) + (double)__int_as_float(__double2loint(v));
@@ -197,6 +268,8 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
             // particle's sums: the reduction is told
             const int bad = max(acc.fv, me.ev) >= kFxBad ? 3 : (max(acc.fa, me.ea) >= kFxBad ? 2 : 0);
             if (bad) atomicOr(L.bad, bad);
+        } else if constexpr (P == NB_EX) {
+            T::finish(acc, nullptr, 0, o);
         } else {
             T::finish(acc, o);
         }
@@ -235,8 +308,8 @@ __global__ void __launch_bounds__(kSymRedTPB) k_sym_reduce(const Dev d, const Sy
 #pragma unroll
             for (int x = 0; x < 8; ++x) above += t[x];
         }
-        // the potential's shares are sums of m y, its sum carries the sign
-        sums[q][k] = q == 9 ? sum - above : sum + above;
+        // FP64's shares of the potential are sums of m y, its sum carries the sign
+        sums[q][k] = q == 9 && P != NB_EX ? sum - above : sum + above;
     }
     __syncthreads();
     const int64_t il = (int64_t)tile * kTJ + threadIdx.x;
@@ -295,24 +368,27 @@ cudaError_t launch_sym_check(const int32_t *active, int64_t n, int64_t off, int 
     return cudaGetLastError();
 }
 cudaError_t launch_sym(const Dev &d, int mode, const SymLaunch &L, int grid, cudaStream_t st) {
+    const bool ex = d.precision == NB_EX;
     switch (mode) {
-    case kModeOut: return go<NB_FP64, kModeOut>(d, L, grid, st);
-    case kModeOut4: return go<NB_FP64, kModeOut4>(d, L, grid, st);
-    case kModeInit1: return go<NB_FP64, kModeInit1>(d, L, grid, st);
-    case kModeInit2: return go<NB_FP64, kModeInit2>(d, L, grid, st);
-    case kModeInit4: return go<NB_FP64, kModeInit4>(d, L, grid, st);
+    case kModeOut: return ex ? go<NB_EX, kModeOut>(d, L, grid, st) : go<NB_FP64, kModeOut>(d, L, grid, st);
+    case kModeOut4: return ex ? go<NB_EX, kModeOut4>(d, L, grid, st) : go<NB_FP64, kModeOut4>(d, L, grid, st);
+    case kModeInit1: return ex ? go<NB_EX, kModeInit1>(d, L, grid, st) : go<NB_FP64, kModeInit1>(d, L, grid, st);
+    case kModeInit2: return ex ? go<NB_EX, kModeInit2>(d, L, grid, st) : go<NB_FP64, kModeInit2>(d, L, grid, st);
+    case kModeInit4: return ex ? go<NB_EX, kModeInit4>(d, L, grid, st) : go<NB_FP64, kModeInit4>(d, L, grid, st);
     case kModePot: return go<kPrecPot, kModePot>(d, L, grid, st);
     default: return cudaErrorInvalidValue;
     }
 }
-int sym_resident(int mode) {
+int sym_resident(int precision, int mode) {
+    if (mode == kModePot) return resident<kPrecPot, kModePot>();
+    if (precision != NB_FP64 && precision != NB_EX) return 0;
+    const bool ex = precision == NB_EX;
     switch (mode) {
-    case kModeOut: return resident<NB_FP64, kModeOut>();
-    case kModeOut4: return resident<NB_FP64, kModeOut4>();
-    case kModeInit1: return resident<NB_FP64, kModeInit1>();
-    case kModeInit2: return resident<NB_FP64, kModeInit2>();
-    case kModeInit4: return resident<NB_FP64, kModeInit4>();
-    case kModePot: return resident<kPrecPot, kModePot>();
+    case kModeOut: return ex ? resident<NB_EX, kModeOut>() : resident<NB_FP64, kModeOut>();
+    case kModeOut4: return ex ? resident<NB_EX, kModeOut4>() : resident<NB_FP64, kModeOut4>();
+    case kModeInit1: return ex ? resident<NB_EX, kModeInit1>() : resident<NB_FP64, kModeInit1>();
+    case kModeInit2: return ex ? resident<NB_EX, kModeInit2>() : resident<NB_FP64, kModeInit2>();
+    case kModeInit4: return ex ? resident<NB_EX, kModeInit4>() : resident<NB_FP64, kModeInit4>();
     default: return 0;
     }
 }

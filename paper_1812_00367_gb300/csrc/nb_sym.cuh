@@ -40,6 +40,6 @@ struct SymLaunch {
 
 cudaError_t launch_sym_check(const int32_t *active, int64_t n, int64_t off, int *gate, cudaStream_t st);
 cudaError_t launch_sym(const Dev &d, int mode, const SymLaunch &L, int grid, cudaStream_t st);
-int sym_resident(int mode);  // CTAs per SM (0: not available)
+int sym_resident(int precision, int mode);  // CTAs per SM (0: not available)
 
 }  // namespace nb
