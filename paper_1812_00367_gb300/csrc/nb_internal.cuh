@@ -325,22 +325,22 @@ __host__ __device__ inline bool sk_use(int64_t tiles, int64_t Ti, int64_t ntj, i
 }
 
 // Lanes per i of a single cluster's launch: the table's choice for the
-// active-set size, doubled while the launch has fewer units than stream-K
-// wants (few active particles, or a small cluster) and an even share still
-// gives every lane of the grid kLanesMinPairs pairs: below that the epilogue
-// of the extra pieces costs more than the idle SMs.  The share a lane needs
-// falls with the cost of a pair.  Measured (us, one evaluation, table's lanes
-// -> these): N = A = 1024 FP64 128 -> 59, EX 59 -> 47; N = A = 256 FP64 64 -> 15;
-// FP32, N = A = 1024, 21 -> 37 if its lanes were doubled too.
-__host__ __device__ constexpr int sk_min_pairs(int precision) {
-    return precision == NB_FP64 ? 0 : precision == NB_EX ? 8 : precision == NB_FP32X ? 32 : 64;
-}
+// active-set size, doubled (FP64, EX) while the launch has fewer units than
+// stream-K wants (few active particles, or a small cluster).  EX pairs cost
+// less: it doubles only where an even share still gives every lane of the grid
+// eight pairs; below that the epilogue of the extra pieces costs more than the
+// idle SMs.  FP32 and FP32X keep the table's lanes: the order of their single
+// precision sums, and with it their rounding, follows the lanes.  Measured (us,
+// one evaluation, table's lanes -> these): N = A = 1024 FP64 128 -> 59, EX 59 ->
+// 47; N = A = 256 FP64 64 -> 15.
+__host__ __device__ constexpr int sk_min_pairs(int precision) { return precision == NB_FP64 ? 0 : 8; }
 // Units per CTA that the doubling aims at: with FP64's costly units a finer cut
 // still pays (block steps of N = 16384: 24.04 -> 23.90 ms with 8 instead of 4).
 __host__ __device__ constexpr int64_t sk_lane_units(int precision) {
     return precision == NB_FP64 ? 2 * kStreamKMinUnits : kStreamKMinUnits;
 }
 __host__ __device__ inline int sk_lanes(int gl, int64_t A, int64_t ntj, int64_t G, int precision) {
+    if (precision != NB_FP64 && precision != NB_EX) return gl;
     if (A * ntj * kTJ < (int64_t)sk_min_pairs(precision) * G * kTPB) return gl;
     while (gl < 32 && cdiv(A, kTPB / gl) * ntj < sk_lane_units(precision) * G) gl *= 2;
     return gl;

@@ -36,6 +36,8 @@ int main() {
                         if (gl > gl0)
                             CHECK(cdiv(A, kTPB / (gl / 2)) * ntj < sk_lane_units(p) * G, "raised too far: %d", gl);
                         if (p == NB_FP64) CHECK(gl == 32 || U >= sk_lane_units(p) * G, "gl %d U %lld", gl, (long long)U);
+                        // single-precision sums keep the table's lanes
+                        if (p == NB_FP32 || p == NB_FP32X) CHECK(gl == gl0, "gl %d", gl);
                         // never for a share below the arithmetic's least
                         if (A * ntj * kTJ < (int64_t)sk_min_pairs(p) * G * kTPB) CHECK(gl == gl0, "gl %d", gl);
                         // splits: at least one range, each of at least one tile
