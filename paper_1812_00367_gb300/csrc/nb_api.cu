@@ -548,6 +548,8 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
     ALLOC(d.partial, ctx->cap_items * 10 * kTPB);
     const int64_t max_tiles = n + n_clusters + 1;
     ALLOC(d.tile_cnt, max_tiles);
+    const int64_t max_groups = d.partial_cap / kGrpStride + 1;
+    ALLOC(d.grp_cnt, max_groups);
     ALLOC(ctx->d_ctl, 1);
     d.ctr_steps = &ctx->d_ctl->steps;
     d.ctr_inter = &ctx->d_ctl->inter;
@@ -599,6 +601,7 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
     up(d_cc0, cluster_chunk0.data(), cluster_chunk0.size() * sizeof(int32_t));
     up(ctx->d_table, ctx->table.data(), kBuckets * sizeof(PlanEntry));
     if (ok && cudaMemsetAsync(d.tile_cnt, 0, max_tiles * sizeof(int32_t), s0) != cudaSuccess) ok = false;
+    if (ok && cudaMemsetAsync(d.grp_cnt, 0, max_groups * sizeof(int32_t), s0) != cudaSuccess) ok = false;
     if (ok && cudaMemsetAsync(ctx->d_ctl, 0, sizeof(Ctl), s0) != cudaSuccess) ok = false;
     if (ok && cudaMemsetAsync(d.sel_ctr, 0, sizeof(unsigned int), s0) != cudaSuccess) ok = false;
     // the chunk tables live in pageable host vectors: finish the copies here

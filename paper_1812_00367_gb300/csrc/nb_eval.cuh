@@ -34,6 +34,8 @@
 // only its own state in registers.
 #pragma once
 
+#include <type_traits>
+
 #include "nb_fixed.cuh"
 #include "nb_internal.cuh"
 #include "nb_step.cuh"
@@ -745,6 +747,8 @@ struct EvalCfg<NB_EX> {
 template <int P, int MODE>
 constexpr int eval_min_blocks() {
     if constexpr (P == NB_EX && is_order4_mode(MODE)) return NB_EX4_MIN_BLOCKS;
+    if constexpr (P == kPrecPot) return 8;
+    if constexpr (P == NB_FP64 && uses_order4_terms(MODE)) return 5;
     return EvalCfg<P>::min_blocks;
 }
 template <>
@@ -760,12 +764,31 @@ struct EvalCfg<NB_FP32X> {
     static constexpr bool t64_smem = true;
 };
 
-// One piece of work, described by thread 0 for the whole CTA.
+// Pieces from which an i-tile's sum is formed by groups, and the partial sums
+// (doubles) per group counter: a group has at least six pieces of at least 40
+// doubles, so groups' first slots lie in different counters' ranges.
+constexpr int kTreePieces = 32;
+// ... and the pieces times i's, below which the second level of counters costs
+// more than it spares (us, FP64: N = 10007, A = 16, 128 pieces of 4 i's: 26.9 ->
+// 25.3; N = 16384, A = 1, 128 pieces of one: 17.6 -> 18.7).
+constexpr int kTreeSums = 512;
+
+// One piece of work, described by the first warp for the whole CTA.
 struct PieceRec {
-    long long item, item_end;  // current item / unit and the end of this CTA's work
     long long tb, te;          // j-tiles of the piece
     long long local, tile0, pslot0, off, nc, ntj;
-    int c, gl, split, A, tile, sk;  // c < 0: no more work
+    int c, gl, split, A, tile;  // c < 0: no more work
+};
+
+// What the pieces are described from (the launch's fields, kept out of registers).
+struct WorkRec {
+    long long item, item_end;  // item / unit to describe next and the end of this CTA's work
+    const ClusterPlan *plan;   // planned launches; NULL: direct
+    const int64_t *offsets, *jofs;
+    const void *jarr;
+    long long n;
+    int n_clusters, sk;        // sk: stream-K ranges
+    int cluster, gl, split, A, jt0, jt1;  // direct launches
 };
 
 template <int P>
@@ -775,6 +798,7 @@ struct SmemLayout {
     double t64[EvalCfg<P>::t64_smem ? 10 * kTPB : 1];  // FP32 totals, [q][thread]
     uint64_t bar[EvalCfg<P>::stages];
     PieceRec pc;
+    WorkRec work;
     int flag;
     int fail;
 };
@@ -821,12 +845,18 @@ static __device__ __noinline__ LaneSums reduce_lanes(double *o, int gl, int jsub
     return s;
 }
 
+// Largest c with plan[c].item0 <= item, by a full warp: 32 probes a round, so
+// that up to 1024 clusters take two loads in a row where a bisection takes ten.
 __device__ __forceinline__ int find_cluster(const ClusterPlan *plan, int nc, int64_t item) {
-    int lo = 0, hi = nc - 1;  // largest c with plan[c].item0 <= item
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (plan[mid].item0 <= item) lo = mid;
-        else hi = mid - 1;
+    const int lane = threadIdx.x & 31;
+    int lo = 0;
+    while (nc > 1) {  // the answer lies in [lo, lo + nc)
+        const int step = (nc + 31) / 32;
+        const int k = lane * step;
+        const unsigned le = __ballot_sync(0xffffffffu, k < nc && plan[lo + min(k, nc - 1)].item0 <= item);
+        const int hit = (__popc(le) - 1) * step;
+        lo += hit;
+        nc = min(step, nc - hit);
     }
     return lo;
 }
@@ -892,8 +922,69 @@ __device__ __forceinline__ void tile_pairs(const Dev &d, const typename Prec<P>:
 __device__ __forceinline__ int64_t sk_units(const Dev &d, const EvalLaunch &L) {
     const int c = L.direct ? L.cluster : 0;
     const int64_t tiles = L.direct ? L.tiles : d.plan[0].tiles;
-    const int64_t ntj = cdiv(d.offsets[c + 1] - d.offsets[c], kTJ);
+    const int64_t ntj = cdiv(d.n_clusters == 1 ? d.n : d.offsets[c + 1] - d.offsets[c], kTJ);
     return tiles * (L.direct ? (L.jt1 > 0 ? (int64_t)L.jt1 : ntj) - L.jt0 : ntj);
+}
+
+// The first warp: describes the piece at work.item (or the end of the work), and thread 0 starts the copies of its first j-tiles; the CTA reads the
+// record after its next barrier.  Out of line: inlined, it cost the pair loop 4-8 registers.
+template <int P>
+__device__ __noinline__ void describe(SmemLayout<P> &S) {
+    constexpr int kSt = EvalCfg<P>::stages;
+    using J = typename Prec<P>::J;
+    constexpr int kRecs = kTJ / Prec<P>::kPerRec;
+    WorkRec &W = S.work;
+    PieceRec &N = S.pc;
+    __syncwarp();
+    const int64_t item = W.item, item_end = W.item_end;
+    const bool one = W.n_clusters == 1;
+    int c = 0;
+    if (item < item_end && W.plan && !one) c = find_cluster(W.plan, W.n_clusters, item);
+    if (threadIdx.x != 0) return;
+    if (item >= item_end) {
+        N.c = -1;
+        return;
+    }
+    int gl, split, A;
+    int64_t item0 = 0, tile0 = 0, pslot0 = 0;
+    if (W.plan) {
+        const ClusterPlan pl = W.plan[c];
+        gl = pl.gl; split = pl.split; A = pl.active; item0 = pl.item0; tile0 = pl.tile0;
+        pslot0 = pl.pslot0;
+    } else {
+        c = W.cluster; gl = W.gl; split = W.split; A = W.A;
+    }
+    const int64_t off = one ? 0 : W.offsets[c];
+    const int64_t nc = one ? W.n : W.offsets[c + 1] - off;
+    const int64_t jofs = one ? 0 : W.jofs[c];
+    // the j-tiles this launch covers: all of the cluster's, or a host-given
+    // range [jt0, jt0 + ntj) of them (direct launches)
+    const int64_t jt0 = W.plan ? 0 : W.jt0;
+    const int64_t ntj = (!W.plan && W.jt1 > 0 ? (int64_t)W.jt1 : cdiv(nc, kTJ)) - jt0;
+    int tile;
+    int64_t tb, te, local = 0;
+    if (W.sk) {
+        tile = (int)(item / ntj);
+        tb = item - (int64_t)tile * ntj;
+        te = min(ntj, tb + (item_end - item));
+        W.item = item + (te - tb);
+    } else {
+        local = item - item0;
+        tile = (int)(local / split);
+        const int sidx = (int)(local % split);
+        tb = ntj * sidx / split;
+        te = ntj * (sidx + 1) / split;
+    }
+    tb += jt0;
+    te += jt0;
+    const J *jc = reinterpret_cast<const J *>(W.jarr) + jofs / Prec<P>::kPerRec;
+    for (int s = 0; s < kSt && tb + s < te; ++s) {
+        mbar_expect_tx(&S.bar[s], kRecs * sizeof(J));
+        tma_load_1d(&S.tile[s][0], jc + (tb + s) * kRecs, kRecs * sizeof(J), &S.bar[s]);
+    }
+    N.c = c; N.gl = gl; N.split = split; N.A = A; N.tile = tile;
+    N.tile0 = tile0; N.pslot0 = pslot0; N.local = local;
+    N.off = off; N.nc = nc; N.ntj = ntj; N.tb = tb; N.te = te;
 }
 
 template <int P, int MODE>
@@ -904,7 +995,6 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
     constexpr int kRecs = kTJ / T::kPerRec;  // records per j-tile
     extern __shared__ __align__(128) unsigned char smem_raw[];
     SmemLayout<P> &S = *reinterpret_cast<SmemLayout<P> *>(smem_raw);
-    PieceRec &R = S.pc;
     const int tid = threadIdx.x;
     if (L.gate && *L.gate == 0) return;  // done by the form that takes each pair once
 
@@ -912,95 +1002,59 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
     // [U k / G, U (k+1) / G) and walks it piece by piece (one piece per i-tile
     // it touches).  Otherwise work items (cluster, i-tile, split index):
     // direct launches (equal-cost items of one cluster) take a static round
-    // robin; planned launches fetch items dynamically, since clusters of a
-    // batch give items of unequal cost.  Either way a piece's arithmetic and
-    // the reduction order do not depend on the CTA that runs it.  Thread 0
-    // keeps the piece's bookkeeping in shared memory, so that the pair loop
-    // holds only what it uses in registers.
+    // robin; planned launches take item blockIdx.x first and the others
+    // dynamically, since clusters of a batch give items of unequal cost.
+    // Either way a piece's arithmetic and the reduction order do not depend on
+    // the CTA that runs it.  The pieces' bookkeeping stays in shared memory, so
+    // that the pair loop holds only what it uses in registers.
     if (tid == 0) {
         for (int s = 0; s < kSt; ++s) mbar_init(&S.bar[s], 1);
         S.fail = 0;
         fence_mbar_init();
-        R.sk = L.direct ? L.streamk != 0 : (d.n_clusters == 1 && d.plan[0].streamk != 0);
-        if (R.sk) {
-            R.item = sk_begin(sk_units(d, L), gridDim.x, blockIdx.x);
-            R.item_end = sk_begin(sk_units(d, L), gridDim.x, blockIdx.x + 1);
+        WorkRec &W = S.work;
+        W.plan = L.direct ? nullptr : d.plan;
+        W.offsets = d.offsets; W.jofs = d.jofs; W.jarr = d.jarr;
+        W.n = d.n; W.n_clusters = d.n_clusters;
+        W.cluster = L.cluster; W.gl = L.gl; W.split = L.split; W.A = L.n_active;
+        W.jt0 = L.jt0; W.jt1 = L.jt1;
+        W.sk = L.direct ? L.streamk != 0 : (d.n_clusters == 1 && d.plan[0].streamk != 0);
+        if (W.sk) {
+            const int64_t U = sk_units(d, L);
+            W.item = sk_begin(U, gridDim.x, blockIdx.x);
+            W.item_end = sk_begin(U, gridDim.x, blockIdx.x + 1);
         } else {
-            R.item_end = L.direct ? (int64_t)L.tiles * L.split : *d.n_items;
-            R.item = L.direct ? (int64_t)blockIdx.x : (long long)atomicAdd(d.item_ctr, 1ull);
+            W.item = blockIdx.x;
+            W.item_end = L.direct ? (int64_t)L.tiles * L.split : *d.n_items;
         }
     }
-    uint32_t phase = 0;   // bit s: parity of stage s
-    uint32_t pending = 0; // bit s: a copy into stage s is in flight
+    uint32_t phase = 0;  // bit s: parity of stage s
+    if (tid < 32) describe<P>(S);
 
+    const PieceRec &R = S.pc;
     for (;;) {
-        // thread 0: describe the current piece (or the end of the work)
-        if (tid == 0) {
-            const int64_t item = R.item;
-            if (item >= R.item_end) {
-                R.c = -1;
-            } else {
-                int c, gl, split, A;
-                int64_t item0, tile0, pslot0;
-                if (L.direct) {
-                    c = L.cluster; gl = L.gl; split = L.split; A = L.n_active; item0 = 0; tile0 = 0;
-                    pslot0 = 0;
-                } else {
-                    c = R.sk ? 0 : find_cluster(d.plan, d.n_clusters, item);
-                    const ClusterPlan pl = d.plan[c];
-                    gl = pl.gl; split = pl.split; A = pl.active; item0 = pl.item0; tile0 = pl.tile0;
-                    pslot0 = pl.pslot0;
-                }
-                const int64_t off = d.offsets[c];
-                const int64_t nc = d.offsets[c + 1] - off;
-                // the j-tiles this launch covers: all of the cluster's, or a
-                // host-given range [jt0, jt0 + ntj) of them (direct launches)
-                const int64_t jt0 = L.direct ? L.jt0 : 0;
-                const int64_t ntj = (L.direct && L.jt1 > 0 ? (int64_t)L.jt1 : cdiv(nc, kTJ)) - jt0;
-                int tile;
-                int64_t tb, te, local = 0;
-                if (R.sk) {
-                    tile = (int)(item / ntj);
-                    tb = item - (int64_t)tile * ntj;
-                    te = min(ntj, tb + (int64_t)(R.item_end - item));
-                } else {
-                    local = item - item0;
-                    tile = (int)(local / split);
-                    const int sidx = (int)(local % split);
-                    tb = ntj * sidx / split;
-                    te = ntj * (sidx + 1) / split;
-                }
-                tb += jt0;
-                te += jt0;
-                R.c = c; R.gl = gl; R.split = split; R.A = A; R.tile = tile;
-                R.tile0 = tile0; R.pslot0 = pslot0; R.local = local;
-                R.off = off; R.nc = nc; R.ntj = ntj; R.tb = tb; R.te = te;
-            }
-        }
+        // every thread is done with the last piece; this one's record is there
         __syncthreads();
         if (R.c < 0) break;
 
-        const int c = R.c;
         const int gl = R.gl;
         const int64_t tb = R.tb, te = R.te;
         const int ilane = tid / gl;
         const int jsub = tid % gl;
-        const J *jc = reinterpret_cast<const J *>(d.jarr) + d.jofs[c] / T::kPerRec;
+        const J *jc = reinterpret_cast<const J *>(d.jarr) + (d.n_clusters == 1 ? 0 : d.jofs[R.c] / T::kPerRec);
         // this thread's i: global index, bounds-checked against its cluster
-        auto i_of = [&](int il, bool &bad) -> int64_t {
-            const int64_t off = R.off;
+        auto i_of = [&](int64_t off, int64_t nc, int il, bool &bad) -> int64_t {
             int64_t g;
             if (L.identity) g = off + il;
             else if (L.direct) g = L.active[il];
             else g = d.active[off + il];
-            bad = g < off || g >= off + R.nc;
+            bad = g < off || g >= off + nc;
             return bad ? off : g;
         };
         const int il0 = R.tile * (kTPB / gl) + ilane;
         int64_t ji = 0;
         if (il0 < R.A) {
             bool bad;
-            ji = i_of(il0, bad) - R.off;
+            ji = i_of(R.off, R.nc, il0, bad) - R.off;
             if (bad) atomicOr(d.err, kErrIndex);  // caller-given index outside the cluster
         }
         typename T::I me = T::load_i(jc, ji);
@@ -1014,17 +1068,18 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
         for (int q = 0; q < 10; ++q) t64[q * t64st] = 0.0;
         const bool warp_active = __any_sync(0xffffffffu, il0 < R.A);
 
-        // prologue: fill the ring
-        if (tid == 0) {
-            for (int s = 0; s < kSt && tb + s < te; ++s) {
-                mbar_expect_tx(&S.bar[s], kRecs * sizeof(J));
-                tma_load_1d(&S.tile[s][0], jc + (tb + s) * kRecs, kRecs * sizeof(J), &S.bar[s]);
-                pending |= 1u << s;
-            }
-        }
         bool ok = true;
-        for (int64_t tt = tb; tt < te; ++tt) {
-            const int s = (int)((tt - tb) % kSt);
+        // FP64 and FP32 count the piece's tiles in 32 bits from its first, EX
+        // and FP32X by their index in the cluster: the same work, but the loop's
+        // registers differ (all active, N = 65536: FP64 4th order 21.0 -> 20.0
+        // ms, FP32 4th order 5.75 -> 5.71 ms, the other way round EX 1 % and
+        // FP32X 1 % slower)
+        constexpr bool kRel = P == NB_FP64 || P == NB_FP32 || P == kPrecPot;
+        using Tix = std::conditional_t<kRel, int, int64_t>;
+        const Tix t0 = kRel ? 0 : (Tix)tb, t1 = kRel ? (Tix)(te - tb) : (Tix)te;
+        int jrel = (int)(ji - tb * kTJ);  // the thread's i as a j of the current tile
+        for (Tix t = t0; t < t1; ++t) {
+            const int s = (int)((t - t0) % kSt);
             if (ok) ok = mbar_wait_bounded(&S.bar[s], (phase >> s) & 1u);
             phase ^= 1u << s;
             if (ok && warp_active) {
@@ -1032,49 +1087,57 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
                 // the pairs i = j of a warp lie in a few tiles: the others run a
                 // loop without the exclusion's compares and selects (FP32X 5 %,
                 // FP32 3-5 %, EX 1.5-2.5 % faster, the same results)
-                const int js = (int)min(max(ji - tt * kTJ, (int64_t)-1), (int64_t)kTJ);
+                int js;
+                if constexpr (kRel) js = min(max(jrel, -1), kTJ);
+                else js = (int)min(max(ji - t * kTJ, (int64_t)-1), (int64_t)kTJ);
                 if (__any_sync(0xffffffffu, (unsigned)js < (unsigned)kTJ))
                     tile_pairs<P, MODE, true>(d, me, tl, js, jsub, gl, acc);
                 else
                     tile_pairs<P, MODE, false>(d, me, tl, js, jsub, gl, acc);
                 if constexpr (P == NB_FP32 || P == NB_FP32X) {
-                    if ((tt - tb + 1) % kFp32FlushTiles == 0) T::flush(acc, t64, t64st);
+                    if ((t - t0 + 1) % kFp32FlushTiles == 0) T::flush(acc, t64, t64st);
                     else T::tile_done(acc);
                 } else if constexpr (P == NB_EX) {
                     T::tile_done(acc);
                 } else if constexpr (P == NB_FP64) {
                     // every 64 pairs of the lane (four FP64 operations)
-                    if (((int)(tt - tb + 1) & (gl - 1)) == 0) T::tile_done(acc);
+                    if (((int)(t - t0 + 1) & (gl - 1)) == 0) T::tile_done(acc);
                 }
             }
-            if (!ok) S.fail = 1;
+            jrel -= kTJ;
+            if (!ok) S.fail = 1 + (int)(t - t0);
             __syncthreads();
             if (S.fail) break;
-            if (tid == 0) {
-                pending &= ~(1u << s);
-                if (tt + kSt < te) {
-                    mbar_expect_tx(&S.bar[s], kRecs * sizeof(J));
-                    tma_load_1d(&S.tile[s][0], jc + (tt + kSt) * kRecs, kRecs * sizeof(J), &S.bar[s]);
-                    pending |= 1u << s;
-                }
+            if (tid == 0 && t + kSt < t1) {
+                mbar_expect_tx(&S.bar[s], kRecs * sizeof(J));
+                tma_load_1d(&S.tile[s][0], jc + ((kRel ? tb : 0) + t + kSt) * kRecs, kRecs * sizeof(J), &S.bar[s]);
             }
         }
         if (S.fail) {
             // a copy did not land in time: record it, drain (bounded) what this
-            // CTA still has in flight, and leave the kernel
+            // CTA still has in flight (from the failing tile on; the parity of
+            // its stage is one ahead already), and leave the kernel
             if (tid == 0) {
                 atomicOr(d.err, kErrTimeout);
-                for (int s = 0; s < kSt; ++s)
-                    if (pending & (1u << s)) (void)mbar_wait_bounded(&S.bar[s], (phase >> s) & 1u);
+                const int k0 = S.fail - 1, nt = (int)(te - tb);
+                phase ^= 1u << (k0 % kSt);
+                for (int k = k0; k < nt && k < k0 + kSt; ++k)
+                    (void)mbar_wait_bounded(&S.bar[k % kSt], (phase >> (k % kSt)) & 1u);
             }
             return;
         }
 
-        // ---- epilogue: the piece's bookkeeping comes back from shared memory
-        const int tile = R.tile, A = R.A, split = R.split;
+        // ---- epilogue: the piece's bookkeeping comes back from shared memory;
+        // past the barrier below the record describes the next piece.  The
+        // next item is fetched ahead of the sums and its first j-tiles are
+        // under way while this piece's sums are joined.
+        long long next = 0;
+        if (tid == 0 && !S.work.sk)
+            next = gridDim.x + (L.direct ? S.work.item : (long long)atomicAdd(d.item_ctr, 1ull));
+        const int c = R.c, tile = R.tile, A = R.A, split = R.split;
         const int Ti = kTPB / R.gl;
-        const int64_t ntj = R.ntj;
-        const bool sk = R.sk;
+        const int64_t off = R.off, nc = R.nc, ntj = R.ntj, tile0 = R.tile0;
+        const bool sk = S.work.sk;
         // pieces of this i-tile: split items, or the CTAs whose ranges meet it
         int npieces = split;
         int64_t sk_first = 0, sk_maxp = 0, sk_loc0 = 0;
@@ -1102,73 +1165,96 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
         // of q in [held.off, held.lim) in o[0 ..]
         const LaneSums held = reduce_lanes(o, R.gl, tid & (R.gl - 1));
         const int slot = tid / R.gl;
-        if (npieces == 1 && Ti == kTPB) {
-            const int il = tile * Ti + tid;
-            if (il < A) {
-                bool bad;
-                const int64_t gi = i_of(il, bad);
-                if (!bad) finalize_one<P, MODE>(d, L, c, gi, il, o);
-            }
-        } else if (npieces == 1) {
-            // one thread per i gathers its ten sums
+        // this CTA's piece of the tile, and its group when the groups' sums are
+        // formed by their own last CTAs
+        const int piece = sk ? (int)((int64_t)blockIdx.x - sk_first) : (int)(R.local - (int64_t)tile * split);
+        const int Rg = min((npieces + 7) / 8, kTPB / Ti);
+        const int nv = min(Ti, A - tile * Ti);  // valid i in this tile
+        const bool tree = npieces >= kTreePieces && npieces * nv >= kTreeSums;
+        const int grp = tree ? ((piece + 1) * Rg - 1) / npieces : 0;
+        const int g0 = npieces * grp / Rg, g1 = npieces * (grp + 1) / Rg;
+        if (npieces > 1) {
+            held.store(o, d.partial + piece_slot(piece) + slot, Ti);
+            __threadfence();
+        } else if (Ti < kTPB) {
             held.store(o, S.red + slot, Ti);
-            __syncthreads();
+        }
+        __syncthreads();
+        if (tid < 32) {
+            int prev = 0;
+            if (tid == 0) {
+                if (tree) prev = atomicAdd(&d.grp_cnt[piece_slot(g0) / kGrpStride], 1);
+                else if (npieces > 1) prev = atomicAdd(&d.tile_cnt[tile0 + tile], 1);
+                if (!sk) S.work.item = next;
+            }
+            describe<P>(S);
+            if (tid == 0) S.flag = (prev == (tree ? g1 - g0 : npieces) - 1);
+        }
+        if (npieces == 1) {
+            // one thread per i (gathering its ten sums if lanes shared it)
             const int il = tile * Ti + tid;
             if (tid < Ti && il < A) {
-                double sum[10];
+                if (Ti < kTPB) {
 #pragma unroll
-                for (int q = 0; q < 10; ++q) sum[q] = S.red[q * Ti + tid];
+                    for (int q = 0; q < 10; ++q) o[q] = S.red[q * Ti + tid];
+                }
                 bool bad;
-                const int64_t gi = i_of(il, bad);
-                if (!bad) finalize_one<P, MODE>(d, L, c, gi, il, sum);
+                const int64_t gi = i_of(off, nc, il, bad);
+                if (!bad) finalize_one<P, MODE>(d, L, c, gi, il, o);
             }
         } else {
-            // this CTA's piece of the tile
-            double *part = d.partial + (sk ? piece_slot((int64_t)blockIdx.x - sk_first)
-                                           : pslot0 + R.local * (int64_t)(10 * Ti));
-            held.store(o, part + slot, Ti);
-            __threadfence();
+            // The last CTA of this i-tile adds the pieces for every (i, q) pair
+            // in two fixed-order levels: contiguous groups of pieces, each in
+            // piece order, then the group sums in group order.  The order
+            // depends only on the pieces and the tile's width, so results are
+            // reproducible and the same for every i.  Groups of eight pieces
+            // (more when S.red would overflow): a chain of hundreds of loads and
+            // additions in a handful of threads took longer than the pairs
+            // themselves.  From kTreePieces pieces on, the last CTA of each group
+            // forms its sum (in the place of the group's first piece): one CTA
+            // adding 76 pieces of 16 i's took 38 us at the end of a launch of
+            // 316 (N = 65536, A = 128), its SM alone at work.
+            const int npair = nv * 10;
+            // pieces at a fixed stride (the first of a stream-K tile sits elsewhere)
+            const int64_t stride = (sk ? sk_maxp : (int64_t)1) * (10 * Ti);
+            double *first = d.partial + piece_slot(0);
+            double *rest = first - (sk ? sk_loc0 : (int64_t)0) * (10 * Ti);
+            auto at = [&](int s) { return s == 0 ? first : rest + s * stride; };
+            // the sum of pieces s0 .. s1 - 1 at an offset, eight loads in flight
+            auto sum_pieces = [&](int s0, int s1, int col) {
+                double sum = 0.0;
+                for (int sp = s0; sp < s1; sp += 8) {
+                    double t[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) t[u] = sp + u < s1 ? __ldcg(at(sp + u) + col) : 0.0;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if (sp + u < s1) sum += t[u];
+                }
+                return sum;
+            };
             __syncthreads();
-            if (tid == 0) {
-                const int prev = atomicAdd(&d.tile_cnt[R.tile0 + tile], 1);
-                S.flag = (prev == npieces - 1);
-            }
-            __syncthreads();
-            if (S.flag) {
-                // Last CTA of this i-tile: add the partials of its pieces for
-                // every (i, q) pair in two fixed-order levels.  Level 1: thread
-                // (p, r) sums the r-th contiguous group of pieces of pair p in
-                // piece order; level 2 adds the Rg group sums in group order.
-                // The order depends only on the pieces and the tile's width, so
-                // results are reproducible and the same for every i.  Groups of
-                // eight pieces (more when S.red would overflow): a tile of few
-                // i's may have hundreds of pieces, and a chain of that many
-                // loads and additions in a handful of threads took longer than
-                // the pairs themselves.
+            if (tree && S.flag) {
                 __threadfence();
-                const int nv = min(Ti, A - tile * Ti);     // valid i in this tile
-                const int npair = nv * 10;
-                const int Rg = min((npieces + 7) / 8, kTPB / Ti);
+                for (int p = tid; p < npair; p += kTPB) {
+                    const int col = p / nv * Ti + p % nv;
+                    at(g0)[col] = sum_pieces(g0, g1, col);
+                }
+                __threadfence();
+                __syncthreads();
+                if (tid == 0) {
+                    d.grp_cnt[piece_slot(g0) / kGrpStride] = 0;
+                    S.flag = atomicAdd(&d.tile_cnt[tile0 + tile], 1) == Rg - 1;
+                }
+                __syncthreads();
+            }
+            if (S.flag) {
+                __threadfence();
                 for (int w = tid; w < npair * Rg; w += kTPB) {
                     const int p = w % npair, r = w / npair;
-                    const int q = p / nv, il = p % nv;
-                    const int s0 = (int)((int64_t)npieces * r / Rg), s1 = (int)((int64_t)npieces * (r + 1) / Rg);
-                    // pieces at a fixed stride (the first of a stream-K tile
-                    // sits elsewhere), eight loads in flight
-                    const int64_t stride = (sk ? sk_maxp : (int64_t)1) * (10 * Ti);
-                    const double *base = d.partial + piece_slot(0) + q * Ti + il;
-                    const double *rest = base - (sk ? sk_loc0 : (int64_t)0) * (10 * Ti);
-                    double acc2 = 0.0;
-                    for (int sp = s0; sp < s1; sp += 8) {
-                        double t[8];
-#pragma unroll
-                        for (int u = 0; u < 8; ++u)
-                            t[u] = sp + u < s1 ? __ldcg(sp + u == 0 ? base : rest + (sp + u) * stride) : 0.0;
-#pragma unroll
-                        for (int u = 0; u < 8; ++u)
-                            if (sp + u < s1) acc2 += t[u];
-                    }
-                    S.red[r * npair + p] = acc2;
+                    const int col = p / nv * Ti + p % nv;
+                    const int s0 = npieces * r / Rg, s1 = npieces * (r + 1) / Rg;
+                    S.red[r * npair + p] = tree ? __ldcg(at(s0) + col) : sum_pieces(s0, s1, col);
                 }
                 __syncthreads();
                 for (int p = tid; p < npair; p += kTPB) {
@@ -1183,18 +1269,11 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
                     for (int q = 0; q < 10; ++q) sum[q] = S.red[q * nv + tid];
                     const int il = tile * Ti + tid;
                     bool bad;
-                    const int64_t g2 = i_of(il, bad);
+                    const int64_t g2 = i_of(off, nc, il, bad);
                     if (!bad) finalize_one<P, MODE>(d, L, c, g2, il, sum);
                 }
-                if (tid == 0) d.tile_cnt[R.tile0 + tile] = 0;
+                if (tid == 0) d.tile_cnt[tile0 + tile] = 0;
             }
-        }
-        // next piece: every thread is done with this piece's record
-        __syncthreads();
-        if (tid == 0) {
-            if (R.sk) R.item += R.te - R.tb;
-            else if (L.direct) R.item += gridDim.x;
-            else R.item = (long long)atomicAdd(d.item_ctr, 1ull);
         }
     }
 }

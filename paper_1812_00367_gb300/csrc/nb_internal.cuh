@@ -61,6 +61,7 @@ constexpr int kChunk = 2048;   // particles per select / predict chunk
 constexpr int kSelTPB = 256;   // threads per select CTA
 constexpr int kPredTPB = 64;   // threads per predict CTA
 constexpr int kPlanTPB = 1024; // threads of the single planning CTA
+constexpr int kGrpStride = 160;  // doubles of partial sums per group counter (nb_eval.cuh)
 constexpr int kBuckets = 32;   // active-set size buckets (floor log2 A)
 constexpr int kFp32FlushTiles = 32;  // FP32 path: j-tiles summed in FP32 before
                                      // promotion to FP64 (32 x 64 = 2048 j)
@@ -235,6 +236,7 @@ struct Dev {
     uint64_t eps_x;
     uint32_t eps_emin;
     FxK fxk;  // {1, 2} as run-time values (nb_fixed.cuh)
+    int32_t *grp_cnt;  // [partial_cap / kGrpStride + 1]: pieces of a group done
 };
 
 // The small values host and device exchange, in one block: the host reads it

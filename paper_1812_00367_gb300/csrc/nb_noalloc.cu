@@ -29,7 +29,10 @@ constexpr size_t kNaTileBytes = (size_t)kNaMaxTiles * sizeof(int32_t);
 constexpr size_t kNaOffJarr = 0;
 constexpr size_t kNaOffPart = kNaOffJarr + kNaJarrBytes;
 constexpr size_t kNaOffTile = kNaOffPart + kNaPartBytes;
-constexpr size_t kNaOffAux = kNaOffTile + ((kNaTileBytes + 255) / 256) * 256;
+constexpr int64_t kNaMaxGroups = kNaMaxItems * 10 * kTPB / kGrpStride + 1;
+constexpr size_t kNaGrpBytes = (size_t)kNaMaxGroups * sizeof(int32_t);
+constexpr size_t kNaOffGrp = kNaOffTile + ((kNaTileBytes + 255) / 256) * 256;
+constexpr size_t kNaOffAux = kNaOffGrp + ((kNaGrpBytes + 255) / 256) * 256;
 constexpr size_t kNaBytes = kNaOffAux + 256;  // about 5.8 MB in all
 
 struct NaAux {
@@ -70,6 +73,8 @@ __global__ void k_na_prepare(unsigned char *base, const double *jp, int64_t n, i
         jarr[i] = jfx_pack(x, v, a, m);
     }
     for (int64_t k = i0; k < tiles; k += stride) tc[k] = 0;
+    int32_t *gc = reinterpret_cast<int32_t *>(base + kNaOffGrp);
+    for (int64_t k = i0; k < kNaMaxGroups; k += stride) gc[k] = 0;
     if (i0 == 0) {
         aux->offsets[0] = 0;
         aux->offsets[1] = n;
@@ -168,6 +173,7 @@ extern "C" nb_status nb_evaluate_noalloc(const double *jpred, int64_t n, double 
     d.partial = reinterpret_cast<double *>(slot.base + kNaOffPart);
     d.partial_cap = kNaMaxItems * 10 * kTPB;  // doubles
     d.tile_cnt = reinterpret_cast<int32_t *>(slot.base + kNaOffTile);
+    d.grp_cnt = reinterpret_cast<int32_t *>(slot.base + kNaOffGrp);
     d.err = &aux->err;
     set_eps2(d, eps);
     d.neg_one = -1.0;
