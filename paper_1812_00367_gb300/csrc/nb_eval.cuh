@@ -866,10 +866,6 @@ __device__ __forceinline__ void finalize_one(const Dev &d, const EvalLaunch &L, 
                                              int iloc, const double o[10]) {
     if constexpr (MODE == kModeOut || MODE == kModeOut4) {
         for (int q = 0; q < 10; ++q) L.out[(int64_t)q * L.n_active + iloc] = o[q];
-    } else if constexpr (MODE == kModeStep) {
-        correct_particle(d, gi, d.tnext[c], o);
-    } else if constexpr (MODE == kModeStep4) {
-        correct_particle4(d, gi, d.tnext[c], o);
     } else if constexpr (MODE == kModeInit1 || MODE == kModeInit2 || MODE == kModeInit4) {
         const int64_t n = d.n;
         for (int k = 0; k < 3; ++k) {
@@ -1170,13 +1166,19 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
         const int piece = sk ? (int)((int64_t)blockIdx.x - sk_first) : (int)(R.local - (int64_t)tile * split);
         const int Rg = min((npieces + 7) / 8, kTPB / Ti);
         const int nv = min(Ti, A - tile * Ti);  // valid i in this tile
+        constexpr bool kStep = MODE == kModeStep || MODE == kModeStep4;
+        auto particle = [&](int il) -> int64_t {
+            bool bad;
+            const int64_t gi = i_of(off, nc, tile * Ti + il, bad);
+            return bad ? -1 : gi;
+        };
         const bool tree = npieces >= kTreePieces && npieces * nv >= kTreeSums;
         const int grp = tree ? ((piece + 1) * Rg - 1) / npieces : 0;
         const int g0 = npieces * grp / Rg, g1 = npieces * (grp + 1) / Rg;
         if (npieces > 1) {
             held.store(o, d.partial + piece_slot(piece) + slot, Ti);
             __threadfence();
-        } else if (Ti < kTPB) {
+        } else if (Ti < kTPB || kStep) {
             held.store(o, S.red + slot, Ti);
         }
         __syncthreads();
@@ -1190,7 +1192,9 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
             describe<P>(S);
             if (tid == 0) S.flag = (prev == (tree ? g1 - g0 : npieces) - 1);
         }
-        if (npieces == 1) {
+        if (npieces == 1 && kStep) {
+            correct_tile<MODE == kModeStep4>(d, nv, d.tnext[c], S.red, Ti, particle);
+        } else if (npieces == 1) {
             // one thread per i (gathering its ten sums if lanes shared it)
             const int il = tile * Ti + tid;
             if (tid < Ti && il < A) {
@@ -1263,7 +1267,9 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
                     S.red[p] = a2;
                 }
                 __syncthreads();
-                if (tid < nv) {
+                if constexpr (kStep) {
+                    correct_tile<MODE == kModeStep4>(d, nv, d.tnext[c], S.red, nv, particle);
+                } else if (tid < nv) {
                     double sum[10];
 #pragma unroll
                     for (int q = 0; q < 10; ++q) sum[q] = S.red[q * nv + tid];
