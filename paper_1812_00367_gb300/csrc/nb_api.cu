@@ -541,6 +541,8 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
     ALLOC(d.nact, n_clusters);
     ALLOC(d.active, n);
     ALLOC(d.plan, n_clusters);
+    ALLOC(d.order_item0, n_clusters);
+    ALLOC(d.order_cluster, n_clusters);
     ALLOC(d.n_items, 1);
     ALLOC(d.item_ctr, 1);
     ALLOC(d.sel_ctr, 1);

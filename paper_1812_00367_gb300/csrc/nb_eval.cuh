@@ -784,7 +784,8 @@ struct PieceRec {
 struct WorkRec {
     long long item, item_end;  // item / unit to describe next and the end of this CTA's work
     const ClusterPlan *plan;   // planned launches; NULL: direct
-    const int64_t *offsets, *jofs;
+    const int64_t *offsets, *jofs, *order_item0;
+    const int32_t *order_cluster;
     const void *jarr;
     long long n;
     int n_clusters, sk;        // sk: stream-K ranges
@@ -845,15 +846,15 @@ static __device__ __noinline__ LaneSums reduce_lanes(double *o, int gl, int jsub
     return s;
 }
 
-// Largest c with plan[c].item0 <= item, by a full warp: 32 probes a round, so
+// Largest k with item0[k] <= item, by a full warp: 32 probes a round, so
 // that up to 1024 clusters take two loads in a row where a bisection takes ten.
-__device__ __forceinline__ int find_cluster(const ClusterPlan *plan, int nc, int64_t item) {
+__device__ __forceinline__ int find_cluster(const int64_t *item0, int nc, int64_t item) {
     const int lane = threadIdx.x & 31;
     int lo = 0;
     while (nc > 1) {  // the answer lies in [lo, lo + nc)
         const int step = (nc + 31) / 32;
         const int k = lane * step;
-        const unsigned le = __ballot_sync(0xffffffffu, k < nc && plan[lo + min(k, nc - 1)].item0 <= item);
+        const unsigned le = __ballot_sync(0xffffffffu, k < nc && item0[lo + min(k, nc - 1)] <= item);
         const int hit = (__popc(le) - 1) * step;
         lo += hit;
         nc = min(step, nc - hit);
@@ -935,7 +936,7 @@ __device__ __noinline__ void describe(SmemLayout<P> &S) {
     const int64_t item = W.item, item_end = W.item_end;
     const bool one = W.n_clusters == 1;
     int c = 0;
-    if (item < item_end && W.plan && !one) c = find_cluster(W.plan, W.n_clusters, item);
+    if (item < item_end && W.plan && !one) c = W.order_cluster[find_cluster(W.order_item0, W.n_clusters, item)];
     if (threadIdx.x != 0) return;
     if (item >= item_end) {
         N.c = -1;
@@ -1010,6 +1011,7 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
         WorkRec &W = S.work;
         W.plan = L.direct ? nullptr : d.plan;
         W.offsets = d.offsets; W.jofs = d.jofs; W.jarr = d.jarr;
+        W.order_item0 = d.order_item0; W.order_cluster = d.order_cluster;
         W.n = d.n; W.n_clusters = d.n_clusters;
         W.cluster = L.cluster; W.gl = L.gl; W.split = L.split; W.A = L.n_active;
         W.jt0 = L.jt0; W.jt1 = L.jt1;

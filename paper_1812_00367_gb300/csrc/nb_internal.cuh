@@ -237,6 +237,9 @@ struct Dev {
     uint32_t eps_emin;
     FxK fxk;  // {1, 2} as run-time values (nb_fixed.cuh)
     int32_t *grp_cnt;  // [partial_cap / kGrpStride + 1]: pieces of a group done
+    // several clusters: the active ones by first item (unused: INT64_MAX)
+    int64_t *order_item0;    // [nc]
+    int32_t *order_cluster;  // [nc]
 };
 
 // The small values host and device exchange, in one block: the host reads it

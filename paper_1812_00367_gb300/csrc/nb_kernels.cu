@@ -12,6 +12,9 @@
 // particles in order.  The planner and the predictor need only t_next and the
 // count, so they run beside pass 2.  The active list takes no atomics and is
 // deterministic.
+#include <climits>
+#include <cstdint>
+
 #include "nb_internal.cuh"
 #include "nb_step.cuh"
 
@@ -274,7 +277,8 @@ __device__ __forceinline__ ClusterPlan plan_cluster(const Dev &d, int64_t ncl, i
 
 // One CTA.  Per cluster: A -> bucket floor(log2 A) -> (gl, target items) ->
 // i-tiles and split S (clamped to the cluster's j-tiles); exclusive scans
-// give each cluster its first item and first tile.  If the items that need
+// give each cluster its first tile and partial sums, a counting sort by cost its
+// first item.  If the items that need
 // partial sums exceed the scratch capacity, every split falls back to 1.
 // mode_init: every particle active (start-up and energy evaluations).
 __global__ void __launch_bounds__(kPlanTPB) k_plan(const Dev d, int mode_init, int count) {
@@ -301,12 +305,29 @@ __global__ void __launch_bounds__(kPlanTPB) k_plan(const Dev d, int mode_init, i
         }
         return;
     }
+    // Items are numbered by cost, dearest first (in classes of a factor of two):
+    // the items fetched last, which the other CTAs wait for, are then the
+    // cheapest (block steps of 96 clusters, N up to 4096: FP64 22.5 -> 22.0 ms, EX
+    // 13.8 -> 13.4; 8 clusters, few items a CTA, 2.72 -> 2.74).  The order within
+    // a class is the atomics'; no result depends on it.  s_cls: a class's totals,
+    // then its next free place: clusters in the upper 24 bits, items below.
+    __shared__ unsigned long long s_cls[32];
+    constexpr unsigned long long kOne = 1ull << 40;
+    auto cost_class = [&](const ClusterPlan &pl, int64_t ncl) {
+        const long long cost = (kTPB / pl.gl) * cdiv(cdiv(ncl, kTJ), pl.split);  // i's x j-tiles
+        return __clz((int)min(cost, (long long)INT_MAX));
+    };
     for (int fallback = 0; fallback < 2; ++fallback) {
-        long long carry_items = 0, carry_tiles = 0, carry_slots = 0;
+        long long carry_tiles = 0, carry_slots = 0;
+        if (tid < 32) s_cls[tid] = 0ull;
+        __syncthreads();
+        ClusterPlan pl{};  // of this thread's last cluster, `mine`
+        int mine = -1;
         double inter = 0.0, busy = 0.0;
         for (int base = 0; base < d.n_clusters; base += (int)blockDim.x) {
             const int c = base + tid;
-            ClusterPlan pl{1, 1, 0, 0, 0, 0, 0, 0, 0};
+            pl = ClusterPlan{1, 1, 0, 0, 0, 0, 0, 0, 0};
+            mine = c;
             long long items = 0, tiles = 0;
             double my_inter = 0.0;
             if (c < d.n_clusters) {
@@ -316,35 +337,42 @@ __global__ void __launch_bounds__(kPlanTPB) k_plan(const Dev d, int mode_init, i
                     pl = plan_cluster(d, ncl, A, fallback != 0, items);
                     tiles = pl.tiles;
                     my_inter = (double)A * (double)(ncl - 1);
+                    atomicAdd(&s_cls[cost_class(pl, ncl)], kOne + items);
                 }
             }
             // partial sums: 10 doubles per i of every item of a split cluster
             const long long sitems = pl.split > 1 ? items * 10 * (kTPB / pl.gl) : 0;
-            const long long ii = block_scan_incl(items, s_l);
             const long long it = block_scan_incl(tiles, s_l);
             const long long is = block_scan_incl(sitems, s_l);
-            pl.item0 = carry_items + ii - items;
+            pl.item0 = items;  // its place follows below
             pl.tile0 = carry_tiles + it - tiles;
             pl.pslot0 = carry_slots + is - sitems;
-            if (c < d.n_clusters) d.plan[c] = pl;
+            if (c < d.n_clusters && base + (int)blockDim.x < d.n_clusters) d.plan[c] = pl;
             // the last thread holds the inclusive totals
             if (tid == (int)blockDim.x - 1) {
-                s_l[0] = ii;
-                s_l[1] = it;
-                s_l[2] = is;
+                s_l[0] = it;
+                s_l[1] = is;
             }
             __syncthreads();
-            carry_items += s_l[0];
-            carry_tiles += s_l[1];
-            carry_slots += s_l[2];
+            carry_tiles += s_l[0];
+            carry_slots += s_l[1];
             __syncthreads();
             inter += block_sum_d(my_inter, s_d);
             busy += block_sum_d(pl.active > 0 ? 1.0 : 0.0, s_d);
         }
         // the split items' partial sums must fit the scratch (uniform decision)
         if (!fallback && carry_slots > d.partial_cap) continue;
+        if (tid < 32) {  // the classes' first places
+            unsigned long long at = s_cls[tid];
+            const unsigned long long own = at;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long add = __shfl_up_sync(0xffffffffu, at, o);
+                if (tid >= o) at += add;
+            }
+            s_cls[tid] = at - own;
+            if (tid == 31) *d.n_items = (long long)(at & (kOne - 1));
+        }
         if (tid == 0) {
-            *d.n_items = carry_items;
             *d.item_ctr = 0ull;
             *d.busy = (int)busy;
             if (count && !mode_init) {
@@ -352,6 +380,19 @@ __global__ void __launch_bounds__(kPlanTPB) k_plan(const Dev d, int mode_init, i
                 *d.ctr_inter += inter;
             }
         }
+        __syncthreads();
+        for (int c = tid; c < d.n_clusters; c += (int)blockDim.x) {
+            ClusterPlan q = c == mine ? pl : d.plan[c];  // written by this thread
+            if (q.active > 0) {
+                const int64_t ncl = d.offsets[c + 1] - d.offsets[c];
+                const unsigned long long at = atomicAdd(&s_cls[cost_class(q, ncl)], kOne + (unsigned long long)q.item0);
+                q.item0 = (int64_t)(at & (kOne - 1));
+                d.order_item0[at >> 40] = q.item0;
+                d.order_cluster[at >> 40] = c;
+            }
+            d.plan[c] = q;
+        }
+        for (int k = (int)busy + tid; k < d.n_clusters; k += (int)blockDim.x) d.order_item0[k] = INT64_MAX;
         break;
     }
 }
