@@ -11,7 +11,7 @@
 // i.e. NM08's A1 = m v/s^3 - 3 alpha A0 and A2 = m a/s^3 - 6 alpha A1 - 3 beta A0
 // with the large alpha terms cancelling inside each pair before it is summed
 // (that keeps the FP32 path within its bound on strongly cancelling sums).
-// FP64: the pair terms run in block fixed point on the integer pipes
+// FP64: the pair terms run in fixed point on the integer pipes
 // (nb_fixed.cuh); 12 FP64 instructions per pair remain, the coordinate
 // differences and the nine running sums (9 in the 4th-order form); the
 // potential m y is summed in float-float on the FP32 pipe.  The 4th-order
@@ -46,26 +46,25 @@ template <int P>
 struct Prec;
 
 // ===================================================================== FP64
-// Block fixed-point pair terms (nb_fixed.cuh): the coordinate differences and
-// the nine running sums stay on the FP64 pipe (12 instructions per pair, 9 in
-// the 4th-order form), everything between them runs on the integer pipes.
+// Fixed-point pair terms (nb_fixed.cuh): the coordinate differences and the nine
+// running sums stay on the FP64 pipe (12 instructions per pair, 9 in the 4th-order
+// form), everything between them runs on the integer pipes.
 // Bound: the issue of half-rate integer instructions (shifts, logic,
-// IMAD.WIDE; about 650 instructions a pair and warp; ALU and FP64 pipes both
-// near 60 % busy).  Measured, N = 65536 all active: 133.2 ms (3.22e10 pairs/s)
-// against 361.2 ms for the same terms in doubles (50 DFMA a pair, the FP64
-// pipe 95 % busy); 4th order, N = 30011: 17.3 against 44.8 ms; A = 48: 144
-// against 324 us.  Residency: 3, 4, 5 or 6 CTAs per SM measured within 1 % of
-// one another.  Converting w1, w2 with the count of leading zeros of the high
-// word (a general conversion where a component is that small) instead of a
-// float's exponent: 138.6 -> 133.2 ms.
+// IMAD.WIDE; 778 instructions a pair and warp; ALU 59 % and FP64 pipe 53 % busy).
+// Measured, N = 65536, A = 1000: 2.51 ms (2.61e10 pairs/s) against 5.70 ms for the
+// same terms in doubles (50 DFMA a pair, the FP64 pipe 95 % busy); A = 48: 157
+// against 324 us.  Residency: 3 and 4 CTAs per SM measured within 1 % of one
+// another over the FP64 cases (A = 48 3 % faster, a batch 3 % slower with 3).
+// Converting w1, w2 with the count of leading zeros of the high word (a general
+// conversion where a component is that small) instead of a float's exponent: 138.6
+// -> 133.2 ms for all pairs of N = 65536.
 template <>
 struct Prec<NB_FP64> {
     using J = JFX;
     static constexpr int kPerRec = 1;  // particles per record
     struct I {
         double x[3];
-        int64_t v[3], a[3];
-        int32_t ev, ea;
+        FxP3 v, a;
         double m1;       // -1.0 from the kernel parameters (see Dev)
         uint64_t eps_x;  // eps^2 as a fixed-point number and its block exponent
         uint32_t emin;
@@ -74,7 +73,7 @@ struct Prec<NB_FP64> {
     struct Acc {
         double a[3], j[3], s[3], p;
         ff pf;         // the current j-tile's potential as a float pair
-        int32_t fv, fa;  // largest stored exponent of v, a seen (kFxBad: a non-finite one)
+        int32_t fv, fa;  // largest exponent field of a velocity, an acceleration
     };
     static __device__ __forceinline__ void prepare(I &i, const Dev &d) {
         i.m1 = d.neg_one;
@@ -86,13 +85,9 @@ struct Prec<NB_FP64> {
         const J e = jarr[k];
         I r;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            r.x[q] = e.x[q];
-            r.v[q] = e.v[q];
-            r.a[q] = e.a[q];
-        }
-        r.ev = jfx_ev(e);
-        r.ea = jfx_ea(e);
+        for (int q = 0; q < 3; ++q) r.x[q] = e.x[q];
+        r.v = jfx_v(e);
+        r.a = jfx_a(e);
         return r;
     }
     static __device__ __forceinline__ void zero(Acc &c) {
@@ -100,7 +95,7 @@ struct Prec<NB_FP64> {
         for (int k = 0; k < 3; ++k) c.a[k] = c.j[k] = c.s[k] = 0.0;
         c.p = 0.0;
         c.pf = ff{0.f, 0.f};
-        c.fv = c.fa = kFxMinExp;
+        c.fv = c.fa = 0;
     }
     // potential term m y in float-float, renormalised every term (|lo| stays
     // below half an ulp of hi): a 64-term tile sum is good to ~2^-45, and
@@ -124,74 +119,15 @@ struct Prec<NB_FP64> {
     };
     template <bool kOrder6>
     static __device__ __forceinline__ void terms(const I &i, const J &jj, Acc &c, Terms &o) {
-        double (&r)[3] = o.r, (&w1)[3] = o.w1, (&w2)[3] = o.w2;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) r[k] = fma_rn_f64(i.x[k], i.m1, jj.x[k]);
-        const int evj = jfx_ev(jj);
-        const Fx3 R = fx_decode(r, i.emin);
-        const Fx3 V = fx_diff_norm(jj.v, evj, i.v, i.ev);
-        FxS Rs[3], Vs[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            Rs[k] = fx_split(R.w[k]);
-            Vs[k] = fx_split(V.w[k]);
-        }
-        const FxRoot t = o.t = fx_root(Rs, R.e, i.eps_x, i.emin, i.K);
-        c.fv = max(c.fv, evj);
-        Fx3 A;
-        if constexpr (kOrder6) {
-            const int eaj = jfx_ea(jj);
-            c.fa = max(c.fa, eaj);
-            A = fx_diff_norm(jj.a, eaj, i.a, i.ea);
-        }
-        if (fx_inside(r, i.emin)) {
-            // r below the softening's scale (and the pair i == j): its block
-            // would carry too few bits, so alpha, beta, w1 and w2 are formed
-            // in doubles.  Rare: a few pairs of each particle.
-            double v[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) v[k] = fx_to_double(V.w[k], V.e - 61 + 1023);
-            const double y2 = fx_to_double((int64_t)t.y2, -60 - 2 * t.g + 1023);
-            const double rv = fma(r[0], v[0], fma(r[1], v[1], r[2] * v[2]));
-            const double al = rv * y2;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) w1[k] = fma(-3.0 * al, r[k], v[k]);
-            if constexpr (kOrder6) {
-                double a[3];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) a[k] = fx_to_double(A.w[k], A.e - 61 + 1023);
-                const double w = fma(v[0], v[0], fma(v[1], v[1], fma(v[2], v[2],
-                                 fma(r[0], a[0], fma(r[1], a[1], r[2] * a[2])))));
-                const double be3 = 3.0 * fma(al, al, w * y2);
-#pragma unroll
-                for (int k = 0; k < 3; ++k) w2[k] = fma(-be3, r[k], fma(-6.0 * al, w1[k], a[k]));
-            }
-        } else {
-            const FxS Y2 = fx_split((int64_t)t.y2);
-            const FxW1 u = fx_w1(Rs, Vs, V.w, t, Y2, i.K);
-            int64_t x2[3];
-            int base1 = V.e - 59 + 1023, base2 = 0;
-            uint32_t high = min(fx_high(u.w[0]), min(fx_high(u.w[1]), fx_high(u.w[2])));
-            if constexpr (kOrder6) {
-                int ez;
-                fx_w2(Rs, R.e, Vs, V.e, A, t, Y2, u, x2, ez, i.K);
-                base2 = min(ez - R.e, 900) - 52 + 1023;
-                high = min(high, min(fx_high(x2[0]), min(fx_high(x2[1]), fx_high(x2[2]))));
-            }
-            if (high != 0) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    w1[k] = fx_to_double_high(u.w[k], base1);
-                    if constexpr (kOrder6) w2[k] = fx_to_double_high(x2[k], base2);
-                }
-            } else {  // a component below 2^-30 of its vector's scale (or zero)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    w1[k] = fx_to_double(u.w[k], base1);
-                    if constexpr (kOrder6) w2[k] = fx_to_double(x2[k], base2);
-                }
-            }
-        }
+        for (int k = 0; k < 3; ++k) o.r[k] = fma_rn_f64(i.x[k], i.m1, jj.x[k]);
+        FxC3 D[2] = {};  // v, a
+        int top[2] = {0, 0};
+        const FxP3 pj[2] = {jfx_v(jj), jfx_a(jj)}, pi[2] = {i.v, i.a};
+        fx_differences<kOrder6 ? 2 : 1>(pj, pi, D, top);
+        c.fv = max(c.fv, top[0]);
+        if constexpr (kOrder6) c.fa = max(c.fa, top[1]);
+        fx_vectors<kOrder6>(o.r, D[0], D[1], max(top[0], top[1]), i.eps_x, i.emin, i.K, o.t, o.w1, o.w2);
     }
     template <bool kOrder6>
     static __device__ __forceinline__ void pair(const I &i, const J &jj, bool self, Acc &c) {
@@ -223,7 +159,7 @@ struct Prec<NB_FP64> {
         // velocity jerk and snap, an acceleration the snap
         const double nan = __hiloint2double(0x7ff80000, 0);
         const bool bad_x = !(isfinite(c.a[0]) && isfinite(c.a[1]) && isfinite(c.a[2]));
-        const bool bad_v = bad_x || max(c.fv, i.ev) >= kFxBad, bad_a = bad_v || max(c.fa, i.ea) >= kFxBad;
+        const bool bad_v = bad_x || c.fv >= 0x7ff, bad_a = bad_v || c.fa >= 0x7ff;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             o[k] = bad_x ? nan : c.a[k];

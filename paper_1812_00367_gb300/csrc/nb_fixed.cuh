@@ -1,22 +1,21 @@
-// nb_fixed.cuh -- block fixed-point arithmetic of the FP64 pair terms.
+// nb_fixed.cuh -- fixed-point arithmetic of the FP64 pair terms.
 //
 // GB300 retires 2 FP64 lanes per clock and SM, but 64 lanes of IMAD.WIDE
 // (32 x 32 -> 64 bits, 64-bit addend), 64 of shifts and logic and 128 of FP32
 // (measured).  One FP64 instruction therefore costs as much as 32 integer
-// ones, and a 62 x 62 bit product is three IMAD.WIDE.  The pair terms keep the
+// ones, and a 62 x 62 bit product is four IMAD.WIDE.  The pair terms keep the
 // FP64 pipe for what needs its range per particle (the coordinate differences
-// and the nine running sums) and evaluate the rest on the integer pipe: the
-// three vectors r, v, a of a pair are block fixed-point numbers (three signed
-// 62-bit integers with one exponent, taken from the largest component), dot
-// products are sums of integer products, the reciprocal square root is an SFU
-// seed with one third-order step on integers, and w1, w2, q return to doubles
-// by a shift.
+// and the nine running sums) and evaluate the rest on the integer pipe: every
+// component of r, v and a of a pair is a 62-bit integer with an exponent of its
+// own (fx_vectors), the reciprocal square root is an SFU seed with one
+// third-order step on integers, and w1, w2, q return to doubles by a shift.
 //
-// Accuracy (relative to a vector's norm, rms over pairs of any scale, u =
-// 2^-53; CPU test): acceleration term 0.4-0.5 u, jerk 0.6-0.8 u, snap 0.8-1.5
-// u, against 1.7 u, 2.2-2.9 u and 2.8-4.8 u of the same terms in doubles.  A
-// component far below its vector's largest one is exact to 2^-58 of that one,
-// not to its own size; a component that vanishes stays zero.
+// Accuracy (u = 2^-53; CPU tests).  Relative to a vector's norm, rms over pairs
+// of any scale: acceleration term 0.4-0.5 u, jerk 0.6-0.8 u, snap 0.6-0.9 u,
+// against 1.7 u, 2.2-2.9 u and 2.8-4.8 u of the same terms in doubles.  Each
+// component relative to its own summands, in systems thin along an axis down to
+// 1e-12, chains, bulk motion: 0.4-0.7 u against 1.1-2.9 u in doubles.  Range: as
+// the doubles', except that a component of jerk or snap below 1e-285 is zero.
 //
 // The functions run on the host too (the check of the arithmetic against long
 // double is a CPU test); there the SFU seed is a rounded reciprocal root.
@@ -34,7 +33,7 @@
 
 namespace nb {
 
-// A vector of three: component k is w[k] 2^(e - 61), |w[k]| < 2^62.
+// A vector of three with one exponent: component k is w[k] 2^(e - 61), |w[k]| < 2^62.
 struct Fx3 {
     int64_t w[3];
     int32_t e;
@@ -44,7 +43,7 @@ struct FxS {
     int32_t h, l;
 };
 
-// Exponents of the stored blocks lie in [kFxMinExp, kFxMaxExp]; a block with a
+// Block forms (fx_pack): exponents lie in [kFxMinExp, kFxMaxExp]; a block with a
 // non-finite component (or one beyond 2^kFxMaxExp) carries kFxBad and turns
 // the sums that use it into NaN.
 constexpr int kFxMinExp = -900;
@@ -171,6 +170,14 @@ NB_HD uint64_t fx_madu(uint32_t a, uint32_t b, uint64_t c) {
     return fx_mulu(a, b) + c;
 #endif
 }
+NB_HD int32_t fx_max3(int32_t a, int32_t b, int32_t c) {
+    const int32_t m = a > b ? a : b;
+    return m > c ? m : c;
+}
+NB_HD uint32_t fx_min3(uint32_t a, uint32_t b, uint32_t c) {
+    const uint32_t m = a < b ? a : b;
+    return m < c ? m : c;
+}
 // The factors 1 and 2 as run-time values: x.hi is added to a 64-bit sum by
 // one IMAD.WIDE with them, where a constant factor would be turned into a
 // sign extension and a carry chain (three instructions).
@@ -191,6 +198,11 @@ constexpr int64_t kFxHalf = (int64_t)1 << 31;
 NB_HD int64_t fx_mulhi(FxS a, FxS b, FxK K) {
     const int64_t c = fx_mad(a.l, b.h, fx_mad(a.h, b.l, kFxHalf));
     return fx_mad(fx_hi(c), K.one, fx_mul(a.h, b.h));
+}
+// a^2 / 2^64, as fx_mulhi
+NB_HD int64_t fx_sqrhi(FxS a, FxK K) {
+    const int64_t c = fx_mad(a.h, a.l, kFxHalf);
+    return fx_mad(fx_hi(c), K.two, fx_mul(a.h, a.h));
 }
 // a b / 2^64 for unsigned factors of at most 2^63, floor to within two units
 NB_HD uint64_t fx_mulhi_u(uint64_t a, uint64_t b, FxK K) {
@@ -218,7 +230,11 @@ NB_HD int64_t fx_norm2(const FxS a[3], FxK K) {
     return fx_mad(fx_hi(c), K.two, h);
 }
 
-// ------------------------------------------------------------- pack (stored)
+// ------------------------------------------------ vectors with one exponent
+// fx_decode, fx_root and the conversions serve the kernels; fx_pack,
+// fx_diff_norm, fx_inside, fx_dot, fx_w1 and fx_w2 are the pair term with one
+// exponent for a vector, which the CPU check of the arithmetic compares: as exact
+// as the kernels' against a vector's norm, not component by component.
 // A vector of doubles as integers of at most 61 bits (component k is
 // w[k] 2^(e - 60)): exact for components down to 2^-8 of the largest,
 // below that cut at 2^-60 of it.
@@ -448,6 +464,188 @@ NB_HD void fx_w2(const FxS R[3], int er, const FxS V[3], int ev, const Fx3 &A, c
         int64_t h = fx_mad(a3.h, w1.h, fx_sar(A.w[k], da + 9));
         h = fx_mad(b3.h, R[k].h, h);
         w2[k] = fx_mad(fx_hi(c2), K.one, fx_mad(fx_hi(c1), K.one, h));
+    }
+}
+
+// ------------------------------------- a pair's vectors, component by component
+// The pair term of the kernels.  Every component of r, v and a has an exponent of
+// its own, every product of a dot is aligned to the largest of the dot's products
+// only, and w1_k, w2_k are sums of products of normalised integers aligned to the
+// largest of their own summands.  Each component of jerk and snap is therefore at
+// least as exact against its own summands (|v_k| + 3 |alpha r_k|, |a_k| + 6 |alpha
+// w1_k| + 3 |beta r_k|) as in doubles, however thin the system is along an axis.
+// With one exponent for a vector a component 2^-k of its vector's norm had k - 5
+// bits less than in doubles (z / x = 1e-6: jerk z 2.9e-12 instead of 2.3e-16); the
+// exponents cost 130 of now 778 instructions a pair and warp (FP64, N = 65536, A =
+// 1000: 2.17 -> 2.51 ms; all, each pair once: 90.4 -> 97.4 ms).  Differences of v
+// and a in doubles instead of integers: 742 instructions and 18 FP64 ones instead
+// of 12, 2.68 and 110.6 ms, and less exact than doubles' exact difference allows.
+struct FxC3 {
+    int64_t w[3];  // component k is w[k] 2^(f[k] - 1023 - 61), 2^61 <= |w[k]| < 2^62, or 0
+    int32_t f[3];  // exponent fields (below 0: under the doubles' range)
+    int32_t e;     // the largest
+};
+// r from its doubles.  None of them is -0: the records hold no -0, so their
+// differences are none.
+NB_HD FxC3 fx_components(const double d[3]) {
+    FxC3 o;
+    for (int k = 0; k < 3; ++k) {
+        const uint32_t h = (uint32_t)((uint64_t)fx_d2bits(d[k]) >> 32), lo = (uint32_t)fx_d2bits(d[k]);
+        o.f[k] = (int32_t)((h >> 20) & 0x7ffu);
+        const uint32_t mh = o.f[k] == 0 ? 0u : (h & 0xfffffu) | 0x100000u;
+        // one's complement: a negative component is off by one unit, 2^-61
+        o.w[k] = (int64_t)((((uint64_t)mh << 32) | lo) << 9) ^ ((int64_t)(int32_t)h >> 31);
+    }
+    o.e = fx_max3(o.f[0], o.f[1], o.f[2]);
+    return o;
+}
+// A particle's velocity or acceleration as it is stored: component k is
+// w[k] 2^(f[k] - 1023 - 60), 2^60 <= |w[k]| < 2^61, or 0.
+struct FxP3 {
+    int64_t w[3];
+    int32_t f[3];  // exponent fields; 0x7ff: not finite
+};
+NB_HD FxP3 fx_pack_components(const double d[3]) {
+    FxP3 o;
+    for (int k = 0; k < 3; ++k) {
+        const int64_t b = fx_d2bits(d[k]);
+        o.f[k] = (int32_t)((uint64_t)b >> 52) & 0x7ff;
+        const int64_t m = o.f[k] == 0 ? 0 : (int64_t)((((uint64_t)b & 0xfffffffffffffull) | ((uint64_t)1 << 52)) << 8);
+        o.w[k] = b < 0 ? -m : m;
+    }
+    return o;
+}
+// Differences of kVecs stored vectors: exact where the doubles' would be rounded,
+// except below 2^-60 of the larger component.  top[q]: the largest stored field.
+template <int kVecs>
+NB_HD void fx_differences(const FxP3 *j, const FxP3 *i, FxC3 *o, int32_t *top) {
+    int m[kVecs][3];
+    uint32_t t[kVecs][3], low = 0xffffffffu;
+    for (int q = 0; q < kVecs; ++q) {
+        for (int k = 0; k < 3; ++k) {
+            m[q][k] = j[q].f[k] > i[q].f[k] ? j[q].f[k] : i[q].f[k];
+            o[q].w[k] = fx_sar(j[q].w[k], m[q][k] - j[q].f[k]) - fx_sar(i[q].w[k], m[q][k] - i[q].f[k]);  // < 2^62
+            t[q][k] = fx_high(o[q].w[k]);
+        }
+        low = low < t[q][0] ? low : t[q][0];
+        low = fx_min3(low, t[q][1], t[q][2]);
+        top[q] = fx_max3(m[q][0], m[q][1], m[q][2]);
+    }
+    if (low != 0) {
+        for (int q = 0; q < kVecs; ++q)
+            for (int k = 0; k < 3; ++k) {
+                const int n = fx_clz(t[q][k]) - 2;
+                o[q].w[k] = (int64_t)fx_shl((uint64_t)o[q].w[k], n);
+                o[q].f[k] = m[q][k] + 1 - n;
+            }
+    } else {  // a component below 2^-29 of the particles' own (or zero)
+        for (int q = 0; q < kVecs; ++q)
+            for (int k = 0; k < 3; ++k) {
+                const int64_t w = o[q].w[k];
+                const int n = (t[q][k] ? fx_clz(t[q][k]) : 32 + fx_clz((uint32_t)(w ^ (w >> 63)))) - 2;
+                o[q].w[k] = (int64_t)fx_shl((uint64_t)w, n);
+                o[q].f[k] = w == 0 ? -8192 : m[q][k] + 1 - n;
+            }
+    }
+    for (int q = 0; q < kVecs; ++q) o[q].e = fx_max3(o[q].f[0], o[q].f[1], o[q].f[2]);
+}
+// Fields below kFxLow stand for zero (results under 2^-900); terms whose
+// scale reaches kFxHigh may leave the doubles' range: fx_to_double_any.
+constexpr int kFxLow = 64, kFxHigh = 2030;
+// The same conversion for any w and any scale: zero at the bottom, infinity (or
+// no number) at the top.
+NB_HD double fx_to_double_any(int64_t w, int m) {
+    const int64_t s = w >> 63;
+    const uint64_t a = (uint64_t)(w ^ s);
+    if (a == 0 || m <= kFxLow) return 0.0;
+    const int n = (a >> 32) ? fx_clz((uint32_t)(a >> 32)) : 32 + fx_clz((uint32_t)a);
+    const uint64_t x = (fx_shl(a, n) >> 1) + 0x200;
+    const int e = m - 57 + 62 - n;
+    uint32_t hi = (uint32_t)(x >> 42) + ((uint32_t)(e > 2046 ? 2046 : e) << 20);
+    return fx_bits2d(hi | ((uint32_t)(s >> 32) & 0x80000000u), (uint32_t)(x >> 10));
+}
+// From the differences r, v, a (a in the 6th-order form only): the root t, w1 =
+// v - 3 alpha r and w2 = a - 6 alpha w1 - 3 beta r as doubles.  top: the largest
+// stored field of v and a.
+template <bool kOrder6>
+NB_HD void fx_vectors(const double r[3], const FxC3 &V, const FxC3 &A, int top, uint64_t eps_x,
+                      uint32_t emin_field, FxK K, FxRoot &t, double w1[3], double w2[3]) {
+    const FxC3 R = fx_components(r);
+    const int emin = (int)(emin_field >> 20);
+    const int er = R.e > emin ? R.e : emin;
+    FxS Rs[3], Vs[3];
+    {
+        FxS B[3];  // r as a block, for r^2
+        for (int k = 0; k < 3; ++k) B[k] = fx_split(fx_sar(R.w[k], er - R.f[k]));
+        t = fx_root(B, er - 1023, eps_x, emin_field, K);
+    }
+    for (int k = 0; k < 3; ++k) {
+        Rs[k] = fx_split(R.w[k]);
+        Vs[k] = fx_split(V.w[k]);
+    }
+    const FxS Y2 = fx_split((int64_t)t.y2);
+    // alpha = al 2^(ea - 60), al in +-[2^60, 2^61)
+    const int g0 = R.f[0] + V.f[0], g1 = R.f[1] + V.f[1], g2 = R.f[2] + V.f[2];
+    const int G = fx_max3(g0, g1, g2);
+    const int64_t rv = fx_sar(fx_mulhi(Rs[0], Vs[0], K), G - g0) + fx_sar(fx_mulhi(Rs[1], Vs[1], K), G - g1) +
+                       fx_sar(fx_mulhi(Rs[2], Vs[2], K), G - g2);  // units 2^(G - 58), below 2^61.6
+    int64_t al = fx_mulhi(fx_split(rv), Y2, K);                      // units 2^(G - 2 er + s - 58), below 2^59.6
+    const int na = fx_clz(fx_high(al)) - 3;
+    al = (int64_t)fx_shl((uint64_t)al, na);
+    const int ea = G - 2 * er + t.s + 2 - na;
+    const FxS a3 = fx_split(-3 * al);
+    int64_t u1[3];  // w1_k = u1[k] 2^(m1[k] - 1023 - 57)
+    int m1[3];
+    for (int k = 0; k < 3; ++k) {
+        const int ep = ea + R.f[k];
+        m1[k] = fx_max3(ep, V.f[k], kFxLow);
+        u1[k] = fx_sar(V.w[k], 4 + m1[k] - V.f[k]) + fx_sar(fx_mulhi(a3, Rs[k], K), m1[k] - ep);
+    }
+    uint32_t high = fx_min3(fx_high(u1[0]), fx_high(u1[1]), fx_high(u1[2]));
+    int64_t u2[3];
+    int m2[3];
+    if (kOrder6) {
+        FxS As[3];
+        for (int k = 0; k < 3; ++k) As[k] = fx_split(A.w[k]);
+        // v.v + r.a, its six products aligned to the largest
+        const int h0 = R.f[0] + A.f[0], h1 = R.f[1] + A.f[1], h2 = R.f[2] + A.f[2];
+        const int H = fx_max3(h0, h1, h2);
+        const int ez = 2 * V.e > H ? 2 * V.e : H;
+        int64_t w = fx_sar(fx_mulhi(Rs[0], As[0], K), ez - h0) + fx_sar(fx_mulhi(Rs[1], As[1], K), ez - h1) +
+                    fx_sar(fx_mulhi(Rs[2], As[2], K), ez - h2);
+        for (int k = 0; k < 3; ++k) w += fx_sar(fx_sqrhi(Vs[k], K), ez - 2 * V.f[k]);
+        // units 2^(ez - 58), below 2^62.6; 3 zeta in units 2^(eZ - 58)
+        const int64_t z3 = 3 * fx_mulhi(fx_split(w), Y2, K);
+        const int eZ = ez - 2 * er + t.s;
+        const int64_t aa3 = fx_mulhi(a3, fx_split(al), K);  // -3 alpha^2, units 2^(2 ea - 56)
+        const int eA = 2 * ea + 2;
+        const int mB = eA > eZ ? eA : eZ;
+        int64_t b3 = fx_sar(aa3, mB - eA + 1) - fx_sar(z3, mB - eZ + 1);  // -3 beta, units 2^(mB - 57)
+        const int nb = fx_clz(fx_high(b3)) - 2;
+        b3 = (int64_t)fx_shl((uint64_t)b3, nb);  // below 2^62, units 2^(mB - 57 - nb)
+        const FxS B3 = fx_split(b3);
+        const int eb = mB + 3 - nb;
+        for (int k = 0; k < 3; ++k) {
+            const int f1 = ea + m1[k] + 5, f2 = eb + R.f[k];
+            const int m = m2[k] = fx_max3(f1, f2, A.f[k] > kFxLow ? A.f[k] : kFxLow);
+            u2[k] = fx_sar(A.w[k], 4 + m - A.f[k]) + fx_sar(fx_mulhi(a3, fx_split(u1[k]), K), m - f1) +
+                    fx_sar(fx_mulhi(B3, Rs[k], K), m - f2);
+        }
+        top = top > ez - er ? top : ez - er;
+        high = fx_min3(high, fx_high(u2[0]), fx_high(u2[1]));
+        high = high < fx_high(u2[2]) ? high : fx_high(u2[2]);
+    }
+    high = top > kFxHigh ? 0u : high;
+    if (high != 0) {
+        for (int k = 0; k < 3; ++k) {
+            w1[k] = fx_to_double_high(u1[k], m1[k] - 57);
+            if (kOrder6) w2[k] = fx_to_double_high(u2[k], m2[k] - 57);
+        }
+    } else {  // a component below 2^-26 of its summands' scale (or zero), or the range's ends
+        for (int k = 0; k < 3; ++k) {
+            w1[k] = fx_to_double_any(u1[k], m1[k]);
+            if (kOrder6) w2[k] = fx_to_double_any(u2[k], m2[k]);
+        }
     }
 }
 

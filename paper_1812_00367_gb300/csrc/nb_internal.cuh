@@ -84,37 +84,46 @@ constexpr int kPrecPot = 64;
 struct alignas(16) J64 {
     double2 q[5];  // (x,y) (z,m) (vx,vy) (vz,ax) (ay,az)
 };
-// FP64 evaluation: the position as doubles, velocity and acceleration as
-// block fixed-point vectors (component k is w[k] 2^(e - 60), nb_fixed.cuh),
-// the mass as a 63-bit integer (|m| = mm 2^(em - 62)) and as a float pair.
+// FP64 evaluation: the position as doubles (none -0, nb_fixed.cuh), velocity and
+// acceleration as integers with an exponent field each (FxP3), the mass as a
+// 63-bit integer (|m| = mm 2^(em - 62)) and as a float pair.  112 bytes: lanes
+// that share an i read records side by side, eight of them in different banks.
 struct alignas(16) JFX {
     double x[3];
     uint64_t mm;
     int64_t v[3], a[3];
     float2 mf;      // (m_hi, m_lo) for the potential
-    int32_t eva;    // exponents: ev in the low half, ea in the high half
+    uint32_t f[3];  // exponent fields, two in a word: vx vy, vz ax, ay az
     int32_t ems;    // 2 em + (m < 0)
 };
-static_assert(sizeof(JFX) == 96, "JFX layout");
-__device__ __forceinline__ int jfx_ev(const JFX &j) { return (int)(short)j.eva; }
-__device__ __forceinline__ int jfx_ea(const JFX &j) { return j.eva >> 16; }
+static_assert(sizeof(JFX) == 112, "JFX layout");
 __device__ __forceinline__ int jfx_em(const JFX &j) { return j.ems >> 1; }
 __device__ __forceinline__ uint32_t jfx_sign(const JFX &j) { return (uint32_t)j.ems << 31; }
+__device__ __forceinline__ FxP3 jfx_v(const JFX &j) {
+    return FxP3{{j.v[0], j.v[1], j.v[2]},
+                {(int)(j.f[0] & 0xffffu), (int)(j.f[0] >> 16), (int)(j.f[1] & 0xffffu)}};
+}
+__device__ __forceinline__ FxP3 jfx_a(const JFX &j) {
+    return FxP3{{j.a[0], j.a[1], j.a[2]},
+                {(int)(j.f[1] >> 16), (int)(j.f[2] & 0xffffu), (int)(j.f[2] >> 16)}};
+}
 __device__ __forceinline__ JFX jfx_pack(const double x[3], const double v[3], const double a[3],
                                         double m) {
     JFX w;
-    const Fx3 fv = fx_pack(v[0], v[1], v[2]), fa = fx_pack(a[0], a[1], a[2]);
+    const FxP3 pv = fx_pack_components(v), pa = fx_pack_components(a);
     for (int k = 0; k < 3; ++k) {
-        w.x[k] = x[k];
-        w.v[k] = fv.w[k];
-        w.a[k] = fa.w[k];
+        w.x[k] = x[k] + 0.0;  // -0 + 0 = +0
+        w.v[k] = pv.w[k];
+        w.a[k] = pa.w[k];
     }
+    w.f[0] = (uint32_t)pv.f[0] | ((uint32_t)pv.f[1] << 16);
+    w.f[1] = (uint32_t)pv.f[2] | ((uint32_t)pa.f[0] << 16);
+    w.f[2] = (uint32_t)pa.f[1] | ((uint32_t)pa.f[2] << 16);
     int em;
     uint32_t sign;
     fx_pack_mass(m, w.mm, em, sign);
     const float hi = (float)m;
     w.mf = make_float2(hi, (float)(m - (double)hi));
-    w.eva = (int32_t)(((uint32_t)fa.e << 16) | ((uint32_t)fv.e & 0xffffu));
     w.ems = 2 * em + (int32_t)(sign >> 31);
     return w;
 }

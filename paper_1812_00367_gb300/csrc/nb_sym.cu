@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
             T::finish(me, acc, o);
             // a velocity or acceleration that is not finite spoils every other
             // particle's sums: the reduction is told
-            const int bad = max(acc.fv, me.ev) >= kFxBad ? 3 : (max(acc.fa, me.ea) >= kFxBad ? 2 : 0);
+            const int bad = acc.fv >= 0x7ff ? 3 : (acc.fa >= 0x7ff ? 2 : 0);
             if (bad) atomicOr(L.bad, bad);
         } else if constexpr (P == NB_EX) {
             T::finish(acc, nullptr, 0, o);
