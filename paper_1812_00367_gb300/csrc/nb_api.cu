@@ -297,38 +297,29 @@ nb_status eval_sym(nb_ctx *ctx, const Dev &d, int mode, const int32_t *active, d
     return NB_OK;
 }
 
-// Whether whole-cluster evaluations take each pair once, and their scratch: one
-// cluster of enough particles (N >= 7,800 or so) whose columns' partial sums
-// stay within kSymMaxBytes (N <= 113,000 for the pair terms of FP64 and EX,
-// 357,000 for the potential).  NB_NO_STREAMK keeps the split-item sums everywhere.
-nb_status setup_sym(nb_ctx *ctx) {
-    if (ctx->nc != 1 || (ctx->p.flags & NB_NO_STREAMK)) return NB_OK;
+// Whether whole-cluster evaluations take each pair once: one cluster of enough
+// particles (N >= 7,800 or so; up to kSymMaxUnits).  Their scratch is that of the
+// other evaluations (d.partial), which run before or after them on the context's
+// stream.  NB_NO_STREAMK keeps the split-item sums everywhere.
+void setup_sym(nb_ctx *ctx) {
+    if (ctx->nc != 1 || (ctx->p.flags & NB_NO_STREAMK)) return;
     SymLaunch &L = ctx->sym;
     const int64_t ntj = cdiv(ctx->n, kTJ), units = sym_units(ntj);
     const bool order4 = ctx->d.order == 4;
     auto usable = [&](int mode) {
-        ctx->sym_grid[mode] = sym_resident(ctx->p.precision, mode) * ctx->sm_count;
-        return ctx->sym_grid[mode] > 0 && units >= kSymMinUnits * ctx->sym_grid[mode];
+        const int64_t grid = (int64_t)sym_resident(ctx->p.precision, mode) * ctx->sm_count;
+        ctx->sym_grid[mode] = (int)grid;
+        return grid > 0 && units >= kSymMinUnits * grid &&
+               sym_bands(ntj, grid, sym_values(mode), ctx->d.partial_cap) > 0;
     };
-    ctx->sym_force = (ctx->p.precision == NB_FP64 || ctx->p.precision == NB_EX) && units * kSymUnitBytes <= kSymMaxBytes &&
+    ctx->sym_force = (ctx->p.precision == NB_FP64 || ctx->p.precision == NB_EX) && units <= kSymMaxUnits &&
                      (order4 ? usable(kModeOut4) && usable(kModeInit4)
                              : usable(kModeOut) && usable(kModeInit1) && usable(kModeInit2));
-    ctx->sym_pot = units * kSymUnitBytes / 10 <= kSymMaxBytes && usable(kModePot);
-    if (!ctx->sym_force && !ctx->sym_pot) return NB_OK;
+    ctx->sym_pot = units <= 10 * kSymMaxUnits && usable(kModePot);
     L.cluster = 0;
     L.ntj = (int32_t)ntj;
     L.n = ctx->n;
-    L.units = units;
-    const int64_t grid = 8LL * ctx->sm_count;  // at least any mode's
-    if (dalloc(ctx, &L.jpart, (size_t)(units * kTJ * (ctx->sym_force ? 10 : 1))) != cudaSuccess ||
-        dalloc(ctx, &L.ipart, (size_t)((sym_rows(ntj) + grid) * 10 * kTPB)) != cudaSuccess ||
-        dalloc(ctx, &L.gate, 2) != cudaSuccess) {
-        cudaGetLastError();  // no room: the one-sided evaluation does without
-        ctx->sym_force = ctx->sym_pot = false;
-        return NB_OK;
-    }
     L.bad = L.gate + 1;
-    return NB_OK;
 }
 
 // The potential of every particle on the FP64 predicted state.
@@ -553,6 +544,7 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
     const int64_t max_groups = d.partial_cap / kGrpStride + 1;
     ALLOC(d.grp_cnt, max_groups);
     ALLOC(ctx->d_ctl, 1);
+    ALLOC(ctx->sym.gate, 2);
     d.ctr_steps = &ctx->d_ctl->steps;
     d.ctr_inter = &ctx->d_ctl->inter;
     d.ctr_underflow = &ctx->d_ctl->underflow;
@@ -574,11 +566,7 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
     ctx->d_pot.precision = NB_FP64;
     ctx->d_pot.grid_eval = ctx->grid_pot;
 
-    if (nb_status ss = setup_sym(ctx); ss != NB_OK) {
-        g_init_err = ctx->err;
-        nb_free(ctx);
-        return ss;
-    }
+    setup_sym(ctx);
     default_table(ctx);
     if (p->flags & NB_TIME_EVAL) {
         ctx->ev.resize(2 * (kMultiSteps + 1));

@@ -25,8 +25,9 @@
 // Order of the sums: units (row, column) are cut into equal ranges over a fixed
 // grid (as stream-K); each range leaves one partial per row it touches and each
 // unit one per column particle, in slots of its own; k_sym_reduce adds them in
-// row order.  No atomics: results are reproducible.  A column's partials take
-// 5 KB a unit (1.3 GB at N = 65536), so the form is used up to kSymMaxBytes.
+// row order.  No atomics: results are reproducible.  The units are taken in
+// bands whose columns' partials fit the evaluation's scratch (199 MB; 8 bands at N
+// = 65536), one launch of each kernel a band.
 #include "nb_eval.cuh"
 #include "nb_sym.cuh"
 
@@ -154,8 +155,8 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
         for (int s = 0; s < kStages; ++s) mbar_init(&S.bar[s], 1);
         S.fail = 0;
         fence_mbar_init();
-        S.u = sk_begin(L.units, gridDim.x, blockIdx.x);
-        S.u_end = sk_begin(L.units, gridDim.x, blockIdx.x + 1);
+        S.u = L.u0 + sk_begin(L.units, gridDim.x, blockIdx.x);
+        S.u_end = L.u0 + sk_begin(L.units, gridDim.x, blockIdx.x + 1);
     }
     uint32_t phase = 0, pending = 0;  // as in k_eval
     for (;;) {
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
                 }
             }
             if (!own_cols) {  // the warps' sums of the tile's particles, in warp order
-                double *out = L.jpart + (S.u + (tt - tb)) * (int64_t)(NV * kTJ);
+                double *out = L.jpart + (S.u - L.u0 + (tt - tb)) * (int64_t)(NV * kTJ);
                 for (int e = tid; e < NV * kTJ; e += kTPB) {
                     const int q = e / kTJ, k = e % kTJ;
                     double sum = 0.0;
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
         } else {
             T::finish(acc, o);
         }
-        double *part = L.ipart + ((int64_t)row + blockIdx.x) * (10 * kTPB) + tid;
+        double *part = L.ipart + (row - L.row0 + blockIdx.x) * (10 * kTPB) + tid;
 #pragma unroll
         for (int q = 0; q < 10; ++q) part[q * kTPB] = o[q];
         __syncthreads();
@@ -281,36 +282,49 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
     }
 }
 
-// One j-tile's particles: the pieces of their own row, then the shares from the
-// rows above, in row order.
+// One j-tile's particles: what the earlier bands gave, the band's pieces of their
+// own row, then the shares from the band's rows above, in row order.
 constexpr int kSymRedTPB = 320;
 template <int P, int MODE>
 __global__ void __launch_bounds__(kSymRedTPB) k_sym_reduce(const Dev d, const SymLaunch L, int grid_sym) {
     constexpr int NV = sym_nv<MODE>();
     __shared__ double sums[10][kTJ];
     if (L.gate && *L.gate != 0) return;
-    const int tile = blockIdx.x, row = tile / 2, il0 = (tile & 1) * kTJ;
-    const long long u0 = sym_first(row, L.ntj), u1 = sym_first(row + 1, L.ntj);
-    const long long k0 = sk_owner(L.units, grid_sym, u0), k1 = sk_owner(L.units, grid_sym, u1 - 1);
+    const int tile = (int)(2 * L.row0) + blockIdx.x, row = tile / 2, il0 = (tile & 1) * kTJ;
+    const long long u1 = L.u0 + L.units, f0 = sym_first(row, L.ntj), f1 = sym_first(row + 1, L.ntj);
+    const bool last = f1 <= u1;  // the particles' own row ends here: nothing more to come
+    long long k0 = 0, k1 = -1;
+    if (f0 < u1) {
+        k0 = sk_owner(L.units, grid_sym, max(f0, (long long)L.u0) - L.u0);
+        k1 = sk_owner(L.units, grid_sym, min(f1, u1) - L.u0 - 1);
+    }
+    // rows above with their unit of this column in the band: the first and the
+    // last of them may be just outside
+    auto unit = [&](long long r) { return sym_first(r, L.ntj) + (tile - 2 * r); };
+    int r0 = (int)L.row0, r1 = min(row, sym_row(u1 - 1, L.ntj) + 1);
+    if (r0 < r1 && unit(r0) < L.u0) ++r0;
+    if (r0 < r1 && unit(r1 - 1) >= u1) --r1;
+    double *so_far = L.sums + (int64_t)tile * (NV * kTJ);
     for (int e = threadIdx.x; e < NV * kTJ; e += kSymRedTPB) {
         const int v = e / kTJ, k = e % kTJ, q = sym_q<MODE>(v);
-        double sum = 0.0;
+        double sum = L.u0 > 0 ? so_far[e] : 0.0;
         for (long long c = k0; c <= k1; ++c)
-            sum += __ldcs(L.ipart + (row + c) * (10 * kTPB) + q * kTPB + il0 + k);
+            sum += __ldcs(L.ipart + (row - L.row0 + c) * (10 * kTPB) + q * kTPB + il0 + k);
         double above = 0.0;
-        for (int r = 0; r < row; r += 8) {
+        for (int r = r0; r < r1; r += 8) {
             double t[8];
 #pragma unroll
             for (int x = 0; x < 8; ++x)
-                t[x] = r + x < row ? __ldcs(L.jpart + (sym_first(r + x, L.ntj) + (tile - 2LL * (r + x))) *
-                                                          (int64_t)(NV * kTJ) + e)
-                                   : 0.0;
+                t[x] = r + x < r1 ? __ldcs(L.jpart + (unit(r + x) - L.u0) * (int64_t)(NV * kTJ) + e) : 0.0;
 #pragma unroll
             for (int x = 0; x < 8; ++x) above += t[x];
         }
         // FP64's shares of the potential are sums of m y, its sum carries the sign
-        sums[q][k] = q == 9 && P != NB_EX ? sum - above : sum + above;
+        sum = q == 9 && P != NB_EX ? sum - above : sum + above;
+        if (!last) so_far[e] = sum;
+        sums[q][k] = sum;
     }
+    if (!last) return;
     __syncthreads();
     const int64_t il = (int64_t)tile * kTJ + threadIdx.x;
     if (threadIdx.x < kTJ && il < L.n) {
@@ -342,13 +356,26 @@ __global__ void k_sym_check(const int32_t *active, int64_t n, int64_t off, int *
 }
 
 template <int P, int MODE>
-cudaError_t go(const Dev &d, const SymLaunch &L, int grid, cudaStream_t st) {
+cudaError_t go(const Dev &d, const SymLaunch &L0, int grid, cudaStream_t st) {
     constexpr size_t smem = sizeof(SymSmem<P, MODE>);
-    k_sym<P, MODE><<<grid, kTPB, smem, st>>>(d, L);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_sym_reduce<P, MODE><<<L.ntj, kSymRedTPB, 0, st>>>(d, L, grid);
-    return cudaGetLastError();
+    constexpr int NV = sym_nv<MODE>();
+    SymLaunch L = L0;
+    const int64_t bands = sym_bands(L.ntj, grid, NV, d.partial_cap);
+    if (bands <= 0) return cudaErrorInvalidValue;
+    L.ipart = d.partial;
+    L.sums = L.ipart + sym_piece_doubles(L.ntj, grid);
+    L.jpart = L.sums + sym_sum_doubles(L.ntj, NV);
+    for (int64_t b = 0; b < bands; ++b) {
+        L.u0 = sym_band_first(L.ntj, grid, bands, b);
+        L.units = sym_band_first(L.ntj, grid, bands, b + 1) - L.u0;
+        L.row0 = sym_row(L.u0, L.ntj);
+        k_sym<P, MODE><<<grid, kTPB, smem, st>>>(d, L);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        k_sym_reduce<P, MODE><<<(unsigned)(L.ntj - 2 * L.row0), kSymRedTPB, 0, st>>>(d, L, grid);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 template <int P, int MODE>
 int resident() {  // CTAs per SM, after raising the shared-memory limit
@@ -379,6 +406,7 @@ cudaError_t launch_sym(const Dev &d, int mode, const SymLaunch &L, int grid, cud
     default: return cudaErrorInvalidValue;
     }
 }
+int sym_values(int mode) { return mode == kModePot ? 1 : (uses_order4_terms(mode) ? 7 : 10); }
 int sym_resident(int precision, int mode) {
     if (mode == kModePot) return resident<kPrecPot, kModePot>();
     if (precision != NB_FP64 && precision != NB_EX) return 0;

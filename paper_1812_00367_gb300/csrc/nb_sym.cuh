@@ -22,24 +22,52 @@ __host__ __device__ inline int sym_row(int64_t u, int64_t ntj) {
 }
 
 // Used from kSymMinUnits units per CTA (below, the triangle's cut is too
-// coarse) while the columns' partials fit kSymMaxBytes.
+// coarse) up to the sizes it was measured at: kSymMaxUnits units (N = 113,000) for
+// the pair terms, ten times as many (N = 357,000) for the potential.
 constexpr int64_t kSymMinUnits = 6;
-constexpr int64_t kSymMaxBytes = 4000000000ll;
-constexpr int64_t kSymUnitBytes = 10 * kTJ * (int64_t)sizeof(double);
+constexpr int64_t kSymMaxUnits = 781250;
+
+// Scratch: the evaluation's partial sums (Dev::partial), which nothing else uses
+// meanwhile.  The units are taken in bands whose columns' partials fit there: they
+// are 64 doubles a unit and value (5 KB, 1.3 GB at N = 65536 for all units at
+// once).  Besides them it holds the rows' pieces and, between bands, the sums so
+// far.  In doubles, for nv values on a grid of `grid` CTAs:
+__host__ __device__ inline int64_t sym_piece_doubles(int64_t ntj, int64_t grid) {
+    return (sym_rows(ntj) + grid) * 10 * kTPB;
+}
+__host__ __device__ inline int64_t sym_sum_doubles(int64_t ntj, int64_t nv) { return ntj * nv * kTJ; }
+// Bands (0: the scratch is too small).  Their units are multiples of the grid, but
+// for the last one's: a CTA's share of all bands together is then that of one
+// launch (bands of whole rows left shares of 55 and 56 units: N = 65536 98.5 against
+// 97.9 ms).  Every
+// band has at least as many units as CTAs.
+__host__ __device__ inline int64_t sym_bands(int64_t ntj, int64_t grid, int64_t nv, int64_t cap) {
+    const int64_t fit = (cap - sym_piece_doubles(ntj, grid) - sym_sum_doubles(ntj, nv)) / (nv * kTJ);
+    const int64_t most = fit / grid;  // units a CTA
+    return fit < 0 || most < kSymMinUnits ? 0 : cdiv(cdiv(sym_units(ntj), grid), most);
+}
+// First unit of band b (b = bands: the number of units).
+__host__ __device__ inline int64_t sym_band_first(int64_t ntj, int64_t grid, int64_t bands, int64_t b) {
+    return b >= bands ? sym_units(ntj) : grid * (cdiv(sym_units(ntj), grid) * b / bands);
+}
 
 struct SymLaunch {
     int32_t cluster;
     int32_t ntj;      // columns
-    int64_t n, units;
-    double *jpart;    // [units][values][64]
-    double *ipart;    // [rows + grid][10][128]; slot row + CTA
+    int64_t n;
+    int64_t u0, units, row0;  // the band: its first unit, its units, the row of the first
+    double *jpart;    // [units of the band][values][64]
+    double *ipart;    // [rows + grid][10][128]; slot row - row0 + CTA
+    double *sums;     // [ntj][values][64]: what the earlier bands add up to
     int *gate;        // run only while *gate == 0 (NULL: always)
     int *bad;         // bit 0: a velocity, bit 1: an acceleration is not finite
     double *out;      // mode out: [10][n]
 };
 
 cudaError_t launch_sym_check(const int32_t *active, int64_t n, int64_t off, int *gate, cudaStream_t st);
+// All bands, in the scratch d.partial.  L: cluster, ntj, n, gate, bad, out.
 cudaError_t launch_sym(const Dev &d, int mode, const SymLaunch &L, int grid, cudaStream_t st);
+int sym_values(int mode);  // values per particle in the partials
 int sym_resident(int precision, int mode);  // CTAs per SM (0: not available)
 
 }  // namespace nb
