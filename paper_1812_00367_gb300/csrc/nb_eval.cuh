@@ -704,6 +704,7 @@ struct EvalCfg<NB_FP32X> {
 // (doubles) per group counter: a group has at least six pieces of at least 40
 // doubles, so groups' first slots lie in different counters' ranges.
 constexpr int kTreePieces = 32;
+static_assert(6 * 10 * (kTPB / 32) >= kGrpStride, "groups' first slots must not share a counter");
 // ... and the pieces times i's, below which the second level of counters costs
 // more than it spares (us, FP64: N = 10007, A = 16, 128 pieces of 4 i's: 26.9 ->
 // 25.3; N = 16384, A = 1, 128 pieces of one: 17.6 -> 18.7).

@@ -14,11 +14,12 @@ namespace nb {
 
 // ---------------------------------------------------------------- constants
 #ifndef NB_EVAL_TPB
-#define NB_EVAL_TPB 128       // threads per evaluation CTA (64, 128 or 256)
+#define NB_EVAL_TPB 128       // threads per evaluation CTA
 #endif
 constexpr int kTPB = NB_EVAL_TPB;
-static_assert(kTPB == 64 || kTPB == 128 || kTPB == 256, "evaluation CTA: 64, 128 or 256 threads");
 constexpr int kTJ = 64;        // j-particles per shared-memory tile
+// the whole-cluster evaluation's rows are two columns (nb_sym.cuh), its CTAs one row
+static_assert(kTPB == 2 * kTJ, "evaluation CTA: 128 threads");
 #ifndef NB_EVAL_STAGES
 #define NB_EVAL_STAGES 4
 #endif
