@@ -273,8 +273,12 @@ nb_status nb_get_counters(nb_ctx *ctx, nb_counters *out);
 /*
  * nb_autotune -- time the evaluation kernel for active-set sizes 1, 2, 4,
  * ... up to the largest cluster, over candidate (lanes per i, j-split)
- * choices, and install the fastest per size bucket.  cache_path: optional
- * file to read a previous table from / write the new one to (NULL: none).
+ * choices, and install the fastest per size bucket.  Timed is what the block
+ * steps of this context launch: stream-K ranges for one cluster, split items for
+ * a batch or with NB_NO_STREAMK.  cache_path: optional file to read a previous
+ * table from / write the new one to (NULL: none); a written table is read back by
+ * contexts of the same precision, order, grid and way of launching, one whose
+ * first line gives "nbtune <precision> <grid>" alone by any of the precision.
  * The state is not modified.  Errors: NB_ECUDA, NB_EINVAL.
  */
 nb_status nb_autotune(nb_ctx *ctx, const char *cache_path);

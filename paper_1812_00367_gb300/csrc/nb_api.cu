@@ -239,27 +239,26 @@ nb_status set_tend(nb_ctx *ctx, double t_end) {
     return NB_OK;
 }
 
+// The plan's split, reduced to what the partial sums have room for.
+int cap_split(const nb_ctx *ctx, const EvalPlan &p) {
+    const int64_t per_item = 10LL * (kTPB / p.gl);  // partial doubles per item
+    if (p.split > 1 && (int64_t)p.tiles * p.split * per_item > ctx->d.partial_cap)
+        return (int)std::max<int64_t>(1, ctx->d.partial_cap / (per_item * p.tiles));
+    return p.split;
+}
+
 // Plan a direct (host-driven) evaluation of n_active particles of one cluster.
 void plan_direct(const nb_ctx *ctx, int cluster, int32_t n_active, int &gl, int &split, int &tiles,
                  int &streamk, int64_t jtiles = -1) {
     const int b = 31 - __builtin_clz((unsigned)std::max(n_active, 1));
-    const PlanEntry e = ctx->table[b];
     const int64_t ncl = ctx->h_offsets[cluster + 1] - ctx->h_offsets[cluster];
     const int64_t ntj = jtiles >= 0 ? jtiles : cdiv(ncl, kTJ);  // j-tiles evaluated
-    gl = ctx->p.flags & NB_NO_STREAMK ? e.gl : sk_lanes(e.gl, n_active, ntj, ctx->grid_eval,
-                                                       ctx->p.precision);
-    tiles = (int)cdiv(n_active, kTPB / gl);
-    streamk = !(ctx->p.flags & NB_NO_STREAMK) &&
-              sk_use(tiles, kTPB / gl, ntj, ctx->grid_eval, ctx->d.partial_cap) ? 1 : 0;
-    if (streamk) {
-        split = 1;
-        return;
-    }
-    int64_t S = choose_split(tiles, ntj, e.target_items, ctx->grid_eval, ctx->p.precision);
-    const int64_t per_item = 10LL * (kTPB / gl);  // partial doubles per item
-    if (S > 1 && (int64_t)tiles * S * per_item > ctx->d.partial_cap)
-        S = std::max<int64_t>(1, ctx->d.partial_cap / (per_item * tiles));
-    split = (int)S;
+    const EvalPlan p = plan_eval(ctx->table[b], n_active, ntj, !(ctx->p.flags & NB_NO_STREAMK), ctx->grid_eval,
+                                 ctx->d.partial_cap, ctx->p.precision);
+    gl = p.gl;
+    tiles = p.tiles;
+    streamk = p.streamk;
+    split = cap_split(ctx, p);
 }
 nb_status eval_direct(nb_ctx *ctx, int cluster, const int32_t *active, int32_t n_active, double *out,
                       int gl, int split, int tiles, int streamk, int32_t jt0 = 0, int32_t jt1 = 0,
@@ -854,17 +853,25 @@ nb_status nb_sync(nb_ctx *ctx) {
 
 nb_status nb_autotune(nb_ctx *ctx, const char *cache_path) {
     if (!ctx) return fail(nullptr, NB_EINVAL, "nb_autotune: NULL context");
+    // whether the steps' planner may use stream-K ranges
+    const int tune_streamk = ctx->nc == 1 && !(ctx->p.flags & NB_NO_STREAMK) ? 1 : 0;
     // cached table?
     if (cache_path) {
         FILE *f = std::fopen(cache_path, "r");
         if (f) {
+            // header: precision and grid, and, since tables are timed for one
+            // way of launching, the order and whether stream-K ranges are used (a
+            // header without them: a table for any context of the precision)
             std::vector<PlanEntry> t(kBuckets);
-            int prec = -1, grid = -1, okc = 1;
-            if (std::fscanf(f, "nbtune %d %d", &prec, &grid) != 2) okc = 0;
-            for (int b = 0; okc && b < kBuckets; ++b)
-                if (std::fscanf(f, "%d %d", &t[b].gl, &t[b].target_items) != 2) okc = 0;
+            char line[128];
+            int prec = -1, grid = -1, order = -1, streamk = -1;
+            int got = std::fgets(line, sizeof line, f)
+                          ? std::sscanf(line, "nbtune %d %d %d %d", &prec, &grid, &order, &streamk) : 0;
+            for (int b = 0; got >= 2 && b < kBuckets; ++b)
+                if (std::fscanf(f, "%d %d", &t[b].gl, &t[b].target_items) != 2) got = 0;
             std::fclose(f);
-            if (okc && prec == ctx->p.precision) {
+            if (prec == ctx->p.precision &&
+                (got == 2 || (got == 4 && grid == ctx->grid_eval && order == ctx->d.order && streamk == tune_streamk))) {
                 ctx->table = t;
                 return upload_table(ctx);
             }
@@ -897,17 +904,22 @@ nb_status nb_autotune(nb_ctx *ctx, const char *cache_path) {
         float best = 1e30f;
         PlanEntry bestE = ctx->table[b];
         int reps = 2;
+        std::vector<EvalPlan> timed;         // different entries may come to the same launch
         for (int gl : gls) {
             if (A >= 4096 && gl > 2) continue;   // wide i-sets: j broadcast wins
             for (int64_t tg : targets) {
                 if (tg > ctx->cap_items / 2) continue;
-                ctx->table[b] = PlanEntry{gl, (int32_t)tg};
-                int g2, sp, tl, skm;
-                plan_direct(ctx, cmax, A, g2, sp, tl, skm);
+                EvalPlan pl = plan_eval(PlanEntry{gl, (int32_t)tg}, A, cdiv(ncl, kTJ), tune_streamk != 0, G,
+                                        ctx->d.partial_cap, ctx->p.precision);
+                pl.split = cap_split(ctx, pl);
+                if (std::any_of(timed.begin(), timed.end(), [&](const EvalPlan &q) {
+                        return q.gl == pl.gl && q.split == pl.split && q.streamk == pl.streamk; }))
+                    continue;
+                timed.push_back(pl);
                 float ms_best = 1e30f;
                 for (int rep = 0; rep < reps; ++rep) {
                     if ((e = cudaEventRecord(e0, ctx->stream)) != cudaSuccess) break;
-                    st = eval_direct(ctx, cmax, d_act, A, d_out, g2, sp, tl, skm);
+                    st = eval_direct(ctx, cmax, d_act, A, d_out, pl.gl, pl.split, pl.tiles, pl.streamk);
                     if (st != NB_OK) break;
                     if ((e = cudaEventRecord(e1, ctx->stream)) != cudaSuccess) break;
                     if ((e = cudaEventSynchronize(e1)) != cudaSuccess) break;
@@ -919,7 +931,7 @@ nb_status nb_autotune(nb_ctx *ctx, const char *cache_path) {
                 if (ms_best > 50.f) reps = 1;    // long launches: one timing is enough
                 if (ms_best < best) {
                     best = ms_best;
-                    bestE = ctx->table[b];
+                    bestE = PlanEntry{pl.gl, (int32_t)tg};
                 }
             }
             if (st != NB_OK || e != cudaSuccess) break;
@@ -937,7 +949,7 @@ nb_status nb_autotune(nb_ctx *ctx, const char *cache_path) {
     if (cache_path) {
         FILE *f = std::fopen(cache_path, "w");
         if (f) {
-            std::fprintf(f, "nbtune %d %d\n", ctx->p.precision, ctx->grid_eval);
+            std::fprintf(f, "nbtune %d %d %d %d\n", ctx->p.precision, ctx->grid_eval, ctx->d.order, tune_streamk);
             for (int b = 0; b < kBuckets; ++b) std::fprintf(f, "%d %d\n", ctx->table[b].gl, ctx->table[b].target_items);
             std::fclose(f);
         }

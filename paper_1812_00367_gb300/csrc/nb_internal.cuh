@@ -408,6 +408,26 @@ __host__ __device__ inline int64_t choose_split(int64_t tiles, int64_t ntj, int6
     return best;
 }
 
+// How an evaluation of A active particles over ntj j-tiles is launched, from its
+// bucket's table entry: in the planner of the steps, for the host-planned
+// evaluations, and in the autotuner, which times what the planner will run and
+// stores lanes that this gives back unchanged.  streamk: the launch may use
+// stream-K ranges (one cluster, NB_NO_STREAMK not set); otherwise the entry's lanes
+// and split items, the same alone and in a batch.
+struct EvalPlan {
+    int32_t gl, split, tiles, streamk;
+};
+__host__ __device__ inline EvalPlan plan_eval(PlanEntry e, int64_t A, int64_t ntj, bool streamk, int64_t grid,
+                                              int64_t partial_cap, int precision) {
+    EvalPlan p;
+    p.gl = streamk ? sk_lanes(e.gl, A, ntj, grid, precision) : e.gl;
+    const int64_t tiles = cdiv(A, kTPB / p.gl);
+    p.tiles = (int32_t)tiles;
+    p.streamk = streamk && sk_use(tiles, kTPB / p.gl, ntj, grid, partial_cap) ? 1 : 0;
+    p.split = p.streamk ? 1 : (int32_t)choose_split(tiles, ntj, e.target_items, grid, precision);
+    return p;
+}
+
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));

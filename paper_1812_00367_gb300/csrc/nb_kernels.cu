@@ -260,19 +260,12 @@ __device__ __forceinline__ double block_sum_d(double v, double *sm) {
 // the partial sums of its splits do not fit the scratch.
 __device__ __forceinline__ ClusterPlan plan_cluster(const Dev &d, int64_t ncl, int A, bool unsplit,
                                                     long long &items) {
-    PlanEntry e = d.table[31 - __clz(A)];
-    const long long ntj = cdiv(ncl, kTJ);
-    const bool single = d.n_clusters == 1 && !d.streamk_off;
-    if (single) e.gl = sk_lanes(e.gl, A, ntj, d.grid_eval, d.precision);
-    const long long tiles = cdiv(A, kTPB / e.gl);
-    if (single && sk_use(tiles, kTPB / e.gl, ntj, d.grid_eval, d.partial_cap)) {
-        // one cluster, enough work: stream-K ranges (one "item")
-        items = 1;
-        return ClusterPlan{e.gl, 1, (int)tiles, A, 0, 0, 0, 1, 0};
-    }
-    const long long S = unsplit ? 1 : choose_split(tiles, ntj, e.target_items, d.grid_eval, d.precision);
-    items = tiles * S;
-    return ClusterPlan{e.gl, (int)S, (int)tiles, A, 0, 0, 0, 0, 0};
+    const EvalPlan p = plan_eval(d.table[31 - __clz(A)], A, cdiv(ncl, kTJ), d.n_clusters == 1 && !d.streamk_off,
+                                 d.grid_eval, d.partial_cap, d.precision);
+    // one cluster, enough work: stream-K ranges (one "item")
+    const int S = unsplit ? 1 : p.split;
+    items = p.streamk ? 1 : (long long)p.tiles * S;
+    return ClusterPlan{p.gl, S, p.tiles, A, 0, 0, 0, p.streamk, 0};
 }
 
 // One CTA.  Per cluster: A -> bucket floor(log2 A) -> (gl, target items) ->
