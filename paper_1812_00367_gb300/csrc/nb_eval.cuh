@@ -100,12 +100,9 @@ struct Prec<NB_FP64> {
     // potential term m y in float-float, renormalised every term (|lo| stays
     // below half an ulp of hi): a 64-term tile sum is good to ~2^-45, and
     // tiles add up in FP64
-    static __device__ __forceinline__ void pot_term(float2 m, const FxRoot &t, ff &sum) {
-        // y = Y 2^(-62 - g) as 24 + 24 bits
-        const float s1 = __int_as_float((127 - 23 - t.g) << 23);
-        const float yh = __fmul_rn((float)(uint32_t)(t.y >> 39), s1);
-        const float yl = __fmul_rn((float)((uint32_t)(t.y >> 15) & 0xffffffu), __fmul_rn(s1, 5.9604644775390625e-08f));
-        sum = ff_add(sum, ff_mul_lazy(ff{m.x, m.y}, ff{yh, yl}));
+    static __device__ __forceinline__ void pot_term(float2 m, float yh, float yl, ff &sum) {
+        const bool none = m.x == 0.f;  // massless or excluded: zero at any separation
+        sum = ff_add(sum, ff_mul_lazy(ff{m.x, m.y}, ff{none ? 0.f : yh, none ? 0.f : yl}));
     }
     // After 64 pairs: their float-pair potential joins the FP64 total.
     static __device__ __forceinline__ void tile_done(Acc &c) {
@@ -133,7 +130,9 @@ struct Prec<NB_FP64> {
     static __device__ __forceinline__ void pair(const I &i, const J &jj, bool self, Acc &c) {
         Terms o;
         terms<kOrder6>(i, jj, c, o);
-        pot_term(self ? make_float2(0.f, 0.f) : jj.mf, o.t, c.pf);
+        float yh, yl;
+        fx_root_to_floats(o.t, yh, yl);
+        pot_term(self ? make_float2(0.f, 0.f) : jj.mf, yh, yl, c.pf);
         const double q = fx_q(fx_y3(o.t, i.K), o.t.g, jj.mm, jfx_em(jj), jfx_sign(jj), self, i.K);
         add<kOrder6>(q, o, c);
     }

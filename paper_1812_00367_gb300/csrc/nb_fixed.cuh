@@ -75,6 +75,13 @@ NB_HD float fx_fma_rz(float a, float b, float c) {
     return f;
 #endif
 }
+NB_HD float fx_fmul(float a, float b) {  // not to be joined with an addition
+#if defined(__CUDA_ARCH__)
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
 NB_HD uint32_t fx_f2bits(float f) {
 #if defined(__CUDA_ARCH__)
     return (uint32_t)__float_as_int(f);
@@ -407,12 +414,21 @@ NB_HD FxRoot fx_root(const FxS R[3], int e, uint64_t eps_x, uint32_t emin_field,
 }
 
 // 1/sqrt(r^2 + eps^2) as a double; no number when r (block exponent e) is not
-// finite.
+// finite, 2^-1022 when it is larger than that says.
 NB_HD double fx_root_to_double(const FxRoot &t, int e) {
     const uint64_t m = (t.y + 0x200) >> 10;  // leading one at bit 52
-    uint32_t hi = (uint32_t)(m >> 32) + ((uint32_t)(1023 - 1 - t.g) << 20);
+    const int x = 1023 - 1 - t.g;
+    uint32_t hi = (uint32_t)(m >> 32) + ((uint32_t)(x > 0 ? x : 0) << 20);
     hi = e >= 1024 ? 0x7ff80000u : hi;
     return fx_bits2d(hi, (uint32_t)m);
+}
+// 1/sqrt(r^2 + eps^2) as a pair of floats, 24 + 24 bits; no number outside
+// [2^-102, 2^126], where a float's exponent or the low part's bits end.
+NB_HD void fx_root_to_floats(const FxRoot &t, float &yh, float &yl) {
+    const uint32_t x = (uint32_t)(127 - 23 - t.g);
+    const float s = fx_bits2f(x - 2u <= 228u ? x << 23 : 0x7fc00000u);
+    yh = fx_fmul((float)(uint32_t)(t.y >> 39), s);
+    yl = fx_fmul((float)((uint32_t)(t.y >> 15) & 0xffffffu), fx_fmul(s, 5.9604644775390625e-08f));
 }
 
 // y^3 in units of 2^(-58 - 3 g)

@@ -66,7 +66,9 @@ __device__ __forceinline__ void sym_pair(const Prec<NB_FP64>::I &i, const JFX &o
     constexpr bool k6 = !uses_order4_terms(MODE);
     T::Terms o;
     T::terms<k6>(i, jj, c, o);
-    T::pot_term(jj.mf, o.t, c.pf);
+    float yh, yl;
+    fx_root_to_floats(o.t, yh, yl);
+    T::pot_term(jj.mf, yh, yl, c.pf);
     const uint64_t y3 = fx_y3(o.t, i.K);
     T::add<k6>(fx_q(y3, o.t.g, jj.mm, jfx_em(jj), jfx_sign(jj), false, i.K), o, c);
     // -q_i: the sign bit turned
@@ -79,7 +81,7 @@ __device__ __forceinline__ void sym_pair(const Prec<NB_FP64>::I &i, const JFX &o
     }
     double &pj = js[sym_nv<MODE>() - 1][k];  // the float pair of j's potential
     ff p{__int_as_float(__double2hiint(pj)), __int_as_float(__double2loint(pj))};
-    T::pot_term(valid ? own.mf : make_float2(0.f, 0.f), o.t, p);
+    T::pot_term(valid ? own.mf : make_float2(0.f, 0.f), yh, yl, p);
     pj = __hiloint2double(__float_as_int(p.hi), __float_as_int(p.lo));
 }
 // EX: one record, two pairs.
