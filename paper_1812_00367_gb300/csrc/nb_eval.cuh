@@ -152,10 +152,12 @@ struct Prec<NB_FP64> {
     static __device__ __forceinline__ void interact4(const I &i, const J &jj, bool self, Acc &c) {
         pair<false>(i, jj, self, c);
     }
-    static __device__ __forceinline__ void finish(const I &i, const Acc &c, double o[10]) {
+    template <bool kOrder6>
+    static __device__ __forceinline__ void finish(const Acc &c, double o[10]) {
         // what is not finite spreads as in doubles: a position (seen in the
         // acceleration, its differences are doubles) takes every sum, a
-        // velocity jerk and snap, an acceleration the snap
+        // velocity jerk and snap, an acceleration the snap; the 4th-order form
+        // has no snap: zero whatever the state
         const double nan = __hiloint2double(0x7ff80000, 0);
         const bool bad_x = !(isfinite(c.a[0]) && isfinite(c.a[1]) && isfinite(c.a[2]));
         const bool bad_v = bad_x || c.fv >= 0x7ff, bad_a = bad_v || c.fa >= 0x7ff;
@@ -163,7 +165,7 @@ struct Prec<NB_FP64> {
         for (int k = 0; k < 3; ++k) {
             o[k] = bad_x ? nan : c.a[k];
             o[3 + k] = bad_v ? nan : c.j[k];
-            o[6 + k] = bad_a ? nan : c.s[k];
+            o[6 + k] = !kOrder6 ? 0.0 : (bad_a ? nan : c.s[k]);
         }
         o[9] = bad_x ? nan : -(c.p + ((double)c.pf.hi + (double)c.pf.lo));
     }
@@ -1092,7 +1094,7 @@ __global__ void __launch_bounds__(kTPB, (eval_min_blocks<P, MODE>())) k_eval(con
             return pslot0 + ((int64_t)tile * split + s) * (10 * Ti);
         };
         double o[10];
-        if constexpr (P == NB_FP64) T::finish(me, acc, o);
+        if constexpr (P == NB_FP64) T::template finish<!uses_order4_terms(MODE)>(acc, o);
         else if constexpr (P == kPrecPot) T::finish(acc, o);
         else T::finish(acc, t64, t64st, o);
         // the sums of the lanes sharing an i; after this, the lane holds those

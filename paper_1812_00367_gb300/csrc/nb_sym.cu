@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
         }
         double o[10];
         if constexpr (P == NB_FP64) {
-            T::finish(me, acc, o);
+            T::template finish<!uses_order4_terms(MODE)>(acc, o);
             // a velocity or acceleration that is not finite spoils every other
             // particle's sums: the reduction is told
             const int bad = acc.fv >= 0x7ff ? 3 : (acc.fa >= 0x7ff ? 2 : 0);
@@ -342,7 +342,9 @@ __global__ void __launch_bounds__(kSymRedTPB) k_sym_reduce(const Dev d, const Sy
             const bool bad_x = !(isfinite(o[0]) && isfinite(o[1]) && isfinite(o[2]));
 #pragma unroll
             for (int q = 0; q < 10; ++q)
-                if (bad_x || (q >= 3 && q < 6 && (bad & 1)) || (q >= 6 && q < 9 && bad)) o[q] = nan;
+                if ((bad_x || (q >= 3 && q < 6 && (bad & 1)) || (q >= 6 && q < 9 && bad)) &&
+                    !(uses_order4_terms(MODE) && q >= 6 && q < 9))
+                    o[q] = nan;
         }
         EvalLaunch E{};
         E.out = L.out;
