@@ -739,9 +739,9 @@ nb_status nb_run(nb_ctx *ctx, double t_end, int64_t max_block_steps, int64_t *bl
         else NB_CU(ctx, read_ctl());
         if (multi) harvest_events(ctx, 0, kMultiSteps);
         else harvest_events(ctx, kMultiSteps, 1);
+        if (ctx->h_ctl->busy == 0) break;
         // a device-side failure stops time from advancing: never spin on it
         if ((s = error_status(ctx, ctx->h_ctl->err)) != NB_OK) return s;
-        if (ctx->h_ctl->busy == 0) break;
     }
     if (block_steps_out) *block_steps_out = (int64_t)(ctx->h_ctl->steps - steps0);
     if (interactions_out) *interactions_out = ctx->h_ctl->inter - inter0;
