@@ -171,7 +171,11 @@ nb_status nb_predict(nb_ctx *ctx, double t_next, double *out);
  *   pot  -= m_j / s2^{1/2}
  * With order 4 only A0, A1 and pot are summed (a is not read; snap = 0).
  * j == i is excluded by index.  The j range may be split across thread
- * blocks; partial sums are combined in a fixed order (deterministic).
+ * blocks; partial sums are combined in a fixed order (deterministic).  With
+ * every particle of a one-cluster NB_FP64 or NB_EX context listed in order
+ * (about 7,800 to 113,000 particles, NB_NO_STREAMK not set) each pair is
+ * evaluated once for both its members: the same accuracy, other roundings
+ * than the same particle's in another list or in a block step.
  *   active  : DEVICE int32 [n_active], global particle indices inside the
  *             cluster's range (duplicates allowed)
  *   out_ajs : DEVICE double [10][n_active]: acc[3], jerk[3], snap[3], pot

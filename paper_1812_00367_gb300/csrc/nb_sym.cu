@@ -268,7 +268,8 @@ __global__ void __launch_bounds__(kTPB, 4) k_sym(const Dev d, const SymLaunch L)
         if constexpr (P == NB_FP64) {
             T::template finish<!uses_order4_terms(MODE)>(acc, o);
             // a velocity or acceleration that is not finite spoils every other
-            // particle's sums: the reduction is told
+            // particle's sums: the reduction is told (row 0 meets every particle
+            // and lies in the first band, so no band's reduction comes too early)
             const int bad = acc.fv >= 0x7ff ? 3 : (acc.fa >= 0x7ff ? 2 : 0);
             if (bad) atomicOr(L.bad, bad);
         } else if constexpr (P == NB_EX) {
