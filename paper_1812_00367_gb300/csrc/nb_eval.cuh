@@ -50,14 +50,15 @@ struct Prec;
 // running sums stay on the FP64 pipe (12 instructions per pair, 9 in the 4th-order
 // form), everything between them runs on the integer pipes.
 // Bound: the issue of half-rate integer instructions (shifts, logic,
-// IMAD.WIDE; 778 instructions a pair and warp; ALU 59 % and FP64 pipe 53 % busy).
-// Measured, N = 65536, A = 1000: 2.51 ms (2.61e10 pairs/s) against 5.70 ms for the
-// same terms in doubles (50 DFMA a pair, the FP64 pipe 95 % busy); A = 48: 157
-// against 324 us.  Residency: 3 and 4 CTAs per SM measured within 1 % of one
+// IMAD.WIDE; 760 instructions a pair and warp, 461 in the 4th-order form; ALU 59 %
+// and FP64 pipe 54 % busy).
+// Measured, N = 65536, A = 1000: 2.46 ms (2.67e10 pairs/s) against 5.70 ms for the
+// same terms in doubles (50 DFMA a pair, the FP64 pipe 95 % busy); A = 48: 154
+// against 324 us; all: 151 against 361 ms.  Residency: 3 and 4 CTAs per SM measured within 1 % of one
 // another over the FP64 cases (A = 48 3 % faster, a batch 3 % slower with 3).
 // Converting w1, w2 with the count of leading zeros of the high word (a general
 // conversion where a component is that small) instead of a float's exponent: 138.6
-// -> 133.2 ms for all pairs of N = 65536.
+// -> 133.2 ms for all pairs of N = 65536, with one exponent a vector.
 template <>
 struct Prec<NB_FP64> {
     using J = JFX;

@@ -57,6 +57,17 @@ NB_HD int fx_clz(uint32_t x) {
     return x ? __builtin_clz(x) : 32;
 #endif
 }
+// Place of the highest bit that differs from the sign, -1 if there is none.
+NB_HD int fx_top(int32_t h) {
+#if defined(__CUDA_ARCH__)
+    int r;
+    asm("bfind.s32 %0, %1;" : "=r"(r) : "r"(h));
+    return r;
+#else
+    const uint32_t x = (uint32_t)(h ^ (h >> 31));
+    return x ? 31 - __builtin_clz(x) : -1;
+#endif
+}
 NB_HD float fx_u2f_rz(uint32_t x) {
 #if defined(__CUDA_ARCH__)
     return __uint2float_rz(x);
@@ -180,6 +191,10 @@ NB_HD uint64_t fx_madu(uint32_t a, uint32_t b, uint64_t c) {
 NB_HD int32_t fx_max3(int32_t a, int32_t b, int32_t c) {
     const int32_t m = a > b ? a : b;
     return m > c ? m : c;
+}
+NB_HD int32_t fx_imin3(int32_t a, int32_t b, int32_t c) {
+    const int32_t m = a < b ? a : b;
+    return m < c ? m : c;
 }
 NB_HD uint32_t fx_min3(uint32_t a, uint32_t b, uint32_t c) {
     const uint32_t m = a < b ? a : b;
@@ -492,10 +507,12 @@ NB_HD void fx_w2(const FxS R[3], int er, const FxS V[3], int ev, const Fx3 &A, c
 // w1_k| + 3 |beta r_k|) as in doubles, however thin the system is along an axis.
 // With one exponent for a vector a component 2^-k of its vector's norm had k - 5
 // bits less than in doubles (z / x = 1e-6: jerk z 2.9e-12 instead of 2.3e-16); the
-// exponents cost 130 of now 778 instructions a pair and warp (FP64, N = 65536, A =
-// 1000: 2.17 -> 2.51 ms; all, each pair once: 90.4 -> 97.4 ms).  Differences of v
-// and a in doubles instead of integers: 742 instructions and 18 FP64 ones instead
-// of 12, 2.68 and 110.6 ms, and less exact than doubles' exact difference allows.
+// exponents cost 112 of now 760 instructions a pair and warp (FP64, N = 65536, A =
+// 1000: 2.17 -> 2.46 ms; all, each pair once: 90.4 -> 96.6 ms).  Differences of v
+// and a in doubles instead of integers: 18 FP64 instructions instead of 12, 2.68
+// and 110.6 ms, and a rounding of each difference that the integers do not have.
+// Leading places by bfind.s32 on the signed high word instead of clz of its
+// magnitude: 784 -> 760 instructions, 2.51 -> 2.46 ms.
 struct FxC3 {
     int64_t w[3];  // component k is w[k] 2^(f[k] - 1023 - 61), 2^61 <= |w[k]| < 2^62, or 0
     int32_t f[3];  // exponent fields (below 0: under the doubles' range)
@@ -536,29 +553,28 @@ NB_HD FxP3 fx_pack_components(const double d[3]) {
 template <int kVecs>
 NB_HD void fx_differences(const FxP3 *j, const FxP3 *i, FxC3 *o, int32_t *top) {
     int m[kVecs][3];
-    uint32_t t[kVecs][3], low = 0xffffffffu;
+    int t[kVecs][3], low = 31;
     for (int q = 0; q < kVecs; ++q) {
         for (int k = 0; k < 3; ++k) {
             m[q][k] = j[q].f[k] > i[q].f[k] ? j[q].f[k] : i[q].f[k];
             o[q].w[k] = fx_sar(j[q].w[k], m[q][k] - j[q].f[k]) - fx_sar(i[q].w[k], m[q][k] - i[q].f[k]);  // < 2^62
-            t[q][k] = fx_high(o[q].w[k]);
+            t[q][k] = fx_top(fx_hi(o[q].w[k]));
         }
-        low = low < t[q][0] ? low : t[q][0];
-        low = fx_min3(low, t[q][1], t[q][2]);
+        const int l3 = fx_imin3(t[q][0], t[q][1], t[q][2]);
+        low = low < l3 ? low : l3;
         top[q] = fx_max3(m[q][0], m[q][1], m[q][2]);
     }
-    if (low != 0) {
+    if (low >= 0) {
         for (int q = 0; q < kVecs; ++q)
             for (int k = 0; k < 3; ++k) {
-                const int n = fx_clz(t[q][k]) - 2;
-                o[q].w[k] = (int64_t)fx_shl((uint64_t)o[q].w[k], n);
-                o[q].f[k] = m[q][k] + 1 - n;
+                o[q].w[k] = (int64_t)fx_shl((uint64_t)o[q].w[k], 29 - t[q][k]);
+                o[q].f[k] = m[q][k] + t[q][k] - 28;
             }
     } else {  // a component below 2^-29 of the particles' own (or zero)
         for (int q = 0; q < kVecs; ++q)
             for (int k = 0; k < 3; ++k) {
                 const int64_t w = o[q].w[k];
-                const int n = (t[q][k] ? fx_clz(t[q][k]) : 32 + fx_clz((uint32_t)(w ^ (w >> 63)))) - 2;
+                const int n = t[q][k] >= 0 ? 29 - t[q][k] : 30 + fx_clz((uint32_t)(w ^ (w >> 63)));
                 o[q].w[k] = (int64_t)fx_shl((uint64_t)w, n);
                 o[q].f[k] = w == 0 ? -8192 : m[q][k] + 1 - n;
             }
@@ -606,7 +622,7 @@ NB_HD void fx_vectors(const double r[3], const FxC3 &V, const FxC3 &A, int top, 
     const int64_t rv = fx_sar(fx_mulhi(Rs[0], Vs[0], K), G - g0) + fx_sar(fx_mulhi(Rs[1], Vs[1], K), G - g1) +
                        fx_sar(fx_mulhi(Rs[2], Vs[2], K), G - g2);  // units 2^(G - 58), below 2^61.6
     int64_t al = fx_mulhi(fx_split(rv), Y2, K);                      // units 2^(G - 2 er + s - 58), below 2^59.6
-    const int na = fx_clz(fx_high(al)) - 3;
+    const int na = 28 - fx_top(fx_hi(al));
     al = (int64_t)fx_shl((uint64_t)al, na);
     const int ea = G - 2 * er + t.s + 2 - na;
     const FxS a3 = fx_split(-3 * al);
@@ -637,7 +653,7 @@ NB_HD void fx_vectors(const double r[3], const FxC3 &V, const FxC3 &A, int top, 
         const int eA = 2 * ea + 2;
         const int mB = eA > eZ ? eA : eZ;
         int64_t b3 = fx_sar(aa3, mB - eA + 1) - fx_sar(z3, mB - eZ + 1);  // -3 beta, units 2^(mB - 57)
-        const int nb = fx_clz(fx_high(b3)) - 2;
+        const int nb = 29 - fx_top(fx_hi(b3));
         b3 = (int64_t)fx_shl((uint64_t)b3, nb);  // below 2^62, units 2^(mB - 57 - nb)
         const FxS B3 = fx_split(b3);
         const int eb = mB + 3 - nb;

@@ -13,14 +13,14 @@
 // shared memory.
 //
 // Bound: the FP64 pipe and the issue of integer instructions together (6th
-// order: 21 DFMA a pair for both members, 336 SM clocks a warp, against 2 x 192,
-// and half of the integer work).  Measured, one-sided -> each pair once: N =
-// 65536 6th order 133.2 -> 90.4 ms (98 ms at 2 or 3 CTAs per SM), N = 10007 3.3
-// -> 2.3 ms, 4th order N = 30011 17.3 -> 13.4 ms, potential N = 65536 32.0 ->
-// 20.0 ms (FP64 pipe 85 % busy); EX, bound by its packed FP32 operations (about
-// 620 a pair for both members instead of 2 x 500), N = 65536 62.5 -> 42.9 ms, 4th
-// order N = 30011 7.7 -> 5.6 ms.  Padding the records against two-fold bank
-// conflicts measured the same.
+// order: 21 DFMA a pair for both members, 336 SM clocks a warp, against 2 x 192;
+// 876 instructions against 2 x 760; FP64 pipe 77 % and ALU 48 % busy).  Measured,
+// one-sided -> each pair once, ms: N = 65536 6th order 151.4 -> 96.6, 4th order 88.2
+// -> 64.2; N = 30011 31.9 -> 20.4 and 18.6 -> 13.6; potential N = 65536 32.0 -> 19.7
+// (FP64 pipe 85 % busy); EX, bound by its packed FP32 operations (about 620 a pair
+// for both members instead of 2 x 500), N = 65536 62.5 -> 43.4, 4th order 35.8 ->
+// 26.6, N = 30011 13.2 -> 9.2 and 7.6 -> 5.6.  2 or 3 CTAs per SM instead of 4, FP64:
+// 8 % slower.
 //
 // Order of the sums: units (row, column) are cut into equal ranges over a fixed
 // grid (as stream-K); each range leaves one partial per row it touches and each

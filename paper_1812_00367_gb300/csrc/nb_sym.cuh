@@ -21,9 +21,13 @@ __host__ __device__ inline int sym_row(int64_t u, int64_t ntj) {
     return (int)r;
 }
 
-// Used from kSymMinUnits units per CTA (below, the triangle's cut is too
-// coarse) up to the sizes it was measured at: kSymMaxUnits units (N = 113,000) for
-// the pair terms, ten times as many (N = 357,000) for the potential.
+// Used from kSymMinUnits units per CTA on (N = 7,800 on a grid of 608), below which
+// nb_evaluate of every particle keeps the sums of a block step bit for bit; up to
+// kSymMaxUnits units (N = 113,000) for the pair terms, ten times as many (N =
+// 357,000) for the potential, the sizes it was tried at.  It would pay from about one
+// unit per CTA on (us, each pair once against one-sided; FP64: N = 3000 the same, 4000
+// 488 / 628, 6000 944 / 1392, 8000 1560 / 2350, 12000 3395 / 5316; EX: 4000 233 /
+// 293, 8000 714 / 995).
 constexpr int64_t kSymMinUnits = 6;
 constexpr int64_t kSymMaxUnits = 781250;
 
@@ -39,8 +43,7 @@ __host__ __device__ inline int64_t sym_sum_doubles(int64_t ntj, int64_t nv) { re
 // Bands (0: the scratch is too small).  Their units are multiples of the grid, but
 // for the last one's: a CTA's share of all bands together is then that of one
 // launch (bands of whole rows left shares of 55 and 56 units: N = 65536 98.5 against
-// 97.9 ms).  Every
-// band has at least as many units as CTAs.
+// 97.9 ms).  Every band has at least as many units as CTAs.
 __host__ __device__ inline int64_t sym_bands(int64_t ntj, int64_t grid, int64_t nv, int64_t cap) {
     const int64_t fit = (cap - sym_piece_doubles(ntj, grid) - sym_sum_doubles(ntj, nv)) / (nv * kTJ);
     const int64_t most = fit / grid;  // units a CTA
