@@ -482,7 +482,6 @@ nb_status nb_init(nb_ctx **out, const nb_params *p, int64_t n, const nb_state *s
     d.dt_min = p->dt_min;
     d.dt_max = p->dt_max;
     d.neg_one = -1.0;
-    d.neg_zero = -0.0;
 
     const int occ = std::max(1, eval_occupancy(p->precision, d.order == 4 ? kModeStep4 : kModeStep));
     ctx->grid_eval = occ * ctx->sm_count;

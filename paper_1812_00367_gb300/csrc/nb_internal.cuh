@@ -228,9 +228,9 @@ struct Dev {
     double *energy_part;  // [blocks][8]
     // parameters
     double eps2, eta, eta_init, dt_min, dt_max;
-    // -1.0 and -0.0 as run-time values: FP64 products and differences issued
-    // as FMAs (a*b - 0, a - b = b*(-1) + a) cannot be folded back by compilers
-    double neg_one, neg_zero;
+    // -1.0 as a run-time value: a - b = b*(-1) + a issued as an FMA, which
+    // compilers cannot fold back (DADD runs at 84 % of the DFMA rate)
+    double neg_one;
     // 6: NM08 6th order; 4: Makino & Aarseth 4th order.  Kept last: inserting
     // it among the fields above measured 2.8 % slower FP64 evaluation.
     int32_t order;
@@ -305,7 +305,7 @@ constexpr bool uses_order4_terms(int mode) { return is_order4_mode(mode) || mode
 // ---------------------------------------------------------- small helpers
 __host__ __device__ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-constexpr int kMinTilesPerItem = 4;  // a j-range holds at least 4 x 64 j
+constexpr int kMinTilesPerItem = 4;  // a j-range holds at least 4 x 64 j (FP64: 64, split_max)
 
 // Stream-K decomposition of a single cluster's evaluation.  Its work is
 // U = tiles x ntj units (one i-tile against one j-tile, all of equal cost);
@@ -371,8 +371,8 @@ __host__ __device__ inline int64_t split_max(int64_t ntj, int precision) {
 }
 
 // Number of j-ranges (split S) for `tiles` i-tiles over a cluster of `ntj`
-// j-tiles.  Start from the bucket's target item count; keep at least
-// kMinTilesPerItem j-tiles per item; for `grid` resident CTAs, take the
+// j-tiles.  Start from the bucket's target item count; make at most split_max
+// ranges; for `grid` resident CTAs, take the
 // smallest S in [S0/2, 2 S0] whose items fill the largest fraction of whole
 // waves (equal-cost items: a last, partly filled wave leaves SMs idle).  The
 // result depends on this cluster alone, so a cluster's plan (and therefore
@@ -440,28 +440,6 @@ __device__ __forceinline__ double fma_rn_f64(double a, double b, double c) {
     asm("fma.rn.f64 %0, %1, %2, %3;" : "=d"(r) : "d"(a), "d"(b), "d"(c));
     return r;
 }
-// 1/sqrt(r2) for r2 in [2^-126, 2^128) in five FP64 operations (measured
-// beside the pair terms' own root, nb_probe_rsqrt).  Seed: the exponent and
-// top 20 mantissa bits of r2 are moved into an FP32 word with integer
-// operations, the SFU gives rsqrt.approx, and the result is moved back the
-// same way (relative seed error below 2^-19).  One third-order step
-//   y = y0 (1 + e/2 + 3 e^2/8),  e = 1 - r2 y0^2
-// (the binomial series of (1 - e)^{-1/2}) leaves a truncation error of about
-// (5/16) e^3 < 2^-55; y0 has 21 significant bits, so y0^2 is exact.  Products
-// are FMAs against a run-time -0.0 (x*y + (-0) == x*y, signed zeros included).
-__device__ __forceinline__ double rsqrt_f64_fma(double r2, double neg_zero) {
-    const int hi = __double2hiint(r2);
-    const float f = __int_as_float((hi - 0x38000000) << 3);
-    float yf;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(f));
-    const double y0 = __hiloint2double((__float_as_int(yf) >> 3) + 0x38000000, 0);
-    const double y2 = fma_rn_f64(y0, y0, neg_zero);
-    const double e = fma(-r2, y2, 1.0);
-    const double p = fma(e, 0.375, 0.5);
-    const double t = fma_rn_f64(y0, e, neg_zero);
-    return fma(t, p, y0);
-}
-
 // SFU approximation of 1/sqrt (rsqrt.approx.ftz.f32), per lane for float2.
 __device__ __forceinline__ float rsqrt_sfu(float x) {
     float y;

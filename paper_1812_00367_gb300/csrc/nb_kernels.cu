@@ -300,9 +300,10 @@ __global__ void __launch_bounds__(kPlanTPB) k_plan(const Dev d, int mode_init, i
     }
     // Items are numbered by cost, dearest first (in classes of a factor of two):
     // the items fetched last, which the other CTAs wait for, are then the
-    // cheapest (block steps of 96 clusters, N up to 4096: FP64 22.5 -> 22.0 ms, EX
-    // 13.8 -> 13.4; 8 clusters, few items a CTA, 2.72 -> 2.74).  The order within
-    // a class is the atomics'; no result depends on it.  s_cls: a class's totals,
+    // cheapest (block steps from t = 1/128 to 1/64 of 96 clusters, N up to 4096:
+    // FP64 24.9 -> 24.2 ms, EX 13.9 -> 13.3; 16 clusters 7.11 -> 6.98; 40 of N up to
+    // 2000, many items a CTA in one class, 3.99 -> 4.01).  The order within a class
+    // is the atomics'; no result depends on it.  s_cls: a class's totals,
     // then its next free place: clusters in the upper 24 bits, items below.
     __shared__ unsigned long long s_cls[32];
     constexpr unsigned long long kOne = 1ull << 40;

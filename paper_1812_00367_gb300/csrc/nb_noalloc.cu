@@ -33,7 +33,7 @@ constexpr int64_t kNaMaxGroups = kNaMaxItems * 10 * kTPB / kGrpStride + 1;
 constexpr size_t kNaGrpBytes = (size_t)kNaMaxGroups * sizeof(int32_t);
 constexpr size_t kNaOffGrp = kNaOffTile + ((kNaTileBytes + 255) / 256) * 256;
 constexpr size_t kNaOffAux = kNaOffGrp + ((kNaGrpBytes + 255) / 256) * 256;
-constexpr size_t kNaBytes = kNaOffAux + 256;  // about 5.8 MB in all
+constexpr size_t kNaBytes = kNaOffAux + 256;  // about 6.3 MB in all
 
 struct NaAux {
     int64_t offsets[2];
@@ -51,8 +51,8 @@ std::mutex g_na_mutex;
 DevSlot g_na_slots[128];
 
 // Pack the caller's [10][n] predicted values into the FP64 evaluation's
-// records (JFX, 96 bytes), pad to whole 64-particle tiles with zero-mass particles far away, clear the tile
-// counters and the error word, and write the one-cluster offsets.
+// records (JFX, 112 bytes), pad to whole 64-particle tiles with zero-mass particles
+// far away, clear the tile counters and the error word, and write the one-cluster offsets.
 __global__ void k_na_prepare(unsigned char *base, const double *jp, int64_t n, int64_t npad,
                              int64_t tiles) {
     JFX *jarr = reinterpret_cast<JFX *>(base + kNaOffJarr);
@@ -177,7 +177,6 @@ extern "C" nb_status nb_evaluate_noalloc(const double *jpred, int64_t n, double 
     d.err = &aux->err;
     set_eps2(d, eps);
     d.neg_one = -1.0;
-    d.neg_zero = -0.0;
     EvalLaunch L{};
     L.direct = 1;
     L.cluster = 0;
