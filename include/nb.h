@@ -53,7 +53,8 @@ typedef enum {
  * single-precision numbers).  Particle state, prediction, correction and
  * time steps are FP64 for every choice. */
 typedef enum {
-    NB_FP64 = 0, /* double precision throughout */
+    NB_FP64 = 0, /* double precision; the pair terms in integers with an exponent
+                    per component, no component less exact than in doubles */
     NB_EX = 1,   /* float-float (hi + lo single-precision pair) arithmetic */
     NB_FP32 = 2, /* relative coordinates from split hi/lo singles, FP32 force
                     math, FP32 sums over j-chunks promoted to FP64 */
@@ -169,6 +170,8 @@ nb_status nb_predict(nb_ctx *ctx, double t_next, double *out);
  *   jerk += m_j v / s2^{3/2} - 3 alpha A0            (A1)
  *   snap += m_j a / s2^{3/2} - 6 alpha A1 - 3 beta A0 (A2)
  *   pot  -= m_j / s2^{1/2}
+ * (pot, summed in pairs of floats, is no number where a massive partner is
+ * closer than 1e-38 or farther than 5e30; nb_energy takes any distance.)
  * With order 4 only A0, A1 and pot are summed (a is not read; snap = 0).
  * j == i is excluded by index.  The j range may be split across thread
  * blocks; partial sums are combined in a fixed order (deterministic).  With

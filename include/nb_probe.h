@@ -52,7 +52,7 @@ nb_status nb_selftest_wait_timeout(double budget_seconds, void *stream);
  * nb_probe_rsqrt -- the evaluation kernel's reciprocal square roots applied
  * elementwise, for accuracy tests against a higher-precision reference:
  *   y[k] = 1 / sqrt(x[k])
- *   which : 0 = the form the FP64 pair terms use (block fixed point: SFU seed,
+ *   which : 0 = the form the FP64 pair terms use (fixed point: SFU seed,
  *               one third-order step on integers; here with r = 0 and
  *               eps^2 = x, the result rounded to a double);
  *           1 = the float-float form of the EX pair terms, on x rounded to a
